@@ -22,10 +22,15 @@ LIB = os.path.join(PKG, "liblbfsi.so")
 # and global slot of the step checked, a violation reported as LBFSI_EBOUNDS)
 BUILD_BOUNDS = os.path.join(ROOT, "_build_bounds")
 LIB_BOUNDS = os.path.join(PKG, "liblbfsi_bounds.so")
-SOURCES = ["lbfsi_step.cu", "lbfsi_api.cu", "lbfsi_host.cu", "lbfsi_batch.cu", "lbfsi_noalloc.cu",
-           "lbfsi_elements.cu"]
+SOURCES = ["lbfsi_step.cu", "lbfsi_fields.cu", "lbfsi_stream64.cu", "lbfsi_elements.cu", "lbfsi_api.cu",
+           "lbfsi_host.cu", "lbfsi_batch.cu", "lbfsi_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
+
+
+# the step kernels' instantiations (tile shapes, launch forms) have to round
+# alike: no contraction but the fused operations written out in their sources
+SOURCE_FLAGS = {s: ["-fmad=false"] for s in ("lbfsi_step.cu", "lbfsi_fields.cu", "lbfsi_stream64.cu")}
 
 
 def nvcc() -> str:
@@ -56,7 +61,7 @@ def build(verbose: bool = False, force: bool = False, bounds: bool = False) -> s
         o = os.path.join(build_dir, src.replace(".cu", ".o"))
         objs.append(o)
         if force or _stale(o, [s] + headers):
-            jobs.append([cc, *ARCH, *FLAGS, *extra, "-I", INCLUDE, "-I", CSRC, "-c", s, "-o", o])
+            jobs.append([cc, *ARCH, *FLAGS, *SOURCE_FLAGS.get(src, []), *extra, "-I", INCLUDE, "-I", CSRC, "-c", s, "-o", o])
 
     def run(cmd):
         if verbose:

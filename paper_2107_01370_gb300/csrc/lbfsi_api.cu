@@ -80,6 +80,8 @@ struct lbfsi_mesh_s {
     lbfsi::DeviceMesh dmesh;
     lbfsi::CudaMallocMemory mem;
     int nbatch = 0, precision = 0, variant = 4, order = 1, tile_rows = 16, tiles_per_solve = 0;
+    bool own_shape = true;               // no schedule asked for: the shape follows the size
+    int shape = 4;                       // tile shape launched (step_shape)
     int nbody = 1;                       // bodies per solve (independent bodies of a C-grid)
     size_t slots() const { return (size_t)nbatch * (size_t)nbody; }   // body records
     size_t esize = 8;
@@ -87,8 +89,10 @@ struct lbfsi_mesh_s {
     std::vector<lbfsi_body_desc> bodies;
     void* d_p[2] = {nullptr, nullptr};   // populations, (f_q, g_q) pairs [nbatch][9][N]
     void* d_M[2] = {nullptr, nullptr};
-    void* d_ppost = nullptr;             // collide-only output, same layout
-    void* d_dep = nullptr;               // general meshes: cached static departures ((xi, eta)
+    void* d_ppost = nullptr;             // post-collision populations, same layout (float64: the
+                                         // step's; float: made when the accessor asks)
+    void* d_Y = nullptr;                 // float: correction field [nbatch][2][N]
+    void* d_dep = nullptr;               // general meshes, float64: cached static departures ((xi, eta)
                                          // [9][Nx], then codes [Nx]; see SolveDev::dep_xe)
     double* d_stage = nullptr;  // [nbatch][4][N] float64 staging
     StepMaps* d_maps[2] = {nullptr, nullptr};  // [nbatch][nbody] each
@@ -96,8 +100,9 @@ struct lbfsi_mesh_s {
     BodyStateDev* d_state_b = nullptr;
     double* d_loads_tmp = nullptr;
     double* d_part = nullptr;        // [nbatch][nbody][ntj][3] load partials
-    unsigned* d_counter = nullptr;   // [nbatch][2] CTA completion count, step number
+    unsigned* d_counter = nullptr;   // [nbatch][4] (SolveDev::counter)
     BodyDev* d_bodies = nullptr;     // [nbatch][nbody]
+    lbfsi::BodyProp* d_prop = nullptr;   // [nbatch][nbody]
     lbfsi::MeshDev* d_meshdev = nullptr;
     SolveDev* d_solves = nullptr;    // [nbatch]
     unsigned* d_status = nullptr;
@@ -110,17 +115,18 @@ struct lbfsi_mesh_s {
     // counters), captured on a private stream and replayed on 'stream'
     int graph_steps = 0;
     cudaGraphExec_t graph = nullptr;
+    int64_t graph_launches = 0;
     cudaStream_t cap_stream = nullptr;
     // pinned staging of lbfsi_step_record
     void* h_rec = nullptr;
     size_t h_rec_bytes = 0;
     double* d_rec = nullptr;         // device history of lbfsi_step_record: [steps][records][7]
     size_t d_rec_count = 0;
-    // tensor maps of the float step (StepArgs::tm_p, tm_M) for tiles of
-    // tma_rows rows: -1 not built yet, 0 not used (float64, periodic boxes,
-    // Ntheta not a multiple of 4, LBFSI_TMA=0, or no encoder)
+    // tensor maps of the float step (StepArgs::tm_p, tm_Y) for tiles of
+    // tma_rows rows: -1 not built yet, 0 not used (float64, C-grids, periodic
+    // boxes, Ntheta not a multiple of 4, LBFSI_TMA=0, or no encoder)
     int tma_rows = -1;
-    CUtensorMap tm_p[2], tm_M[2];
+    CUtensorMap tm_p[2], tm_Y;
 
     int cur() const { return (int)(host_k & 1u); }
     bool first() const { return host_k == 0u; }
@@ -220,27 +226,73 @@ void unify_cut_copies(const lbfsi::HostMesh& h, double* user, size_t blocks, int
                     user[(b * h.N + (size_t)j) * w + c] = user[(b * h.N + (size_t)(h.nt - 1 - j)) * w + c];
 }
 
-// One coupled step of every solve: one launch (collide of step k, stream of
-// k + 1), or on a C-grid two: the collision of the rows next to the cut into
-// ppost, because the mirrored rows of one side need the other side's
-// post-collision populations, then the launch in which the first row of tiles
-// streams from ppost and every other tile collides and streams.
-int launches_per_step(lbfsi_mesh m) { return m->host.cgrid ? 2 : 1; }
+lbfsi::StepArgs make_args(lbfsi_mesh m);
 
-cudaError_t launch_one_step(lbfsi_mesh m, lbfsi::StepArgs a, cudaStream_t s) {
-    if (!m->host.cgrid) return lbfsi::launch_step_uniform(a, m->precision, m->variant, m->nbatch, s);
-    lbfsi::StepArgs c = a;
-    c.collide_only = 1;
-    c.cgrid_pre = 1;
-    cudaError_t e = lbfsi::launch_step_uniform(c, m->precision, m->variant, m->nbatch, s);
-    if (e != cudaSuccess) return e;
-    a.stream_post = 1;
-    return lbfsi::launch_step_uniform(a, m->precision, m->variant, m->nbatch, s);
+// Tile shape of a handle: its schedule's variant or, as long as none was asked
+// for, by its size the shape of the most rows that still gives every SM two
+// tiles (float 16 or 8 rows; float64 always one row per block).
+int step_shape(lbfsi_mesh m) {
+    if (!m->own_shape) return m->variant;
+    auto enough = [&](int rows) {
+        return (long long)m->nbatch * m->host.ntj * ((m->host.nr + rows - 1) / rows) >= 304;
+    };
+    return m->precision == LBFSI_FP64 ? 0 : enough(16) ? 1 : 0;
+}
+
+// Tile shape, rows and tiles of the handle's schedule.
+void set_shape(lbfsi_mesh m) {
+    m->shape = step_shape(m);
+    m->tile_rows = m->host.general ? lbfsi::general_tile_rows(m->precision, m->shape)
+                                   : lbfsi::tile_rows(m->precision, m->shape);
+    m->tiles_per_solve = ((m->host.nr + m->tile_rows - 1) / m->tile_rows) * m->host.ntj;
+}
+
+// Field launch (lbfsi_fields.cu) on the current state of every solve.
+cudaError_t launch_fields(lbfsi_mesh m, const lbfsi::StepArgs& a, int loads, int fields, int ustep, double* rec,
+                          cudaStream_t s) {
+    lbfsi::FieldArgs f{};
+    f.umesh = a.umesh;
+    f.usol = a.usol;
+    f.uniform = 1;
+    f.nbatch = m->nbatch;
+    f.loads = loads;
+    f.fields = fields;
+    f.ustep = ustep;
+    f.rec = rec;
+    f.status = m->d_status;
+    return lbfsi::launch_fields(f, m->precision, m->host.general, s);
+}
+
+// n coupled steps of every solve on stream s, two launches per step: the
+// fields of the current state; then per step the step launch and the field
+// launch behind it (the step's loads and bodies, and the next step's fields;
+// behind the last step the loads alone).  The fields are formed anew from the
+// moments by every call, so that moments written between two calls count.
+// rec: device history of the steps' records, or null.
+// host_step < 0: the step numbers come from the device counters.
+cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, cudaStream_t s, int64_t* launches) {
+    if (n <= 0) return cudaSuccess;
+    lbfsi::StepArgs a = make_args(m);
+    const bool host = host_step >= 0;
+    cudaError_t e = cudaSuccess;
+    if (!host || host_step > 0) {   // (the initial state is streamed without colliding)
+        e = launch_fields(m, a, 0, 1, host ? (int)host_step : -1, nullptr, s);
+        ++*launches;
+    }
+    for (int k = 0; k < n && e == cudaSuccess; ++k) {
+        a.ustep = host ? (int)(host_step + k) : -1;
+        e = lbfsi::launch_step_uniform(a, m->precision, m->shape, m->nbatch, s);
+        if (e == cudaSuccess)
+            e = launch_fields(m, a, 1, k + 1 < n, host ? (int)(host_step + k + 1) : -1,
+                              rec ? rec + (size_t)k * m->slots() * 7 : nullptr, s);
+        *launches += 2;
+    }
+    return e;
 }
 
 void free_all(lbfsi_mesh m) {
-    void* ptrs[] = {m->d_p[0], m->d_p[1], m->d_M[0], m->d_M[1], m->d_ppost, m->d_dep, m->d_stage, m->d_maps[0], m->d_maps[1], m->d_state_a, m->d_state_b,
-                    m->d_loads_tmp, m->d_part, m->d_counter, m->d_bodies, m->d_meshdev, m->d_solves,
+    void* ptrs[] = {m->d_p[0], m->d_p[1], m->d_M[0], m->d_M[1], m->d_ppost, m->d_Y, m->d_dep, m->d_stage, m->d_maps[0], m->d_maps[1], m->d_state_a, m->d_state_b,
+                    m->d_loads_tmp, m->d_part, m->d_counter, m->d_bodies, m->d_prop, m->d_meshdev, m->d_solves,
                     m->d_status};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -268,9 +320,11 @@ int upload_solves(lbfsi_mesh m) {
             s.maps[p] = m->d_maps[p] + bb;
         }
         s.ppost = m->d_ppost ? (char*)m->d_ppost + ((size_t)b * 18 * N + 2 * g0) * es : nullptr;
+        s.Y = m->d_Y ? (char*)m->d_Y + ((size_t)b * 2 * N + g0) * es : nullptr;
         s.part = m->d_part + bb * m->host.ntj * 3;
-        s.counter = m->d_counter + 2 * b;
+        s.counter = m->d_counter + 4 * b;
         s.body = m->d_bodies + bb;
+        s.prop = m->d_prop + bb;
         s.dep_xe = m->d_dep ? (char*)m->d_dep + g0 * 2 * es : nullptr;
         s.dep_code = m->d_dep ? reinterpret_cast<unsigned long long*>((char*)m->d_dep + 9 * N * 2 * es) + g0
                               : nullptr;
@@ -282,39 +336,32 @@ int upload_solves(lbfsi_mesh m) {
     return LBFSI_OK;
 }
 
-// Tensor maps of the handle's two population and moment buffers for its
-// current tile shape (built again after a schedule change); false where the
-// step stages by per-thread copies.  Populations: (f, g) float pairs as
-// (2 Ntheta, rows stored, 9, nbatch) floats, box (2 (32 + 8), rows + 4, 9, 1);
-// moments: (Ntheta, rows stored, 4, nbatch), box (32 + 8, rows + 8, 4, 1) --
-// the staged tiles of the step kernel (+-2 and +-4 nodes around the tile).
-// The rows stored are nr, and on a C-grid its G mirrored rows below row 0.
+// Tensor maps of the handle's two population buffers and its correction
+// field for its current tile shape (built again after a schedule change);
+// false where the step stages by per-thread copies.  Populations: (f, g) float
+// pairs as (2 Ntheta, nr, 9, nbatch) floats, box (2 (32 + 8), rows + 4, 9, 1);
+// Y: (Ntheta, nr, 2, nbatch), box (32 + 8, rows + 4, 2, 1) -- the staged tiles
+// of the step kernel (+-2 rows and -4 .. +4 columns around the tile).
 bool tma_maps(lbfsi_mesh m) {
     if (m->tma_rows == m->tile_rows) return true;
     if (m->tma_rows == 0) return false;
     const char* env = std::getenv("LBFSI_TMA");
-    const bool eligible = m->precision == LBFSI_FP32 && !m->host.box && m->host.nt % 4 == 0 &&
-                          !(env && std::atoi(env) == 0);
-    bool ok = eligible;
-    const size_t nt = (size_t)m->host.nt, nr = (size_t)(m->host.nr + m->host.G), nb = (size_t)m->nbatch;
+    bool ok = m->precision == LBFSI_FP32 && !m->host.box && !m->host.cgrid && m->host.nt % 4 == 0 &&
+              !(env && std::atoi(env) == 0);
+    const size_t nt = (size_t)m->host.nt, nr = (size_t)m->host.nr, nb = (size_t)m->nbatch;
     const unsigned rows = (unsigned)m->tile_rows, w = (unsigned)(lbfsi::TILE_J + 8);
-    for (int c = 0; c < 2 && ok; ++c) {
-        ok = lbfsi::encode_box4(&m->tm_p[c], m->d_p[c], 2 * nt, nr, 9, nb, 2 * w, rows + 4, 9) &&
-             lbfsi::encode_box4(&m->tm_M[c], m->d_M[c], nt, nr, 4, nb, w, rows + 8, 4);
-    }
+    for (int c = 0; c < 2 && ok; ++c) ok = lbfsi::encode_box4(&m->tm_p[c], m->d_p[c], 2 * nt, nr, 9, nb, 2 * w, rows + 4, 9);
+    ok = ok && lbfsi::encode_box4(&m->tm_Y, m->d_Y, nt, nr, 2, nb, w, rows + 4, 2);
     m->tma_rows = ok ? m->tile_rows : 0;
     return ok;
 }
 
-lbfsi::StepArgs make_args(lbfsi_mesh m, int collide_only) {
+lbfsi::StepArgs make_args(lbfsi_mesh m) {
     lbfsi::StepArgs a{};
     if (tma_maps(m)) {
         a.tma = 1;
-        a.tma_g = m->host.G;
-        for (int c = 0; c < 2; ++c) {
-            a.tm_p[c] = m->tm_p[c];
-            a.tm_M[c] = m->tm_M[c];
-        }
+        for (int c = 0; c < 2; ++c) a.tm_p[c] = m->tm_p[c];
+        a.tm_Y = m->tm_Y;
     }
     a.umesh = m->dmesh.dev;
     a.usol = m->solves[0];
@@ -322,7 +369,6 @@ lbfsi::StepArgs make_args(lbfsi_mesh m, int collide_only) {
     a.solves = m->d_solves;
     a.tiles = nullptr;
     a.ntiles = m->nbatch * m->tiles_per_solve;
-    a.collide_only = collide_only;
     a.ustep = (int)m->host_k;
     a.uorder = m->order;
     a.status = m->d_status;
@@ -333,15 +379,13 @@ lbfsi::StepArgs make_args(lbfsi_mesh m, int collide_only) {
 // device counters (so the same graph serves every replay).
 int capture_graph(lbfsi_mesh m) {
     lbfsi::TraceRange trace_("lbfsi graph capture");
-    cudaError_t e = lbfsi::prepare_step(m->precision, m->variant, true, m->host.general);
+    cudaError_t e = lbfsi::prepare_step(m->precision, m->shape, true, m->host.general);
     if (e == cudaSuccess && !m->cap_stream) e = cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_fail(e, "graph capture setup");
-    lbfsi::StepArgs a = make_args(m, 0);
-    a.ustep = -1;
     e = cudaStreamBeginCapture(m->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "begin capture");
-    cudaError_t le = cudaSuccess;
-    for (int g = 0; g < m->graph_steps && le == cudaSuccess; ++g) le = launch_one_step(m, a, m->cap_stream);
+    m->graph_launches = 0;
+    const cudaError_t le = launch_steps(m, m->graph_steps, -1, nullptr, m->cap_stream, &m->graph_launches);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(m->cap_stream, &graph);
     if (le != cudaSuccess || e != cudaSuccess) {
@@ -487,11 +531,10 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
     if (const char* v = std::getenv("LBFSI_STEP_VARIANT")) {
         const int k = std::atoi(v);
         m->variant = (k >= 0 && k < lbfsi::step_variants(LBFSI_FP32)) ? k : 4;
+        m->own_shape = m->precision == LBFSI_FP64;
     }
-    if (m->precision == LBFSI_FP64 || m->host.general) m->variant = 0;   // 8-row tiles (general: the one shape)
-    m->tile_rows = m->host.general ? lbfsi::general_tile_rows(m->precision) : lbfsi::tile_rows(m->precision, m->variant);
-    const int nti = (m->host.nr + m->tile_rows - 1) / m->tile_rows;
-    m->tiles_per_solve = nti * m->host.ntj;
+    if (m->precision == LBFSI_FP64 || m->host.general) m->variant = 0;   // (general: the one shape)
+    set_shape(m);
     m->bodies.assign(bodies, bodies + m->slots());
     m->solves.assign(m->nbatch, SolveDev{});
     rc = lbfsi::upload_mesh(m->host, m->precision, m->mem, m->stream, m->dmesh);
@@ -511,8 +554,9 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
     LB_ALLOC(m->d_state_b, ns);
     LB_ALLOC(m->d_loads_tmp, ns * 3);
     LB_ALLOC(m->d_part, ns * ntj * 3);
-    LB_ALLOC(m->d_counter, 2 * nb);
+    LB_ALLOC(m->d_counter, 4 * nb);
     LB_ALLOC(m->d_bodies, ns);
+    LB_ALLOC(m->d_prop, ns);
     LB_ALLOC(m->d_meshdev, 1);
     LB_ALLOC(m->d_solves, nb);
     LB_ALLOC(m->d_status, 1);
@@ -521,12 +565,15 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
         e = cudaMalloc(&m->d_p[k], nb * 18 * N * m->esize);
         if (e == cudaSuccess) e = cudaMalloc(&m->d_M[k], nb * 4 * N * m->esize);
     }
-    if (e == cudaSuccess && m->host.cgrid) e = cudaMalloc(&m->d_ppost, nb * 18 * N * m->esize);
-    // general meshes: departures of the static nodes, solved once per time
-    // step size (LBFSI_NO_DEPARTURE_CACHE=1 solves them every step instead;
+    if (e == cudaSuccess)
+        e = m->precision == LBFSI_FP64 ? cudaMalloc(&m->d_ppost, nb * 18 * N * m->esize)
+                                       : cudaMalloc(&m->d_Y, nb * 2 * N * m->esize);
+    // general meshes and float64: departures of the static nodes, solved once
+    // per time step size (a float step solves the separable mesh's closed form
+    // faster than it reads them; LBFSI_NO_DEPARTURE_CACHE=1 solves them every step instead;
     // the results are the same)
     const char* nc = std::getenv("LBFSI_NO_DEPARTURE_CACHE");
-    if (e == cudaSuccess && m->host.general && !(nc && std::atoi(nc) != 0))
+    if (e == cudaSuccess && (m->host.general || m->precision == LBFSI_FP64) && !(nc && std::atoi(nc) != 0))
         e = cudaMalloc(&m->d_dep, 9 * N * 2 * m->esize + N * sizeof(unsigned long long));
     if (e != cudaSuccess) {
         free_all(m);
@@ -536,7 +583,7 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
     }
     e = cudaMemcpy(m->d_meshdev, &m->dmesh.dev, sizeof(lbfsi::MeshDev), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(m->d_status, 0, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemset(m->d_counter, 0, 2 * nb * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemset(m->d_counter, 0, 4 * nb * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(m->d_part, 0, ns * ntj * 3 * sizeof(double));
     if (e != cudaSuccess) {
         free_all(m);
@@ -569,6 +616,8 @@ int lbfsi_init_fields(lbfsi_mesh m, const lbfsi_flow_params* p, const double* rh
     const size_t ns = m->slots();
     std::vector<BodyDev> bd(ns);
     for (size_t b = 0; b < ns; ++b) bd[b] = lbfsi::body_dev(m->bodies[b], proto.rho_inf, proto.uinf_x);
+    std::vector<lbfsi::BodyProp> prop(ns);
+    for (size_t b = 0; b < ns; ++b) prop[b] = lbfsi::body_prop(bd[b], p->dt);
     // the caller's field goes to the device as it is unless the C-grid's
     // rows need rearranging (cut copies unified, mirrored rows added)
     const bool direct = rho_u_T && !m->host.cgrid && !m->host.G;
@@ -591,6 +640,8 @@ int lbfsi_init_fields(lbfsi_mesh m, const lbfsi_flow_params* p, const double* rh
     if (m->host.G) M = expand_rows(m->host, M.data(), nb * 4, 1);
     cudaError_t e = cudaMemcpyAsync(m->d_bodies, bd.data(), ns * sizeof(BodyDev), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m->d_prop, prop.data(), ns * sizeof(lbfsi::BodyProp), cudaMemcpyHostToDevice, m->stream);
+    if (e == cudaSuccess)
         e = direct ? cudaMemcpyAsync(m->d_stage, rho_u_T, nb * 4 * N * sizeof(double), cudaMemcpyHostToDevice, m->stream)
                    : cudaMemcpyAsync(m->d_stage, M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
@@ -598,7 +649,7 @@ int lbfsi_init_fields(lbfsi_mesh m, const lbfsi_flow_params* p, const double* rh
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->d_loads_tmp, zl.data(), zl.size() * sizeof(double), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->d_status, 0, sizeof(unsigned), m->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->d_counter, 0, 2 * nb * sizeof(unsigned), m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->d_counter, 0, 4 * nb * sizeof(unsigned), m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "init_fields upload");
     m->host_k = 0;
     rc = upload_solves(m);
@@ -617,10 +668,10 @@ int lbfsi_init_fields(lbfsi_mesh m, const lbfsi_flow_params* p, const double* rh
         const size_t Nx = (size_t)m->host.Nx;
         e = cudaMemsetAsync((char*)m->d_dep + 9 * Nx * 2 * m->esize, 0xff, Nx * sizeof(unsigned long long),
                             m->stream);
-        lbfsi::StepArgs a = make_args(m, 0);
+        lbfsi::StepArgs a = make_args(m);
         a.ustep = 0;
         a.record = 1;
-        if (e == cudaSuccess) e = lbfsi::launch_step_uniform(a, m->precision, m->variant, 1, m->stream);
+        if (e == cudaSuccess) e = lbfsi::launch_step_uniform(a, m->precision, m->shape, 1, m->stream);
         m->launches++;
         if (e != cudaSuccess) return cuda_fail(e, "departure cache");
     }
@@ -664,18 +715,13 @@ int lbfsi_step(lbfsi_mesh m, int nsteps) {
         for (; nsteps - s >= m->graph_steps; s += m->graph_steps) {
             const cudaError_t e = cudaGraphLaunch(m->graph, m->stream);
             if (e != cudaSuccess) return cuda_fail(e, "graph launch");
-            m->launches += (int64_t)m->graph_steps * launches_per_step(m);
+            m->launches += m->graph_launches;
             m->host_k += (unsigned)m->graph_steps;
         }
     }
-    lbfsi::StepArgs a = make_args(m, 0);
-    for (; s < nsteps; ++s) {
-        a.ustep = (int)m->host_k;
-        cudaError_t e = launch_one_step(m, a, m->stream);
-        m->launches += launches_per_step(m);
-        if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
-        m->host_k++;
-    }
+    const cudaError_t e = launch_steps(m, nsteps - s, (long long)m->host_k, nullptr, m->stream, &m->launches);
+    if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+    m->host_k += (unsigned)(nsteps - s);
     return LBFSI_OK;
 }
 
@@ -703,36 +749,14 @@ static int download_maps(lbfsi_mesh m, std::vector<StepMaps>& out) {
     return check_status(m);
 }
 
-namespace {
-// The records of one or two consecutive steps, packed: (Fx, Fy, M, h,
-// alpha, hdot, adot) of every (solve, body) from the maps records the steps'
-// epilogues wrote (the two ping-pong sets hold the last two steps' records):
-// prev (may be null) then cur, n records each.
-__global__ void k_pack_records(const StepMaps* prev, const StepMaps* cur, int n, double* out) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const int np = prev ? n : 0;
-    if (r >= np + n) return;
-    const StepMaps& m = r < np ? prev[r] : cur[r - np];
-    double* o = out + (size_t)r * 7;
-    o[0] = m.loads[0];
-    o[1] = m.loads[1];
-    o[2] = m.loads[2];
-    o[3] = m.S_next.h;
-    o[4] = m.S_next.alpha;
-    o[5] = m.S_next.hdot;
-    o[6] = m.S_next.adot;
-}
-}  // namespace
-
 int lbfsi_step_record(lbfsi_mesh m, int nsteps, double* loads_out, lbfsi_body_state* states_out) {
     lbfsi::TraceRange trace_("lbfsi_step_record");
     if (!m || !loads_out) return fail(LBFSI_EINVAL, "null argument");
     if (!m->initialized) return fail(LBFSI_ESTATE, "init_fields first");
     if (nsteps < 0) return fail(LBFSI_EINVAL, "nsteps must be >= 0");
     const size_t nb = m->slots();   // one record per (solve, body)
-    // the records are packed on the device behind every second launch (one
-    // small kernel for two steps: a strided copy of the records per step
-    // costs more), and the history comes back in one copy at the end
+    // the loads blocks of each step write its records into a device history,
+    // which comes back in one copy at the end
     const size_t cnt = (size_t)nsteps * nb * 7;
     if (cnt > m->d_rec_count || cnt * sizeof(double) > m->h_rec_bytes) {
         cudaError_t e = cudaStreamSynchronize(m->stream);
@@ -755,29 +779,9 @@ int lbfsi_step_record(lbfsi_mesh m, int nsteps, double* loads_out, lbfsi_body_st
             return fail(LBFSI_ENOMEM, "staging for the step records");
         }
     }
-    lbfsi::StepArgs a = make_args(m, 0);
-    for (int s = 0; s < nsteps; ++s) {
-        a.ustep = (int)m->host_k;
-        cudaError_t e = launch_one_step(m, a, m->stream);
-        m->launches += launches_per_step(m);
-        if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
-        m->host_k++;
-        // the launch's epilogue wrote the step's loads and new body state into
-        // the maps record of the next launch; the previous step's records are
-        // in the other set until the launch after this one
-        const bool pair = (s & 1) != 0;
-        if (pair || s == nsteps - 1) {
-            const int first = pair ? s - 1 : s;
-            const unsigned nrec = (unsigned)((pair ? 2 : 1) * nb);
-            k_pack_records<<<(nrec + 127) / 128, 128, 0, m->stream>>>(
-                pair ? m->d_maps[m->cur() ^ 1] : nullptr, m->d_maps[m->cur()], (int)nb,
-                m->d_rec + (size_t)first * nb * 7);
-            m->launches++;
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return cuda_fail(e, "step record kernel");
-        }
-    }
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = launch_steps(m, nsteps, (long long)m->host_k, m->d_rec, m->stream, &m->launches);
+    if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+    m->host_k += (unsigned)nsteps;
     if (cnt) e = cudaMemcpyAsync(m->h_rec, m->d_rec, cnt * sizeof(double), cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "step record copy");
@@ -869,8 +873,13 @@ int lbfsi_get_populations(lbfsi_mesh m, int which, double* f, double* g) {
             const int rc = upload_solves(m);
             if (rc) return rc;
         }
-        e = lbfsi::launch_step_uniform(make_args(m, 1), m->precision, m->variant, m->nbatch, m->stream);
+        // the field launch on the current state (float64: it collides)
+        e = launch_fields(m, make_args(m), 0, 1, (int)m->host_k, nullptr, m->stream);
         m->launches++;
+        if (e == cudaSuccess && m->precision == LBFSI_FP32) {
+            e = lbfsi::launch_post(m->solves[0], m->dmesh.dev, m->cur(), m->nbatch, m->stream);
+            m->launches++;
+        }
         if (e != cudaSuccess) return cuda_fail(e, "collide kernel launch");
         ps = m->d_ppost;
     }
@@ -918,11 +927,8 @@ int lbfsi_set_populations(lbfsi_mesh m, const double* f, const double* g, const 
     // the restored state is post-propagation: make the next launch collide it
     // (step number >= 2 with the same parity)
     m->host_k = 2u + (unsigned)c;
-    std::vector<unsigned> ctr(2 * (size_t)m->nbatch);
-    for (int b = 0; b < m->nbatch; ++b) {
-        ctr[2 * b] = 0u;
-        ctr[2 * b + 1] = m->host_k;
-    }
+    std::vector<unsigned> ctr(4 * (size_t)m->nbatch, 0u);
+    for (int b = 0; b < m->nbatch; ++b) ctr[4 * b + 1] = m->host_k;
     cudaError_t e = cudaMemcpyAsync(m->d_counter, ctr.data(), ctr.size() * sizeof(unsigned),
                                     cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
@@ -1005,11 +1011,8 @@ int lbfsi_restore(lbfsi_mesh m, const void* buf, size_t bytes) {
     p += nb * 4 * N * m->esize;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->d_maps[c], p, m->slots() * sizeof(StepMaps), cudaMemcpyHostToDevice, m->stream);
-    std::vector<unsigned> ctr(2 * nb);
-    for (size_t b = 0; b < nb; ++b) {
-        ctr[2 * b] = 0u;
-        ctr[2 * b + 1] = m->host_k;
-    }
+    std::vector<unsigned> ctr(4 * nb, 0u);
+    for (size_t b = 0; b < nb; ++b) ctr[4 * b + 1] = m->host_k;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->d_counter, ctr.data(), ctr.size() * sizeof(unsigned), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->d_status, 0, sizeof(unsigned), m->stream);
@@ -1028,12 +1031,12 @@ int lbfsi_set_schedule(lbfsi_mesh m, int variant, int order) {
     if (variant < 0 || variant >= (m->host.general ? 1 : lbfsi::step_variants(m->precision)) ||
         (order != 0 && order != 1))
         return fail(LBFSI_EINVAL, "variant or order out of range");
-    if (variant == m->variant && order == m->order) return LBFSI_OK;
+    if (!m->own_shape && variant == m->variant && order == m->order) return LBFSI_OK;
     drop_graph(m);
+    m->own_shape = m->host.general;   // (general meshes have the one variant)
     m->variant = variant;
     m->order = order;
-    m->tile_rows = m->host.general ? lbfsi::general_tile_rows(m->precision) : lbfsi::tile_rows(m->precision, m->variant);
-    m->tiles_per_solve = ((m->host.nr + m->tile_rows - 1) / m->tile_rows) * m->host.ntj;
+    set_shape(m);
     return m->initialized ? upload_solves(m) : LBFSI_OK;
 }
 

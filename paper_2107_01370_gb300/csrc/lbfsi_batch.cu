@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -76,6 +77,7 @@ public:
         }
         free_[start] = len;
     }
+    bool owns(const void* p) const { return p && (const char*)p >= base_ && (const char*)p < base_ + size_; }
     size_t free_bytes() const {
         size_t s = 0;
         for (auto& kv : free_) s += kv.second;
@@ -93,6 +95,34 @@ private:
     std::map<size_t, size_t> free_, used_;
 };
 
+// Step workspaces of the admitted solves (the float path's correction field,
+// the float64 path's post-collision populations), beside the pool so that it
+// admits the solves it always did: blocks of at least CHUNK bytes, kept for
+// the next solves and given back with the batch.  Bounded by the solves the
+// pool can hold at once.
+class Workspace {
+public:
+    void* alloc(size_t bytes) {
+        for (auto& c : chunks_)
+            if (void* p = c->alloc(bytes)) return p;
+        auto c = std::make_unique<Pool>();
+        if (c->init(std::max(bytes, CHUNK)) != LBFSI_OK) {
+            c = std::make_unique<Pool>();
+            if (c->init(bytes) != LBFSI_OK) return nullptr;
+        }
+        chunks_.push_back(std::move(c));
+        return chunks_.back()->alloc(bytes);
+    }
+    void release(void* p) {
+        for (auto& c : chunks_)
+            if (c->owns(p)) c->release(p);
+    }
+
+private:
+    static constexpr size_t CHUNK = 16u << 20;
+    std::vector<std::unique_ptr<Pool>> chunks_;
+};
+
 struct MeshEntry {
     lbfsi::HostMesh host;
     lbfsi::DeviceMesh dev;
@@ -102,13 +132,13 @@ struct MeshEntry {
 
 struct Slot {
     bool used = false, finished = false;
-    bool general = false;   // on a mesh given by node coordinates (GEN kernel, 8-row tiles)
-    bool cgrid = false;     // on a C-grid (general; two launches per step)
+    bool general = false;   // on a mesh given by node coordinates (the general kernel)
     int mesh = -1;
     int steps_target = 0, steps_done = 0;
     int ntiles = 0;
     SolveDev dev{};
     std::vector<void*> blocks;
+    void* work = nullptr;   // its step workspace (SolveDev::Y or ppost)
     // the tile rows its tensor maps were made for (-1: none yet, 0: not used)
     int tma_rows = -1;
 };
@@ -117,7 +147,9 @@ struct Slot {
 
 struct lbfsi_batch_s {
     Pool pool;
+    Workspace work;
     int precision = LBFSI_FP32, variant = 4, order = 0, tile_rows = 16;
+    int shape = 4;   // tile shape launched (the variant)
     size_t esize = 4;
     cudaStream_t stream = nullptr;
     std::vector<MeshEntry> meshes;
@@ -126,17 +158,18 @@ struct lbfsi_batch_s {
     SolveDev* d_solves = nullptr;
     TileDev* d_tiles = nullptr;
     size_t tiles_cap = 0;
+    lbfsi::FieldTile* d_ftiles = nullptr;
+    size_t ftiles_cap = 0;
     int max_meshes = 256, max_slots = 4096;
     unsigned* d_status = nullptr;
-    // float separable solves: tensor maps of each slot's populations and
-    // moments, [max_slots][4] (StepArgs::tmaps)
+    // float separable solves: tensor maps of each slot's populations and Y,
+    // [max_slots][4] (StepArgs::tmaps)
     CUtensorMap* d_tmaps = nullptr;
     BodyStateDev* d_zero_state = nullptr;
     double* d_zero_loads = nullptr;
-    int ntiles = 0;    // separable-mesh tiles of the table (first part)
-    int ngtiles = 0;   // general-mesh tiles (second part)
-    int nctiles = 0;   // C-grid tiles (third part)
-    int ncpre = 0;     // leading C-grid tiles that hold every tile of rows < CGRID_PRE_ROWS
+    // per part of the tables (0 separable, 1 general meshes): step tiles, and
+    // in the field table loads blocks followed by field tiles
+    int ntiles[2] = {0, 0}, nload[2] = {0, 0}, nfield[2] = {0, 0};
     bool dirty = true;
     // CUDA graph of graph_steps launches over the current tile table,
     // captured on a private stream, dropped whenever the table changes
@@ -220,6 +253,8 @@ void drop_mesh(lbfsi_batch b, int k) {
 void release_slot_memory(lbfsi_batch b, Slot& s) {
     for (void* p : s.blocks) b->pool.release(p);
     s.blocks.clear();
+    if (s.work) b->work.release(s.work);
+    s.work = nullptr;
 }
 
 void drop_graph(lbfsi_batch b) {
@@ -230,19 +265,61 @@ void drop_graph(lbfsi_batch b) {
     }
 }
 
-// Tile table of the next launches: every tile of every active solve, in the
+int step_rows(lbfsi_batch b, bool general) {
+    return general ? lbfsi::general_tile_rows(b->precision, b->shape) : b->tile_rows;
+}
+
+// CTAs of a slot's step launches in the current tile shape (SolveDev::ntiles,
+// the completion count), uploaded where it changed.
+cudaError_t update_counts(lbfsi_batch b) {
+    cudaError_t e = cudaSuccess;
+    for (size_t k = 0; k < b->slots.size() && e == cudaSuccess; ++k) {
+        Slot& s = b->slots[k];
+        if (!s.used) continue;
+        const lbfsi::HostMesh& h = b->meshes[s.mesh].host;
+        const int rows = step_rows(b, s.general), n = ((h.nr + rows - 1) / rows) * h.ntj;
+        if (n == s.ntiles) continue;
+        s.dev.ntiles = s.ntiles = n;
+        e = cudaMemcpyAsync(b->d_solves + k, &s.dev, sizeof(SolveDev), cudaMemcpyHostToDevice, b->stream);
+    }
+    return e;
+}
+
+// Upload of a host table into a device array that grows as needed.
+template <typename T>
+cudaError_t put_table(lbfsi_batch b, const std::vector<T>& v, T*& dev, size_t& cap) {
+    cudaError_t e = cudaSuccess;
+    if (v.size() > cap) {
+        e = cudaStreamSynchronize(b->stream);
+        if (dev) cudaFree(dev);
+        dev = nullptr;
+        cap = std::max(v.size(), 2 * cap);
+        if (e == cudaSuccess) e = cudaMalloc(&dev, cap * sizeof(T));
+        if (e != cudaSuccess) {
+            cap = 0;
+            return e;
+        }
+    }
+    // stream-ordered: launches already queued read the previous table
+    if (!v.empty()) e = cudaMemcpyAsync(dev, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, b->stream);
+    return e;
+}
+
+// Tables of the next launches: every tile of every active solve, in the
 // batch's order: 0, the tiles of each solve together; 1, tile rows outermost
 // across all solves, so that the wall and blending-region rows (the most
 // expensive tiles) start first and the far-field rows fill the tail.
 int rebuild_tiles(lbfsi_batch b) {
     lbfsi::TraceRange trace_("lbfsi tile table");
     drop_graph(b);
-    // separable-mesh tiles first (tile rows of the batch's shape), then the
-    // general-mesh tiles and the C-grid tiles (the general kernel's tile)
-    std::vector<TileDev> tiles;
+    cudaError_t e = cudaSuccess;
+    auto active = [&](const Slot& s, int part) { return s.used && !s.finished && (s.general ? 1 : 0) == part; };
+    b->shape = b->variant;
+    b->tile_rows = lbfsi::tile_rows(b->precision, b->shape);
+    e = update_counts(b);
+    if (e != cudaSuccess) return cuda_err(e, "solve record upload");
     // float separable solves: tensor maps for the current tile shape (made
     // once per slot and shape, uploaded behind the launches already queued)
-    cudaError_t e = cudaSuccess;
     const char* tenv = std::getenv("LBFSI_TMA");
     const bool tma_on = b->precision == LBFSI_FP32 && b->d_tmaps && !(tenv && std::atoi(tenv) == 0);
     for (size_t k = 0; k < b->slots.size() && tma_on; ++k) {
@@ -250,21 +327,22 @@ int rebuild_tiles(lbfsi_batch b) {
         if (!s.used || s.finished || s.general || s.tma_rows == b->tile_rows) continue;
         const lbfsi::HostMesh& h = b->meshes[s.mesh].host;
         bool ok = h.nt % 4 == 0;
-        CUtensorMap maps[4];
+        CUtensorMap maps[4]{};
         const size_t nt = (size_t)h.nt, nr = (size_t)h.nr;
         const unsigned rows = (unsigned)b->tile_rows, w = (unsigned)(lbfsi::TILE_J + 8);
-        for (int c = 0; c < 2 && ok; ++c)
-            ok = lbfsi::encode_box4(&maps[c], s.dev.p[c], 2 * nt, nr, 9, 1, 2 * w, rows + 4, 9) &&
-                 lbfsi::encode_box4(&maps[2 + c], s.dev.M[c], nt, nr, 4, 1, w, rows + 8, 4);
+        for (int c = 0; c < 2 && ok; ++c) ok = lbfsi::encode_box4(&maps[c], s.dev.p[c], 2 * nt, nr, 9, 1, 2 * w, rows + 4, 9);
+        ok = ok && lbfsi::encode_box4(&maps[2], s.dev.Y, nt, nr, 2, 1, w, rows + 4, 2);
         if (ok) {
             e = cudaMemcpyAsync(b->d_tmaps + 4 * k, maps, sizeof(maps), cudaMemcpyHostToDevice, b->stream);
             if (e != cudaSuccess) return cuda_err(e, "tensor map upload");
         }
         s.tma_rows = ok ? b->tile_rows : 0;
     }
-    auto build = [&](int part) {
-        const bool general = part > 0;
-        const int rows = general ? lbfsi::general_tile_rows(b->precision) : b->tile_rows;
+    std::vector<TileDev> tiles;
+    std::vector<lbfsi::FieldTile> ftiles;
+    for (int part = 0; part < 2; ++part) {
+        const int rows = step_rows(b, part == 1);
+        const size_t t0 = tiles.size(), f0 = ftiles.size();
         auto push = [&](size_t k, int ti, int tj) {
             const Slot& s = b->slots[k];
             TileDev t{};
@@ -281,14 +359,10 @@ int rebuild_tiles(lbfsi_batch b) {
             t.maps[1] = s.dev.maps[1];
             tiles.push_back(t);
         };
-        auto active = [&](size_t k) {
-            const Slot& s = b->slots[k];
-            return s.used && !s.finished && (s.cgrid ? 2 : s.general ? 1 : 0) == part;
-        };
         auto nti_of = [&](size_t k) { return (b->meshes[b->slots[k].mesh].host.nr + rows - 1) / rows; };
         if (b->order == 0) {
             for (size_t k = 0; k < b->slots.size(); ++k) {
-                if (!active(k)) continue;
+                if (!active(b->slots[k], part)) continue;
                 const int nti = nti_of(k), ntj = b->meshes[b->slots[k].mesh].host.ntj;
                 for (int ti = 0; ti < nti; ++ti)
                     for (int tj = 0; tj < ntj; ++tj) push(k, ti, tj);
@@ -296,48 +370,29 @@ int rebuild_tiles(lbfsi_batch b) {
         } else {
             int max_nti = 0;
             for (size_t k = 0; k < b->slots.size(); ++k)
-                if (active(k)) max_nti = std::max(max_nti, nti_of(k));
+                if (active(b->slots[k], part)) max_nti = std::max(max_nti, nti_of(k));
             for (int ti = 0; ti < max_nti; ++ti)
                 for (size_t k = 0; k < b->slots.size(); ++k) {
-                    if (!active(k) || ti >= nti_of(k)) continue;
+                    if (!active(b->slots[k], part) || ti >= nti_of(k)) continue;
                     const int ntj = b->meshes[b->slots[k].mesh].host.ntj;
                     for (int tj = 0; tj < ntj; ++tj) push(k, ti, tj);
                 }
         }
-    };
-    build(0);
-    const size_t nsep = tiles.size();
-    build(1);
-    const size_t ngen = tiles.size() - nsep;
-    build(2);
-    if (tiles.size() > b->tiles_cap) {
-        e = cudaStreamSynchronize(b->stream);
-        if (b->d_tiles) cudaFree(b->d_tiles);
-        b->d_tiles = nullptr;
-        b->tiles_cap = std::max(tiles.size(), 2 * b->tiles_cap);
-        if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, b->tiles_cap * sizeof(TileDev));
-        if (e != cudaSuccess) {
-            b->tiles_cap = 0;
-            return cuda_err(e, "tile table allocation");
-        }
+        b->ntiles[part] = (int)(tiles.size() - t0);
+        b->nload[part] = b->nfield[part] = 0;
+        for (int fields = 0; fields < 2; ++fields)
+            for (size_t k = 0; k < b->slots.size(); ++k) {
+                if (!active(b->slots[k], part)) continue;
+                const lbfsi::HostMesh& h = b->meshes[b->slots[k].mesh].host;
+                const int n = fields ? lbfsi::field_blocks(b->precision, part == 1, h.nr, h.nt) : lbfsi::load_blocks(h.ntj);
+                for (int t = 0; t < n; ++t) ftiles.push_back({(int)k, b->slots[k].mesh, fields, t});
+                (fields ? b->nfield : b->nload)[part] += n;
+            }
     }
-    if (!tiles.empty()) {
-        // stream-ordered: launches already queued read the previous table
-        e = cudaMemcpyAsync(b->d_tiles, tiles.data(), tiles.size() * sizeof(TileDev), cudaMemcpyHostToDevice, b->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-        if (e != cudaSuccess) return cuda_err(e, "tile table upload");
-    }
-    b->ntiles = (int)nsep;
-    b->ngtiles = (int)ngen;
-    b->nctiles = (int)(tiles.size() - nsep - ngen);
-    // tile rows outermost: the tiles of the first rows come first; otherwise
-    // the collide-only launch runs over the whole part (the others return)
-    b->ncpre = b->nctiles;
-    if (b->order == 1) {
-        int k = 0;
-        while (k < b->nctiles && tiles[nsep + ngen + k].i0 < lbfsi::CGRID_PRE_ROWS) ++k;
-        b->ncpre = k;
-    }
+    e = put_table(b, tiles, b->d_tiles, b->tiles_cap);
+    if (e == cudaSuccess) e = put_table(b, ftiles, b->d_ftiles, b->ftiles_cap);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return cuda_err(e, "tile table upload");
     b->dirty = false;
     return LBFSI_OK;
 }
@@ -358,38 +413,47 @@ int check_status(lbfsi_batch b) {
     return LBFSI_OK;
 }
 
-// Launch arguments of one part of the tile table (0 separable, 1 general, 2 C-grid).
-lbfsi::StepArgs step_args(lbfsi_batch b, int part) {
+// Step launch of one part of the tile table (0 separable, 1 general meshes).
+cudaError_t launch_step_part(lbfsi_batch b, int part, cudaStream_t s) {
+    if (b->ntiles[part] == 0) return cudaSuccess;
     lbfsi::StepArgs a{};
     a.meshes = b->d_meshes;
     a.solves = b->d_solves;
-    a.tiles = b->d_tiles + (part == 0 ? 0 : part == 1 ? b->ntiles : b->ntiles + b->ngtiles);
-    a.ntiles = part == 0 ? b->ntiles : part == 1 ? b->ngtiles : b->nctiles;
-    a.collide_only = 0;
+    a.tiles = b->d_tiles + (part ? b->ntiles[0] : 0);
+    a.ntiles = b->ntiles[part];
     a.ustep = -1;
     a.status = b->d_status;
     a.tmaps = part == 0 && b->precision == LBFSI_FP32 ? b->d_tmaps : nullptr;
-    return a;
+    return lbfsi::launch_step(a, b->precision, part == 1, b->shape, s);
 }
 
-// One step of every active solve: the separable-mesh table launch, the
-// general-mesh one and, for C-grids, the collision of the rows next to the
-// cut followed by the launch that streams the first row of tiles from it and
-// collides and streams the others (independent solves, so the order of the
-// parts is free).
-cudaError_t launch_all(lbfsi_batch b, cudaStream_t s) {
+// Field launch of one part: the loads of the last step, the fields of the
+// current state, or both.
+cudaError_t launch_field_part(lbfsi_batch b, int part, int loads, int fields, cudaStream_t s) {
+    lbfsi::FieldArgs f{};
+    f.meshes = b->d_meshes;
+    f.solves = b->d_solves;
+    f.tiles = b->d_ftiles + (part ? b->nload[0] + b->nfield[0] : 0) + (loads ? 0 : b->nload[part]);
+    f.ntiles = (loads ? b->nload[part] : 0) + (fields ? b->nfield[part] : 0);
+    f.loads = loads;
+    f.fields = fields;
+    f.ustep = -1;
+    f.status = b->d_status;
+    return lbfsi::launch_fields(f, b->precision, part == 1, s);
+}
+
+// n steps of every active solve (as launch_steps of the mesh handle): the
+// current state's fields, then per step the step launches of both parts
+// (independent solves, so their order is free) and the field launches.
+cudaError_t launch_run(lbfsi_batch b, int n, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
-    if (b->ntiles > 0) e = lbfsi::launch_step(step_args(b, 0), b->precision, b->variant, s);
-    if (e == cudaSuccess && b->ngtiles > 0) e = lbfsi::launch_step_general_table(step_args(b, 1), b->precision, s);
-    if (e == cudaSuccess && b->nctiles > 0) {
-        lbfsi::StepArgs a = step_args(b, 2);
-        a.collide_only = 1;
-        a.cgrid_pre = 1;
-        a.ntiles = b->ncpre;   // the tiles of rows < CGRID_PRE_ROWS lead the C-grid part
-        e = lbfsi::launch_step_general_table(a, b->precision, s);
-        a = step_args(b, 2);
-        a.stream_post = 1;
-        if (e == cudaSuccess) e = lbfsi::launch_step_general_table(a, b->precision, s);
+    auto both = [&](auto fn) {
+        for (int part = 0; part < 2 && e == cudaSuccess; ++part) e = fn(part);
+    };
+    if (n > 0) both([&](int p) { return launch_field_part(b, p, 0, 1, s); });
+    for (int k = 0; k < n && e == cudaSuccess; ++k) {
+        both([&](int p) { return launch_step_part(b, p, s); });
+        both([&](int p) { return launch_field_part(b, p, 1, k + 1 < n, s); });
     }
     return e;
 }
@@ -399,14 +463,13 @@ cudaError_t launch_all(lbfsi_batch b, cudaStream_t s) {
 // every replay until the table changes).
 int capture_graph(lbfsi_batch b) {
     lbfsi::TraceRange trace_("lbfsi batch graph capture");
-    cudaError_t e = lbfsi::prepare_step(b->precision, b->variant, false);
-    if (e == cudaSuccess && b->ngtiles + b->nctiles > 0) e = lbfsi::prepare_step(b->precision, 0, false, true);
+    cudaError_t e = lbfsi::prepare_step(b->precision, b->shape, false);
+    if (e == cudaSuccess && b->ntiles[1] > 0) e = lbfsi::prepare_step(b->precision, b->shape, false, true);
     if (e == cudaSuccess && !b->cap_stream) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_err(e, "graph capture setup");
     e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_err(e, "begin capture");
-    cudaError_t le = cudaSuccess;
-    for (int g = 0; g < b->graph_steps && le == cudaSuccess; ++g) le = launch_all(b, b->cap_stream);
+    const cudaError_t le = launch_run(b, b->graph_steps, b->cap_stream);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(b->cap_stream, &graph);
     if (le != cudaSuccess || e != cudaSuccess) {
@@ -437,7 +500,8 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
     b->esize = precision == LBFSI_FP64 ? sizeof(double) : sizeof(float);
     b->stream = static_cast<cudaStream_t>(cuda_stream);
     if (precision == LBFSI_FP64) b->variant = 0;   // 8-row tiles
-    b->tile_rows = lbfsi::tile_rows(precision, b->variant);
+    b->shape = b->variant;
+    b->tile_rows = lbfsi::tile_rows(precision, b->shape);
     int rc = b->pool.init(pool_bytes);
     if (rc) {
         delete b;
@@ -464,7 +528,7 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
 int lbfsi_batch_destroy(lbfsi_batch b) {
     if (!b) return lbfsi::set_error(LBFSI_EINVAL, "null batch");
     cudaStreamSynchronize(b->stream);
-    void* ptrs[] = {b->d_meshes, b->d_solves, b->d_tiles, b->d_status, b->d_zero_state,
+    void* ptrs[] = {b->d_meshes, b->d_solves, b->d_tiles, b->d_ftiles, b->d_status, b->d_zero_state,
                     b->d_zero_loads, b->d_tmaps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -537,18 +601,23 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
         }
         ok = ok && (sd.maps[p] = (StepMaps*)take(sizeof(StepMaps))) != nullptr;
     }
-    sd.ppost = nullptr;
-    if (ok && h.cgrid) {
-        void* pp = take(18 * Nx * es);
-        ok = pp != nullptr;
-        if (ok) sd.ppost = (char*)pp + 2 * g0 * es;
-    }
     ok = ok && (sd.part = (double*)take((size_t)h.ntj * 3 * sizeof(double))) != nullptr;
-    ok = ok && (sd.counter = (unsigned*)take(2 * sizeof(unsigned))) != nullptr;
+    ok = ok && (sd.counter = (unsigned*)take(4 * sizeof(unsigned))) != nullptr;
     BodyDev* body = nullptr;
     ok = ok && (body = (BodyDev*)take(sizeof(BodyDev))) != nullptr;
     double* stage = nullptr;
     ok = ok && (stage = (double*)take(4 * Nx * sizeof(double))) != nullptr;
+    if (ok) {
+        // the body's step map, then the populations' or the field's slots
+        const size_t w = b->precision == LBFSI_FP64 ? 2 : 1, head = 512;
+        static_assert(sizeof(lbfsi::BodyProp) <= 512, "workspace head");
+        s.work = b->work.alloc(head + w * (w == 2 ? 9 : 2) * Nx * es);
+        ok = s.work != nullptr;
+        if (ok) {
+            sd.prop = (const lbfsi::BodyProp*)s.work;
+            (w == 2 ? sd.ppost : sd.Y) = (char*)s.work + head + w * g0 * es;
+        }
+    }
     if (!ok) {
         release_slot_memory(b, s);
         drop_mesh(b, mk);
@@ -556,7 +625,7 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
     }
     sd.body = body;
     sd.mesh = mk;
-    const int rows = h.general ? lbfsi::general_tile_rows(b->precision) : b->tile_rows;
+    const int rows = step_rows(b, h.general);
     sd.ntiles = ((h.nr + rows - 1) / rows) * h.ntj;
     // initial state: equilibria of the initial field, bodies at rest
     std::vector<double> M(4 * N);
@@ -586,9 +655,12 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
         M.swap(Mx);
     }
     const BodyDev bd = lbfsi::body_dev(body_desc, sd.rho_inf, sd.uinf_x);
+    const lbfsi::BodyProp prop = lbfsi::body_prop(bd, sd.dt);
     cudaError_t e = cudaMemcpyAsync(stage, M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(body, &bd, sizeof(BodyDev), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(sd.counter, 0, 2 * sizeof(unsigned), b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync((void*)sd.prop, &prop, sizeof(prop), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sd.counter, 0, 4 * sizeof(unsigned), b->stream);
     if (e == cudaSuccess) e = lbfsi::launch_init(b->precision, stage, p0, m0, (int)Nx, 1, sd.Cv, b->stream);
     if (e == cudaSuccess)
         e = lbfsi::launch_prepare(body, b->d_zero_state, b->d_zero_state, b->d_zero_state, b->d_zero_loads, sd.dt,
@@ -607,7 +679,6 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
     s.used = true;
     s.finished = false;
     s.general = h.general;
-    s.cgrid = h.cgrid;
     s.mesh = mk;
     s.steps_target = steps;
     s.steps_done = 0;
@@ -672,7 +743,7 @@ int lbfsi_batch_step(lbfsi_batch b, int nsteps, int* active_after) {
             const int rc = rebuild_tiles(b);
             if (rc) return rc;
         }
-        if (b->ntiles + b->ngtiles + b->nctiles == 0) break;
+        if (b->ntiles[0] + b->ntiles[1] == 0) break;
         // steps until the next solve finishes: the tile table is fixed over them
         int run = nsteps - st;
         for (auto& s : b->slots)
@@ -688,10 +759,8 @@ int lbfsi_batch_step(lbfsi_batch b, int nsteps, int* active_after) {
                 if (e != cudaSuccess) return cuda_err(e, "batch graph launch");
             }
         }
-        for (; done < run; ++done) {
-            const cudaError_t e = launch_all(b, b->stream);
-            if (e != cudaSuccess) return cuda_err(e, "batch step launch");
-        }
+        const cudaError_t e = launch_run(b, run - done, b->stream);
+        if (e != cudaSuccess) return cuda_err(e, "batch step launch");
         st += run;
         for (auto& s : b->slots) {
             if (!s.used || s.finished) continue;
@@ -718,20 +787,7 @@ int lbfsi_batch_set_schedule(lbfsi_batch b, int variant, int order) {
     drop_graph(b);
     b->variant = variant;
     b->order = order;
-    b->tile_rows = lbfsi::tile_rows(b->precision, variant);
-    // the per-solve CTA count of the completion counter follows the tile shape
-    for (size_t k = 0; k < b->slots.size(); ++k) {
-        Slot& s = b->slots[k];
-        if (!s.used || s.general) continue;   // general meshes keep their one tile shape
-        const lbfsi::HostMesh& h = b->meshes[s.mesh].host;
-        s.dev.ntiles = ((h.nr + b->tile_rows - 1) / b->tile_rows) * h.ntj;
-        s.ntiles = s.dev.ntiles;
-        const cudaError_t e = cudaMemcpyAsync(b->d_solves + k, &s.dev, sizeof(SolveDev), cudaMemcpyHostToDevice, b->stream);
-        if (e != cudaSuccess) return cuda_err(e, "solve record upload");
-    }
-    const cudaError_t e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return cuda_err(e, "schedule change");
-    b->dirty = true;
+    b->dirty = true;   // (rebuild_tiles: the tile shape, the per-solve CTA counts, the tables)
     return LBFSI_OK;
 }
 

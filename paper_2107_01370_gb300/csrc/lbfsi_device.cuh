@@ -20,14 +20,27 @@ __host__ __device__ constexpr int cyq(int q) {
 }
 
 // Reciprocal and square root in the precision of the path: the hardware
-// approximations (relative error about 2^-23) on the float path, IEEE
-// operations on the float64 path.
+// approximations (relative error about 2^-23) on the float path.
 __device__ __forceinline__ float rcp_(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__host__ __device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
+// (float64: the hardware's seed of about 20 bits and two Newton steps
+// r += r (1 - x r), which square its error twice: 1/x to about an ulp; the
+// division's exact rounding costs about twice the operations, at 1/64 of the
+// float rate)
+__host__ __device__ __forceinline__ double rcp_(double x) {
+#ifdef __CUDA_ARCH__
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return r;
+#else
+    return 1.0 / x;
+#endif
+}
 __device__ __forceinline__ float sqrt_(float x) {
     float y;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -39,13 +52,17 @@ __device__ __forceinline__ double abs_(double x) { return fabs(x); }
 // Arithmetic with its rounding fixed: the compiler neither fuses nor splits
 // these, so an expression written with them rounds the same way in every
 // kernel it is inlined into (a Newton iterate then converges to the same
-// last bit whatever the tile shape or launch form).
+// last bit whatever the tile shape or launch form).  The step kernels, whose
+// instantiations have to step a node alike, are compiled without contraction
+// (build.py), so the functions they share write their fused operations out.
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__host__ __device__ __forceinline__ float fm(float a, float b, float c) { return fmaf(a, b, c); }
+__host__ __device__ __forceinline__ double fm(double a, double b, double c) { return fma(a, b, c); }
 
 template <typename R>
 struct Macro {
@@ -54,33 +71,47 @@ struct Macro {
 
 // rho = sum f, rho u = sum f c, 2 rho E = sum g, T = (E - u^2/2) / Cv.
 template <typename R>
-__device__ __forceinline__ Macro<R> moments(const R* f, const R* g, R Cv) {
-    R rho = 0, jx = 0, jy = 0, s2 = 0;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        rho += f[q];
-        jx += (R)cxq(q) * f[q];
-        jy += (R)cyq(q) * f[q];
-        s2 += g[q];
-    }
+__device__ __forceinline__ Macro<R> moments(const R* f, const R* g, R iCv) {
+    const R rho = (f[0] + ((f[1] + f[3]) + (f[2] + f[4]))) + ((f[5] + f[7]) + (f[6] + f[8]));
+    const R s2 = (g[0] + ((g[1] + g[3]) + (g[2] + g[4]))) + ((g[5] + g[7]) + (g[6] + g[8]));
+    const R d = f[5] - f[7], e = f[6] - f[8];
+    const R jx = (f[1] - f[3]) + (d - e), jy = (f[2] - f[4]) + (d + e);
     Macro<R> m;
     const R ir = rcp_(rho);
     m.rho = rho;
     m.ux = jx * ir;
     m.uy = jy * ir;
     m.E = R(0.5) * s2 * ir;
-    m.T = (m.E - R(0.5) * (m.ux * m.ux + m.uy * m.uy)) * rcp_(Cv);
+    m.T = fm(R(-0.5), fm(m.ux, m.ux, m.uy * m.uy), m.E) * iCv;
     return m;
 }
 
 // Product-form equilibrium f_i^eq = rho Phi_{cx}(u_x) Phi_{cy}(u_y) (Eq. feq).
 template <typename R>
 __host__ __device__ __forceinline__ void f_equilibrium(R rho, R ux, R uy, R T, R* f) {
-    R ax = ux * ux + T, ay = uy * uy + T;
+    const R ax = fm(ux, ux, T), ay = fm(uy, uy, T);
     R px[3] = {R(0.5) * (ax - ux), R(1) - ax, R(0.5) * (ax + ux)};   // index c+1
     R py[3] = {R(0.5) * (ay - uy), R(1) - ay, R(0.5) * (ay + uy)};
 #pragma unroll
-    for (int q = 0; q < 9; ++q) f[q] = rho * px[cxq(q) + 1] * py[cyq(q) + 1];
+    for (int c = 0; c < 3; ++c) px[c] *= rho;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) f[q] = px[cxq(q) + 1] * py[cyq(q) + 1];
+}
+
+// W_i (z + q.c + A:(c c - T I)/(2T^2)) with the weights W of T: z the zeroth
+// moment, q the first over T, A the second (the Hermite expansions of g and
+// of the non-equilibrium parts); the last term takes five values (rest,
+// x-axis, y-axis and the two diagonal pairs).
+template <typename R>
+__host__ __device__ __forceinline__ void hermite(R T, R iT, R z, R qx, R qy, R axx, R axy, R ayy, R* g) {
+    const R iT2 = iT * iT, i2 = R(0.5) * iT2, A = axx + ayy, TA = T * A;
+    const R w0 = R(0.5) * T, w1 = R(1) - T, Wa = w0 * w1, Wd = w0 * w0;
+    g[0] = w1 * w1 * fm(-TA, i2, z);
+    const R gx = Wa * fm(axx - TA, i2, z), gy = Wa * fm(ayy - TA, i2, z);
+    g[1] = fm(Wa, qx, gx); g[3] = fm(-Wa, qx, gx); g[2] = fm(Wa, qy, gy); g[4] = fm(-Wa, qy, gy);
+    const R gd = Wd * fm(A - TA, i2, z), t = axy * iT2;
+    const R gp = fm(Wd, t, gd), gm = fm(-Wd, t, gd), sp = qx + qy, sm = qx - qy;
+    g[5] = fm(Wd, sp, gp); g[7] = fm(-Wd, sp, gp); g[8] = fm(Wd, sm, gm); g[6] = fm(-Wd, sm, gm);
 }
 
 // g = W_i (2 rho E + q.c/T + (R^eq - 2 rho E T I):(c c - T I)/(2T^2)) + Psi_i
@@ -88,33 +119,22 @@ __host__ __device__ __forceinline__ void f_equilibrium(R rho, R ux, R uy, R T, R
 // Psi_i = B_i . X with B_0 = (1,1), B_{1,3} = (-1/2,0), B_{2,4} = (0,-1/2).
 template <typename R>
 __host__ __device__ __forceinline__ void g_hermite(R rho, R ux, R uy, R T, R E, R qx, R qy, R* g) {
-    const R uxx = ux * ux, uyy = uy * uy, uxy = ux * uy;
+    const R uxx = ux * ux, uyy = uy * uy, p = rho * T, e2 = R(2) * rho * E;
+    const R e4 = fm(R(4), p, e2), pT = R(2) * p * T, iT = rcp_(T);
     // A = R^eq - 2 rho E T I
-    const R axx = R(2) * rho * E * uxx + R(2) * rho * T * (T + R(2) * uxx);
-    const R ayy = R(2) * rho * E * uyy + R(2) * rho * T * (T + R(2) * uyy);
-    const R axy = R(2) * rho * E * uxy + R(4) * rho * T * uxy;
-    const R invT = rcp_(T);
-    const R inv2T2 = R(0.5) * invT * invT;
-    const R pre = rho * (R(1) - R(3) * T) * invT;
-    const R Xx = pre * (T * T + R(2) * uxx * T + E * uxx);
-    const R Xy = pre * (T * T + R(2) * uyy * T + E * uyy);
-    const R w[3] = {R(0.5) * T, R(1) - T, R(0.5) * T};
-    const R twoRhoE = R(2) * rho * E;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const int cx = cxq(q), cy = cyq(q);
-        const R herm = (axx * (R(cx * cx) - T) + R(2) * axy * R(cx * cy) + ayy * (R(cy * cy) - T)) * inv2T2;
-        R v = w[cx + 1] * w[cy + 1] * (twoRhoE + (qx * R(cx) + qy * R(cy)) * invT + herm);
-        if (q == 0) v += Xx + Xy;
-        if (q == 1 || q == 3) v -= R(0.5) * Xx;
-        if (q == 2 || q == 4) v -= R(0.5) * Xy;
-        g[q] = v;
-    }
+    hermite(T, iT, e2, qx * iT, qy * iT, fm(uxx, e4, pT), ux * uy * e4, fm(uyy, e4, pT), g);
+    const R pre = rho * fm(R(-3), T, R(1)) * iT, tE = fm(R(2), T, E), TT = T * T;
+    const R Xx = pre * fm(uxx, tE, TT), Xy = pre * fm(uyy, tE, TT), hx = R(0.5) * Xx, hy = R(0.5) * Xy;
+    g[0] += Xx + Xy;
+    g[1] -= hx;
+    g[3] -= hx;
+    g[2] -= hy;
+    g[4] -= hy;
 }
 
 template <typename R>
 __host__ __device__ __forceinline__ void g_equilibrium(R rho, R ux, R uy, R T, R Cv, R* g) {
-    const R E = Cv * T + R(0.5) * (ux * ux + uy * uy);
+    const R E = fm(Cv, T, R(0.5) * fm(ux, ux, uy * uy));
     const R H2 = R(2) * rho * (E + T);
     g_hermite(rho, ux, uy, T, E, H2 * ux, H2 * uy, g);
 }
@@ -134,96 +154,102 @@ __device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ float2 pair(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 pair(double a, double b) { return make_double2(a, b); }
 
-// Collision at one node (Eq. f_boltz) on its (f_q, g_q) pairs p[9]:
-// f* = f + w (f^eq - f) + dt phi, g* = g + w (g^eq - g) + (w1 - w)(g^qe - g).
-// phi_i = -(1/2) c_i . Y on the axis velocities; q* = q^eq + 2 u.(P - P^eq);
-// 1/w = 1/2 + mu/(rho T dt), 1/w1 = 1/2 + (1/w - 1/2)/Pr.  g^qe differs from
-// g^eq only in the heat flux, so both come from one Hermite expansion, whose
-// (R^eq - 2 rho E T I):(c c - T I)/(2T^2) term takes five values (rest,
-// x-axis, y-axis and the two diagonal pairs).
+// What the collision of a node needs of its populations and relaxes them to.
+// q* = q^eq + 2 u.(P - P^eq); 1/w = 1/2 + mu/(rho T dt), 1/w1 = 1/2 +
+// (1/w - 1/2)/Pr.  g^qe differs from g^eq only in the heat flux, and
+//   w (g^eq - g) + (w1 - w)(g^qe - g) = w1 (g' - g)
+// for the g' of the one Hermite expansion with the flux q^eq + (1 - w/w1)
+// (q* - q^eq), so one relaxation serves both; its (R^eq - 2 rho E T I):
+// (c c - T I)/(2T^2) term takes five values (rest, x-axis, y-axis and the two
+// diagonal pairs).
+template <typename R>
+struct Collision {
+    R rho, e2, ux, uy, T, E, p, ax, ay, uxx, uyy, uxy, w, w1, iT, qx, qy;   // q: that flux over T
+    template <typename R2>
+    __device__ __forceinline__ void moments(const R2* p_, R mu, R muP, R dt, R iCv) {
+        // opposite directions in pairs: their sums give rho, 2 rho E and P,
+        // their differences rho u
+        const R2 a = padd(p_[1], p_[3]), b = padd(p_[2], p_[4]), c = padd(p_[5], p_[7]), d = padd(p_[6], p_[8]);
+        const R2 e = padd(c, d), s = padd(padd(p_[0], a), padd(b, e));
+        rho = s.x;
+        e2 = s.y;
+        const R d5 = p_[5].x - p_[7].x, d6 = p_[6].x - p_[8].x;
+        const R jx = (p_[1].x - p_[3].x) + (d5 - d6), jy = (p_[2].x - p_[4].x) + (d5 + d6);
+        const R ir = rcp_(rho);
+        ux = jx * ir;
+        uy = jy * ir;
+        E = R(0.5) * e2 * ir;
+        uxx = ux * ux;
+        uyy = uy * uy;
+        uxy = ux * uy;
+        T = fm(R(-0.5), uxx + uyy, E) * iCv;
+        p = rho * T;
+        ax = uxx + T;
+        ay = uyy + T;
+        // w = p dt / (p dt / 2 + mu), w1 with mu / Pr; 1 - w/w1 = (mu - mu/Pr) / (p dt / 2 + mu)
+        const R pd = p * dt, rA = rcp_(fm(R(0.5), pd, mu));
+        w = pd * rA;
+        w1 = pd * rcp_(fm(R(0.5), pd, muP));
+        const R dxx = fm(-rho, ax, a.x + e.x), dyy = fm(-rho, ay, b.x + e.x), dxy = fm(-rho, uxy, c.x - d.x);
+        iT = rcp_(T);
+        const R H2 = fm(R(2), p, e2) * iT, r = R(2) * iT * ((mu - muP) * rA);
+        qx = fm(H2, ux, r * fm(ux, dxx, uy * dxy));
+        qy = fm(H2, uy, r * fm(ux, dxy, uy * dyy));
+    }
+    __device__ __forceinline__ void f_target(R* f) const {
+        const R hr = R(0.5) * rho;
+        const R x0 = rho * (R(1) - ax), x1 = hr * (ax + ux), x3 = hr * (ax - ux);
+        const R y0 = R(1) - ay, y1 = R(0.5) * (ay + uy), y3 = R(0.5) * (ay - uy);
+        f[0] = x0 * y0; f[1] = x1 * y0; f[3] = x3 * y0; f[2] = x0 * y1; f[4] = x0 * y3;
+        f[5] = x1 * y1; f[6] = x3 * y1; f[7] = x3 * y3; f[8] = x1 * y3;
+    }
+    __device__ __forceinline__ void g_target(R* g) const {
+        const R iT2 = iT * iT, i2 = R(0.5) * iT2;
+        const R e4 = fm(R(4), p, e2), pT = R(2) * p * T;
+        const R axx = fm(uxx, e4, pT), ayy = fm(uyy, e4, pT), A = axx + ayy, TA = T * A;
+        const R pre = rho * fm(R(-3), T, R(1)) * iT, tE = fm(R(2), T, E), TT = T * T;
+        const R Xx = pre * fm(uxx, tE, TT), Xy = pre * fm(uyy, tE, TT);
+        const R w0 = R(0.5) * T, w1_ = R(1) - T, Wa = w0 * w1_, Wd = w0 * w0;
+        g[0] = fm(w1_ * w1_, fm(-TA, i2, e2), Xx + Xy);
+        const R gx = fm(Wa, fm(axx - TA, i2, e2), R(-0.5) * Xx), gy = fm(Wa, fm(ayy - TA, i2, e2), R(-0.5) * Xy);
+        g[1] = fm(Wa, qx, gx); g[3] = fm(-Wa, qx, gx); g[2] = fm(Wa, qy, gy); g[4] = fm(-Wa, qy, gy);
+        const R gd = Wd * fm(A - TA, i2, e2), t = uxy * e4 * iT2;
+        const R gp = fm(Wd, t, gd), gm = fm(-Wd, t, gd), sp = qx + qy, sm = qx - qy;
+        g[5] = fm(Wd, sp, gp); g[7] = fm(-Wd, sp, gp); g[8] = fm(Wd, sm, gm); g[6] = fm(-Wd, sm, gm);
+    }
+};
+
+// Collision at one node (Eq. f_boltz) on its (f_q, g_q) pairs p[9]: f* = f +
+// w (f^eq - f) + dt phi, g* = g + w (g^eq - g) + (w1 - w)(g^qe - g), phi_i =
+// -(1/2) c_i . Y on the axis velocities.  muP = mu / Pr, iCv = 1 / Cv.
 template <typename R, typename R2>
-__device__ __forceinline__ void collide_pairs(R2* p, R Yx, R Yy, R mu, R dt, R Cv, R iPr) {
-    // rho = sum f, 2 rho E = sum g, rho u = sum f c, P = sum f c c
-    R2 s = p[0];
-#pragma unroll
-    for (int q = 1; q < 9; ++q) s = padd(s, p[q]);
-    const R rho = s.x, twoRhoE = s.y;
-    const R jx = ((p[1].x - p[3].x) + (p[5].x - p[6].x)) + (p[8].x - p[7].x);
-    const R jy = ((p[2].x - p[4].x) + (p[5].x - p[8].x)) + (p[6].x - p[7].x);
-    const R sd = (p[5].x + p[6].x) + (p[7].x + p[8].x);
-    const R pxx = (p[1].x + p[3].x) + sd, pyy = (p[2].x + p[4].x) + sd;
-    const R pxy = (p[5].x - p[6].x) + (p[7].x - p[8].x);
-    const R ir = rcp_(rho);
-    const R ux = jx * ir, uy = jy * ir;
-    const R E = R(0.5) * twoRhoE * ir;
-    const R uxx = ux * ux, uyy = uy * uy, uxy = ux * uy;
-    const R T = (E - R(0.5) * (uxx + uyy)) * rcp_(Cv);
-    const R tau = R(0.5) + mu * rcp_(rho * T * dt);
-    const R om = rcp_(tau);
-    const R om1 = rcp_(R(0.5) + (tau - R(0.5)) * iPr);
-    const R dom = om1 - om;
-    const R dxx = pxx - rho * (uxx + T);
-    const R dxy = pxy - rho * uxy;
-    const R dyy = pyy - rho * (uyy + T);
-    const R invT = rcp_(T);
-    // heat flux of g^eq (2 rho H u) and the quasi-equilibrium shift
-    // q* - q^eq = 2 u.(P - P^eq), both over T
-    const R H2 = R(2) * rho * (E + T) * invT;
-    const R qx = H2 * ux, qy = H2 * uy;
-    const R dqx = R(2) * (ux * dxx + uy * dxy) * invT, dqy = R(2) * (ux * dxy + uy * dyy) * invT;
-    const R rT2 = R(2) * rho * T;
-    const R axx = twoRhoE * uxx + rT2 * (T + R(2) * uxx);
-    const R ayy = twoRhoE * uyy + rT2 * (T + R(2) * uyy);
-    const R axy = twoRhoE * uxy + R(2) * rT2 * uxy;
-    const R inv2T2 = R(0.5) * invT * invT;
-    const R A = axx + ayy, TA = T * A;
-    const R h0 = -TA * inv2T2, hx = (axx - TA) * inv2T2, hy = (ayy - TA) * inv2T2;
-    const R hd = (A - TA) * inv2T2, hxy = R(2) * axy * inv2T2;
-    const R pre = rho * (R(1) - R(3) * T) * invT;
-    const R Xx = pre * (T * T + R(2) * uxx * T + E * uxx);
-    const R Xy = pre * (T * T + R(2) * uyy * T + E * uyy);
-    const R ax = uxx + T, ay = uyy + T;
-    const R px[3] = {R(0.5) * (ax - ux), R(1) - ax, R(0.5) * (ax + ux)};
-    const R py[3] = {R(0.5) * (ay - uy), R(1) - ay, R(0.5) * (ay + uy)};
-    const R w0 = R(0.5) * T, w1 = R(1) - T;
-    const R Wr = w1 * w1, Wa = w0 * w1, Wd = w0 * w0;
-    const R2 om2 = pair(om, om);
+__device__ __forceinline__ void collide_pairs(R2* p, R Yx, R Yy, R mu, R muP, R dt, R iCv) {
+    Collision<R> c;
+    c.moments(p, mu, muP, dt, iCv);
+    R fe[9], ge[9];
+    c.f_target(fe);
+    c.g_target(ge);
+    const R2 om = pair(c.w, c.w1);
     R2 d[9];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const int cx = cxq(q), cy = cyq(q);
-        const R feq = rho * px[cx + 1] * py[cy + 1];
-        const R herm = q == 0 ? h0 : (cy == 0 ? hx : (cx == 0 ? hy : hd + R(cx * cy) * hxy));
-        const R W = q == 0 ? Wr : (cx == 0 || cy == 0 ? Wa : Wd);
-        const R flux = (cx ? R(cx) * qx : R(0)) + (cy ? R(cy) * qy : R(0));
-        R geq = W * (twoRhoE + flux + herm);
-        if (q == 0) geq += Xx + Xy;
-        if (q == 1 || q == 3) geq -= R(0.5) * Xx;
-        if (q == 2 || q == 4) geq -= R(0.5) * Xy;
-        const R shift = (cx ? R(cx) * dqx : R(0)) + (cy ? R(cy) * dqy : R(0));
-        const R gqe = geq + W * shift;
-        // (w (f^eq - f), w (g^eq - g) + (w1 - w)(g^qe - g))
-        d[q] = pfma(om2, psub(pair(feq, geq), p[q]), pair(R(0), dom * (gqe - p[q].y)));
-    }
+    for (int q = 0; q < 9; ++q) d[q] = pmul(om, psub(pair(fe[q], ge[q]), p[q]));
     if constexpr (sizeof(R) == 4) {
         // The relaxation leaves mass, momentum and energy unchanged in exact
-        // arithmetic (sum f^eq = rho, sum f^eq c = rho u, sum g^eq = sum g^qe =
-        // 2 rho E).  In float the rounded equilibria miss that by an ulp, and
+        // arithmetic (sum f^eq = rho, sum f^eq c = rho u, sum g' = 2 rho E).
+        // In float the rounded targets miss that by an ulp, and
         // at a node whose state barely changes the miss has the same sign at
         // every step, so it accumulates.  Its sums over the small changes are
         // exact to far below the populations' ulp: take them out of the rest
         // population (mass, energy) and of the axis pairs (momentum; their
         // sum, hence the mass, unchanged).
-        R2 e = d[0];
-#pragma unroll
-        for (int q = 1; q < 9; ++q) e = padd(e, d[q]);
-        const R ex = ((d[1].x - d[3].x) + (d[5].x - d[6].x)) + (d[8].x - d[7].x);
-        const R ey = ((d[2].x - d[4].x) + (d[5].x - d[8].x)) + (d[6].x - d[7].x);
-        d[0] = psub(d[0], e);
-        d[1].x -= R(0.5) * ex;
-        d[3].x += R(0.5) * ex;
-        d[2].x -= R(0.5) * ey;
-        d[4].x += R(0.5) * ey;
+        const R2 e = padd(padd(padd(d[1], d[3]), padd(d[2], d[4])), padd(padd(d[5], d[7]), padd(d[6], d[8])));
+        const R d5 = d[5].x - d[7].x, d6 = d[6].x - d[8].x;
+        const R ex = R(0.5) * ((d[1].x - d[3].x) + (d5 - d6)), ey = R(0.5) * ((d[2].x - d[4].x) + (d5 + d6));
+        d[0] = pmul(e, pair(R(-1), R(-1)));   // (d[0] minus the sum with d[0])
+        d[1].x -= ex;
+        d[3].x += ex;
+        d[2].x -= ey;
+        d[4].x += ey;
     }
     // dt phi on the axis velocities
     const R hyx = R(0.5) * dt * Yx, hyy = R(0.5) * dt * Yy;
@@ -236,46 +262,54 @@ __device__ __forceinline__ void collide_pairs(R2* p, R Yx, R Yy, R mu, R dt, R C
 }
 
 // Grad's approximation at wall targets (Sec. III A, Eqs. fnoneq, gnoneq,
-// strainrate): f = f^eq + dt f1, g = g^eq + dt g1.  grad u as (d_x u_x, d_y u_x,
-// d_x u_y, d_y u_y), grad T as (d_x T, d_y T).
+// strainrate): f = f^eq + dt f1, g = g^eq + dt g1.  gr: the gradients (d_x u_x,
+// d_y u_x, d_x u_y, d_y u_y, d_x T, d_y T).
+template <typename R>
+struct WallTarget {
+    R rho, ux, uy, T, gr[6];
+};
+// P^(1) of the targets (over dt): xx, xy, yy.
+template <typename R>
+__device__ __forceinline__ void grad_p1(const WallTarget<R>& t, R iom, R iCv, R* p1) {
+    const R cP = -iom * t.rho * t.T, dv = (t.gr[0] + t.gr[3]) * iCv;
+    p1[0] = cP * fm(R(2), t.gr[0], -dv);
+    p1[1] = cP * (t.gr[2] + t.gr[1]);
+    p1[2] = cP * fm(R(2), t.gr[3], -dv);
+}
+template <typename R>
+__device__ __forceinline__ void grad_f(const WallTarget<R>& t, R mu, R dt, R iCv, R* f) {
+    const R iom = fm(mu, rcp_(t.rho * t.T * dt), R(0.5));   // 1/omega
+    R p1[3], h[9];
+    grad_p1(t, iom, iCv, p1);
+    f_equilibrium(t.rho, t.ux, t.uy, t.T, f);
+    hermite(t.T, rcp_(t.T), R(0), R(0), R(0), p1[0], p1[1], p1[2], h);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) f[q] = fm(dt, h[q], f[q]);
+}
+template <typename R>
+__device__ __forceinline__ void grad_g(const WallTarget<R>& t, R mu, R dt, R Cv, R iCv, R iPr, R* g) {
+    const R tau = mu * rcp_(t.rho * t.T * dt), iom = tau + R(0.5), iom1 = fm(tau, iPr, R(0.5));   // 1/omega, 1/omega_1
+    const R ux = t.ux, uy = t.uy, T = t.T;
+    R p1[3], h[9];
+    grad_p1(t, iom, iCv, p1);
+    const R E = fm(Cv, T, R(0.5) * fm(ux, ux, uy * uy)), iT = rcp_(T);
+    const R dEx = fm(Cv, t.gr[4], fm(ux, t.gr[0], uy * t.gr[2])), dEy = fm(Cv, t.gr[5], fm(ux, t.gr[1], uy * t.gr[3]));
+    const R cR = R(-2) * iom1 * t.rho * T, cq = cR * (Cv + R(1)), EpT = fm(R(2), T, E);
+    const R qx = fm(cq, t.gr[4], R(2) * fm(ux, p1[0], uy * p1[1])), qy = fm(cq, t.gr[5], R(2) * fm(ux, p1[1], uy * p1[2]));
+    const R rxx = cR * R(2) * fm(t.gr[0], EpT, ux * dEx), ryy = cR * R(2) * fm(t.gr[3], EpT, uy * dEy);
+    const R rxy = cR * fm(t.gr[2] + t.gr[1], EpT, fm(ux, dEy, dEx * uy));
+    g_equilibrium(t.rho, ux, uy, T, Cv, g);
+    hermite(T, iT, R(0), qx * iT, qy * iT, rxx, rxy, ryy, h);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) g[q] = fm(dt, h[q], g[q]);
+}
 template <typename R>
 __device__ __forceinline__ void grad_populations(R rho, R ux, R uy, R T, R dudx, R dudy, R dvdx,
-                                                 R dvdy, R dTdx, R dTdy, R mu, R dt, R Cv, R Pr,
+                                                 R dvdy, R dTdx, R dTdy, R mu, R dt, R Cv, R iCv, R iPr,
                                                  R* f, R* g) {
-    const R Cp = Cv + R(1);
-    const R iom = R(0.5) + mu * rcp_(rho * T * dt);      // 1/omega
-    const R iom1 = R(0.5) + (iom - R(0.5)) * rcp_(Pr);  // 1/omega_1
-    const R E = Cv * T + R(0.5) * (ux * ux + uy * uy);
-    const R sxx = R(2) * dudx, syy = R(2) * dvdy, sxy = dvdx + dudy;
-    const R div = dudx + dvdy;
-    const R iCv = rcp_(Cv);
-    const R cP = -iom * rho * T;
-    const R p1xx = cP * (sxx - div * iCv), p1yy = cP * (syy - div * iCv), p1xy = cP * sxy;
-    const R dEdx = Cv * dTdx + ux * dudx + uy * dvdx;
-    const R dEdy = Cv * dTdy + ux * dudy + uy * dvdy;
-    const R cq = -R(2) * iom1 * rho * Cp * T;
-    const R q1x = cq * dTdx + R(2) * (ux * p1xx + uy * p1xy);
-    const R q1y = cq * dTdy + R(2) * (ux * p1xy + uy * p1yy);
-    const R cR = -R(2) * iom1 * rho * T;
-    const R EpT = E + R(2) * T;
-    const R r1xx = cR * (sxx * EpT + R(2) * ux * dEdx);
-    const R r1yy = cR * (syy * EpT + R(2) * uy * dEdy);
-    const R r1xy = cR * (sxy * EpT + ux * dEdy + dEdx * uy);
-    f_equilibrium(rho, ux, uy, T, f);
-    g_equilibrium(rho, ux, uy, T, Cv, g);
-    const R w[3] = {R(0.5) * T, R(1) - T, R(0.5) * T};
-    const R invT = rcp_(T);
-    const R inv2T2 = R(0.5) * invT * invT;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const int cx = cxq(q), cy = cyq(q);
-        const R W = w[cx + 1] * w[cy + 1];
-        const R dxx = R(cx * cx) - T, dyy = R(cy * cy) - T, dxy = R(cx * cy);
-        const R hp = (p1xx * dxx + R(2) * p1xy * dxy + p1yy * dyy) * inv2T2;
-        const R hr = (r1xx * dxx + R(2) * r1xy * dxy + r1yy * dyy) * inv2T2;
-        f[q] += dt * W * hp;
-        g[q] += dt * W * ((q1x * R(cx) + q1y * R(cy)) * invT + hr);
-    }
+    const WallTarget<R> t{rho, ux, uy, T, {dudx, dudy, dvdx, dvdy, dTdx, dTdy}};
+    grad_f(t, mu, dt, iCv, f);
+    grad_g(t, mu, dt, Cv, iCv, iPr, g);
 }
 
 // Rotation part of a body state: sin(alpha) and cos(alpha) - 1 written as
@@ -335,29 +369,29 @@ __device__ __forceinline__ bool kinematics(const BodyMap<R>& bm, R X, R Y, R& F0
     F00 = R(1); F01 = R(0); F10 = R(0); F11 = R(1); vx = R(0); vy = R(0);
     if (!bm.active) return false;
     const R dx = X - bm.xc, dy = Y - bm.yc;
-    const R dist = sqrt_(dx * dx + dy * dy);
+    const R dist = sqrt_(fm(dx, dx, dy * dy));
     const R s = (dist - bm.r_in) * bm.inv_w;
     if (s > R(1)) return false;
     R w, drx = R(0), dry = R(0);
     if (s < R(0)) {
         w = R(1);
     } else {
-        const R r5 = s * s * s * (R(10) - R(15) * s + R(6) * s * s);
-        const R d5 = R(30) * s * s * (R(1) - s) * (R(1) - s);
-        w = R(1) - r5;
-        const R gq = d5 * bm.inv_w * rcp_(dist);
+        // r5 = s^3 (10 - 15 s + 6 s^2), dr5/ds = 30 s^2 (1 - s)^2
+        const R t = s * (R(1) - s);
+        w = fm(-(s * s * s), fm(s, fm(R(6), s, R(-15)), R(10)), R(1));
+        const R gq = R(30) * t * t * bm.inv_w * rcp_(dist);
         drx = gq * dx;
         dry = gq * dy;
     }
     const R px = X - bm.xp, py = Y - bm.yp;
-    const R ux = bm.a00 * px + bm.a01 * py + bm.tx;
-    const R uy = bm.a10 * px + bm.a11 * py + bm.ty;
-    F00 = R(1) + w * bm.a00 - ux * drx;
-    F01 = w * bm.a01 - ux * dry;
-    F10 = w * bm.a10 - uy * drx;
-    F11 = R(1) + w * bm.a11 - uy * dry;
-    vx = w * (bm.va00 * px + bm.va01 * py + bm.vtx);
-    vy = w * (bm.va10 * px + bm.va11 * py + bm.vty);
+    const R ux = fm(bm.a00, px, fm(bm.a01, py, bm.tx));
+    const R uy = fm(bm.a10, px, fm(bm.a11, py, bm.ty));
+    F00 = fm(-ux, drx, fm(w, bm.a00, R(1)));
+    F01 = fm(-ux, dry, w * bm.a01);
+    F10 = fm(-uy, drx, w * bm.a10);
+    F11 = fm(-uy, dry, fm(w, bm.a11, R(1)));
+    vx = w * fm(bm.va00, px, fm(bm.va01, py, bm.vtx));
+    vy = w * fm(bm.va10, px, fm(bm.va11, py, bm.vty));
     return true;
 }
 

@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(EM_THREADS) k_em_collide(const EArgs a) {
             }, xX, xY, yX, yY);
             const R Yx = i00 * xX + i10 * xY, Yy = i01 * yX + i11 * yY;
             collide_pairs(pq, Yx, Yy, flowv<R>(a.flow, a.flow.mu, a.flow.mu_f),
-                          flowv<R>(a.flow, a.flow.dt, a.flow.dt_f), Cv,
-                          flowv<R>(a.flow, 1.0 / a.flow.Pr, a.flow.iPr_f));
+                          flowv<R>(a.flow, a.flow.muP, a.flow.muP_f), flowv<R>(a.flow, a.flow.dt, a.flow.dt_f),
+                          flowv<R>(a.flow, a.flow.iCv, a.flow.iCv_f));
         }
     }
 #pragma unroll
@@ -499,7 +499,8 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
                 }
                 R fw[9], gw[9];
                 grad_populations(t[0], vx, vy, t[3], gr[0][0], gr[0][1], gr[1][0], gr[1][1], gr[2][0], gr[2][1],
-                                 flowv<R>(fl, fl.mu, fl.mu_f), dt, Cv, flowv<R>(fl, fl.Pr, fl.Pr_f), fw, gw);
+                                 flowv<R>(fl, fl.mu, fl.mu_f), dt, Cv, flowv<R>(fl, fl.iCv, fl.iCv_f),
+                                 flowv<R>(fl, fl.iPr, fl.iPr_f), fw, gw);
 #pragma unroll
                 for (int q = 0; q < 9; ++q)
                     if (missing & (1u << q)) {
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
                         g[q] = gw[q];
                     }
             }
-            const Macro<R> mc = moments(f, g, Cv);
+            const Macro<R> mc = moments(f, g, flowv<R>(fl, fl.iCv, fl.iCv_f));
             if (!(mc.rho > R(0)) || !(mc.T > R(0)) || !isfinite(mc.ux) || !isfinite(mc.uy))
                 atomicOr(a.status, ST_NONPHYS);
 #pragma unroll
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
                     fd[q] = (double)f[q];
                     gd[q] = (double)g[q];
                 }
-                const Macro<double> md = moments(fd, gd, fl.Cv);
+                const Macro<double> md = moments(fd, gd, fl.iCv);
                 f_equilibrium(md.rho, md.ux, md.uy, md.T, feq);
                 double pxx = 0, pxy = 0, pyy = 0;
 #pragma unroll

@@ -651,6 +651,33 @@ BodyDev body_dev(const lbfsi_body_desc& d, double rho, double U) {
     return b;
 }
 
+// The RK4 map's columns: the step applied to unit states, loads and
+// accelerations (the step is linear and maps zero to zero).
+BodyProp body_prop(const BodyDev& b, double dt) {
+    BodyProp p{};
+    const long long never_forced = 1ll << 60;
+    for (int c = 0; c < 6; ++c) {
+        const double e[6] = {c == 0 ? 1.0 : 0.0, c == 1 ? 1.0 : 0.0, c == 2 ? 1.0 : 0.0,
+                             c == 3 ? 1.0 : 0.0, c == 4 ? 1.0 : 0.0, c == 5 ? 1.0 : 0.0};
+        const BodyStateDev s = rk4_body(b, BodyStateDev{e[0], e[1], e[2], e[3]}, e[4], e[5], dt, never_forced);
+        p.free[0][c] = s.h;
+        p.free[1][c] = s.alpha;
+        p.free[2][c] = s.hdot;
+        p.free[3][c] = s.adot;
+        if (b.dof != 2) continue;
+        // m h'' + S_alpha alpha''(t) + k_h h = F_y with alpha'' prescribed
+        auto acc = [&](double a, double h) { return (e[2] - b.k_h * h - b.s_a * a) / b.m; };
+        const double h0 = e[0], v0 = e[1];
+        const double k1h = v0, k1v = acc(e[3], h0);
+        const double k2h = v0 + 0.5 * dt * k1v, k2v = acc(e[4], h0 + 0.5 * dt * k1h);
+        const double k3h = v0 + 0.5 * dt * k2v, k3v = acc(e[4], h0 + 0.5 * dt * k2h);
+        const double k4h = v0 + dt * k3v, k4v = acc(e[5], h0 + dt * k3h);
+        p.forced[0][c] = h0 + dt / 6.0 * (k1h + 2.0 * k2h + 2.0 * k3h + k4h);
+        p.forced[1][c] = v0 + dt / 6.0 * (k1v + 2.0 * k2v + 2.0 * k3v + k4v);
+    }
+    return p;
+}
+
 double flow_u_inf(const lbfsi_flow_params& p) { return p.ma * std::sqrt(p.gamma * p.t_inf); }
 
 int fill_flow(const lbfsi_flow_params& p, SolveDev& s) {
@@ -663,7 +690,13 @@ int fill_flow(const lbfsi_flow_params& p, SolveDev& s) {
     s.dt = p.dt;
     s.mu = mu;
     s.Cv = 1.0 / (p.gamma - 1.0);
+    s.iCv = 1.0 / s.Cv;
+    s.idt = 1.0 / s.dt;
     s.Pr = p.pr;
+    s.iPr = 1.0 / s.Pr;
+    s.muP = s.mu / s.Pr;
+    s.iCv_f = (float)s.iCv;
+    s.muP_f = (float)s.muP;
     s.rho_inf = p.rho_inf;
     s.uinf_x = U;
     s.uinf_y = 0.0;
@@ -740,7 +773,13 @@ int upload_mesh(const HostMesh& h, int precision, DevMemory& mem, cudaStream_t s
     void *pxw = nullptr, *pfd = nullptr, *px = nullptr, *pj = nullptr, *pc = nullptr, *pfj = nullptr;
     void* pct_ = nullptr;
     int rc = put(h.n0, false, &pn);
-    if (!rc) rc = put(h.wall_geo, false, &pw);
+    // the two edge shares of a wall node, (weight times length, unit normal),
+    // as one vector
+    std::vector<double> share(2 * (size_t)h.nt, 0.0);
+    for (size_t j = 0; j < (size_t)h.nt; ++j)
+        for (int e = 0; e < 2; ++e)
+            for (int c = 0; c < 2; ++c) share[2 * j + c] += h.wall_geo[6 * j + 3 * e] * h.wall_geo[6 * j + 3 * e + 1 + c];
+    if (!rc) rc = put(share, false, &pw);
     if (!rc) rc = put(h.xw, false, &pxw);
     if (!rc) rc = put(h.fardir, false, &pfd);
     if (h.general) {
@@ -774,7 +813,7 @@ int upload_mesh(const HostMesh& h, int precision, DevMemory& mem, cudaStream_t s
     d.r = (const double*)pr;
     d.e = (const double*)pe;
     d.n0 = (const double*)pn;
-    d.wall_geo = (const double*)pw;
+    d.wall_share = (const double*)pw;
     d.rowtab = prt;
     d.coltab = pct;
     d.xw = (const double*)pxw;

@@ -32,6 +32,14 @@ struct BodyStateDev {
     double h, alpha, hdot, adot;
 };
 
+// One RK4 step of a body over the flow's dt under a held load (Sec. III B) as
+// the linear map it is: row r of free gives state entry r from (h, alpha, hdot,
+// adot, F_y, M); forced gives (h, hdot) of a step in the forcing interval from
+// (h, hdot, F_y, alpha'' at the step's start, middle and end).
+struct BodyProp {
+    double free[4][6], forced[2][6];
+};
+
 // Per-row and per-column geometry of the O-grid X = centre + r_i e_j (see
 // the table builder in lbfsi_api.cu for the meaning of each entry).
 // Entries are grouped in fours so that a kernel reads each group with one
@@ -69,15 +77,8 @@ struct StepMaps {
     BodyMap<float> Kf, Sf;
 };
 
-enum StepMode : int { MODE_STREAM_ONLY = 0, MODE_COLLIDE_STREAM = 1, MODE_COLLIDE_ONLY = 2 };
-
-// Mirrored rows kept below row 0 of a C-grid (the +-4 staging halo).
+// Mirrored rows kept below row 0 of a C-grid (the moments' halo).
 constexpr int CGRID_GHOST_ROWS = 4;
-// Rows whose post-collision state a C-grid step's first launch writes: the
-// tiles of the first row of tiles stream from it (their +-2 window reaches
-// the mirrored rows, i.e. the other side's collided nodes); every other tile
-// collides its own window in the second launch.
-constexpr int CGRID_PRE_ROWS = 16;
 // Classes of a C-grid's row-0 columns: on the cut, on a wall chain, a
 // junction (a chain's end next to the cut, one point with its mirror), a
 // second copy of the mirrored column's node (past the middle of row 0), and
@@ -97,7 +98,8 @@ struct MeshDev {
     const double* r;               // [nr]
     const double* e;               // [nt][2]
     const double* n0;              // [nt][2] wall normals (undeformed)
-    const double* wall_geo;        // [nt][6] two (weight*length, n_x, n_y) edge shares per wall node
+    const double* wall_share;      // [nt][2] a wall node's Simpson share of its edges: sum of weight
+                                   // times length times unit normal (undeformed)
     const void* rowtab;            // [nr][ROWTAB] per-row geometry (element type of the path)
     const void* coltab;            // [nt][COLTAB] per-column geometry
     float xm_f, ym_f;
@@ -129,8 +131,9 @@ struct MeshDev {
 // step number k (counter[1]): after k step launches the state is in buffer
 // k & 1, and the launch with k == 0 streams from the initial (post-collision)
 // state without colliding.  counter[0] counts the CTAs of the solve that have
-// finished the current launch; the last one advances the body, resets
-// counter[0] and writes k + 1.
+// finished a step launch that reads k from the device (the last one resets it
+// and writes k + 1), counter[2] its finished loads blocks (the last one
+// advances the bodies).
 struct SolveDev {
     int mesh;
     int ntiles;                    // CTAs of this solve in every step launch
@@ -148,10 +151,16 @@ struct SolveDev {
     void* p[2];                    // populations, (f_q, g_q) pairs [9][N]
     void* M[2];                    // moments [4][N]
     StepMaps* maps[2];             // [nbody] each
-    void* ppost;                   // collide-only output (post-collision pairs)
+    void* ppost;                   // post-collision pairs [9][N] (float64 path: written by the field
+                                   // launch; float: only for the accessor)
+    void* Y;                       // float path: correction field [2][N] of the current state
     double* part;                  // [nbody][ntj][3] load partials of the streamed step
-    unsigned* counter;             // [2]: CTA completion count, step number k
+    unsigned* counter;             // [4]: CTA count of the step launch, step number k, loads
+                                   // blocks done, unused
     const BodyDev* body;           // [nbody]
+    const BodyProp* prop;          // [nbody]
+    double iCv, idt, iPr, muP;     // 1 / Cv, 1 / dt, 1 / Pr, mu / Pr
+    float iCv_f, muP_f;
     // general meshes, uniform launches: departure points of the nodes the
     // blend does not move (g = I, V_G = 0, so the displacement of direction q
     // is -dt c_q for every step): (xi, eta) pairs [9][N] in the element type
@@ -180,40 +189,62 @@ struct StepArgs {
     const SolveDev* solves;
     const TileDev* tiles;
     int ntiles;
-    int collide_only;              // 1: write the collided current state to ppost only
     int ustep;                     // uniform launch: the solves' step number (they advance
                                    // together), or -1 to read it from the device counters
     int uorder;                    // uniform launch: CTA order, 0 = (tile column, tile row,
                                    // solve), 1 = (solve, tile column, tile row)
-    int pf_dist;                   // uniform launch: L2 prefetch distance in CTAs (set by the launcher)
-    int stream_post;               // C-grid step, second launch: the tiles next to the cut
-                                   // (rows < CGRID_PRE_ROWS - tile - 2) stream from ppost
-                                   // (written by the step's collide-only launch) without
-                                   // colliding, every other tile collides and streams in one
-                                   // pass; the step with k == 0 streams the initial state as
-                                   // always
-    int cgrid_pre;                 // C-grid collide-only launch of a step: only the tiles of
-                                   // rows < CGRID_PRE_ROWS (the others return at once)
     int record;                    // general meshes, uniform: fill usol.dep_* (departures of
                                    // the static nodes of solve 0) and write nothing else
     unsigned* status;
-    // uniform launch of the float kernel: stage the populations and M^k of a
+    // uniform launch of the float kernel: stage the populations and Y of a
     // tile whose columns do not wrap by two tensor copies (TMA) into shared
-    // memory instead of per-thread copies.  tm_p[c] / tm_M[c] describe buffer
-    // c (c = k & 1) of all solves as 4-D float arrays: populations
-    // (2 nt, nr + tma_g, 9, nbatch) with boxes (2 (TJ + 8), TI + 4, 9, 1),
-    // moments (nt, nr + tma_g, 4, nbatch) with boxes (TJ + 8, TI + 8, 4, 1);
-    // tma_g: the mirrored rows a C-grid stores below row 0 (lbfsi_api.cu).
+    // memory instead of per-thread copies.  tm_p[c] describes population
+    // buffer c (c = k & 1) of all solves as a 4-D float array (2 nt, nr, 9,
+    // nbatch) with boxes (2 (TJ + 8), TI + 4, 9, 1), tm_Y the correction field
+    // as (nt, nr, 2, nbatch) with boxes (TJ + 8, TI + 4, 2, 1) (lbfsi_api.cu).
     int tma;
-    int tma_g;
     // table launch of the float separable kernel: per solve the tensor maps of
-    // its populations (buffers 0, 1) and moments (buffers 0, 1), in device
-    // memory, [solve][4], each a (2 nt, nr, 9, 1) or (nt, nr, 4, 1) float
-    // array with the boxes above; used by the tiles whose TileDev::tma is set
+    // its populations (buffers 0, 1) and of Y, in device memory, [solve][4]
+    // (the last unused), each an array of one solve with the boxes above;
+    // used by the tiles whose TileDev::tma is set
     const CUtensorMap* tmaps;
     alignas(64) CUtensorMap tm_p[2];
-    alignas(64) CUtensorMap tm_M[2];
+    alignas(64) CUtensorMap tm_Y;
 };
+
+// One block of a table launch of the field kernel: block number 'block' of a
+// solve's fields, or (fields == 0) of its loads.
+struct FieldTile {
+    int solve, mesh, fields, block;
+};
+
+// Field launch (lbfsi_fields.cu): the loads of the step that produced the
+// current state (loads) and the current state's correction field, in float64
+// its collision (fields).
+struct FieldArgs {
+    MeshDev umesh;                 // uniform launch: the mesh and solve 0
+    SolveDev usol;
+    const MeshDev* meshes;         // table launch
+    const SolveDev* solves;
+    const FieldTile* tiles;
+    int ntiles;
+    int uniform, nbatch;
+    int nfield;                    // uniform: field blocks per solve (set by the launcher)
+    int loads, fields;
+    int ustep;                     // uniform: the current state's step number, or -1 (device counters)
+    double* rec;                   // uniform: this step's records [nbatch][nbody][7] (Fx, Fy, M, h,
+                                   // alpha, hdot, adot), or null
+    unsigned* status;
+};
+// Blocks of a solve: of its fields and of its loads.
+int field_blocks(int precision, bool general, int nr, int nt);
+int load_blocks(int ntj);
+cudaError_t launch_fields(FieldArgs a, int precision, bool general, cudaStream_t s);
+// Post-collision populations of the current state of a float handle into
+// ppost, from its Y.
+cudaError_t launch_post(const SolveDev& S, const MeshDev& G, int cur, int nbatch, cudaStream_t s);
+
+// The step launch's tile shape is chosen by variant (see tile_rows).
 
 // Tensor map of a float array of dims (dx, dy, dz, dw), x fastest and dense,
 // read in boxes of (bx, by, bz, 1), elements outside the array as zeros;
@@ -226,23 +257,25 @@ bool encode_box4(CUtensorMap* map, void* base, size_t dx, size_t dy, size_t dz, 
 int set_error(int code, const std::string& msg);
 
 // Launchers (defined in lbfsi_step.cu).  variant selects the tile shape of
-// the step kernel (see tile_rows): five float shapes, float64 tiles of 8, 4
-// or 2 rows.
-cudaError_t launch_step(const StepArgs& a, int precision, int variant, cudaStream_t s);
+// the step kernel (see tile_rows): five float shapes on separable meshes, one
+// on general meshes, float64 blocks of 1, 2 or 4 rows.  Table launch (the batch
+// runtime) of the separable or the general-geometry kernel:
+cudaError_t launch_step(const StepArgs& a, int precision, bool general, int variant, cudaStream_t s);
 // Uniform launch over nbatch solves of one mesh (see StepArgs).
 cudaError_t launch_step_uniform(const StepArgs& a, int precision, int variant, int nbatch,
                                 cudaStream_t s);
 int tile_rows(int precision, int variant);
-// Tile rows of the general-geometry kernel, in uniform (mesh handle) and
-// table (batch runtime) launches alike: 8 in float64 (256 threads, one CTA
-// per SM), 12 in float (384 threads, two CTAs per SM: 24 resident warps
-// where an 8-row tile's registers and shared memory allowed 16).
-constexpr int GEN_TILE_ROWS = 8;
-constexpr int GEN_TILE_ROWS_FP32 = 12;
-inline int general_tile_rows(int precision) { return precision == 0 ? GEN_TILE_ROWS : GEN_TILE_ROWS_FP32; }
-// Table launch of the general-geometry kernel (the batch runtime's solves on
-// meshes given by node coordinates).
-cudaError_t launch_step_general_table(const StepArgs& a, int precision, cudaStream_t s);
+// Stream launch of the float64 path (lbfsi_stream64.cu): blocks of 'rows' rows
+// x 32 columns, each row by four warps that share the directions.
+cudaError_t launch_stream64(const StepArgs& a, bool uniform, bool general, int rows, int nbatch, cudaStream_t s);
+// Tile of the float general-geometry kernel, in uniform (mesh handle) and
+// table (batch runtime) launches alike.
+// (16 rows, three blocks per SM: elliptic O-grid 512 x 256 x 8 solves 103 us a
+// launch, 12 rows with four blocks of 192 threads the same, 8 rows 10% slower)
+constexpr int GEN_TILE_ROWS_FP32 = 16, GEN_THREADS_FP32 = 256, GEN_MINB_FP32 = 3;
+inline int general_tile_rows(int precision, int variant) {
+    return precision == 0 ? tile_rows(0, variant) : GEN_TILE_ROWS_FP32;
+}
 // Number of tile shapes of the float step kernel (variants 0 .. n-1); the
 // float64 kernel has one.
 int step_variants(int precision);

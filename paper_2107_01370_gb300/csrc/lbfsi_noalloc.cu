@@ -46,7 +46,7 @@ template <typename R>
 __global__ void __launch_bounds__(NA_TJ) k_wall_loads_noalloc(
     int nr, int nt, const double* __restrict__ r, const double* __restrict__ e, double xm,
     double ym, const R* __restrict__ f, const R* __restrict__ g,
-    const double* __restrict__ body_ref, double mu, double dt, double Cv,
+    const double* __restrict__ body_ref, double mu, double dt, double iCv,
     double* __restrict__ loads, NoAllocScratch* sc) {
     const int b = blockIdx.y, tile = blockIdx.x, ntj = gridDim.x;
     const int j = tile * NA_TJ + threadIdx.x;
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(NA_TJ) k_wall_loads_noalloc(
         }
         // sigma = -p I - (1 - omega/2) P^(1), P^(1) = sum (f - f^eq) c c (Sec. III),
         // float64 from the populations on, as in the step kernel
-        const lbfsi::Macro<double> mc = lbfsi::moments(fq, gq, Cv);
+        const lbfsi::Macro<double> mc = lbfsi::moments(fq, gq, iCv);
         double feq[9];
         lbfsi::f_equilibrium(mc.rho, mc.ux, mc.uy, mc.T, feq);
         double pxx = 0, pxy = 0, pyy = 0;
@@ -179,13 +179,13 @@ extern "C" int lbfsi_wall_loads_noalloc(int nr, int ntheta, int nbatch, int prec
     if (err != cudaSuccess)
         return lbfsi::set_error(LBFSI_ECUDA, std::string("scratch clear: ") + cudaGetErrorString(err));
     const dim3 grid(ntj, nbatch);
-    const double Cv = 1.0 / (gamma - 1.0);
+    const double iCv = gamma - 1.0;
     if (precision == LBFSI_FP64)
         k_wall_loads_noalloc<double><<<grid, NA_TJ, 0, s>>>(nr, ntheta, r, e, xc, yc, (const double*)f,
-                                                           (const double*)g, body_ref, mu, dt, Cv, loads, sc);
+                                                           (const double*)g, body_ref, mu, dt, iCv, loads, sc);
     else
         k_wall_loads_noalloc<float><<<grid, NA_TJ, 0, s>>>(nr, ntheta, r, e, xc, yc, (const float*)f,
-                                                          (const float*)g, body_ref, mu, dt, Cv, loads, sc);
+                                                          (const float*)g, body_ref, mu, dt, iCv, loads, sc);
     err = cudaGetLastError();
     if (err != cudaSuccess)
         return lbfsi::set_error(LBFSI_ECUDA, std::string("wall loads launch: ") + cudaGetErrorString(err));
