@@ -149,7 +149,8 @@ struct lbfsi_batch_s {
     Pool pool;
     Workspace work;
     int precision = LBFSI_FP32, variant = 4, order = 0, tile_rows = 16;
-    int shape = 4;   // tile shape launched (the variant)
+    bool own_shape = true;   // no schedule asked for: the shape follows the active solves' sizes
+    int shape = 4;           // tile shape launched (rebuild_tiles)
     size_t esize = 4;
     cudaStream_t stream = nullptr;
     std::vector<MeshEntry> meshes;
@@ -315,6 +316,14 @@ int rebuild_tiles(lbfsi_batch b) {
     cudaError_t e = cudaSuccess;
     auto active = [&](const Slot& s, int part) { return s.used && !s.finished && (s.general ? 1 : 0) == part; };
     b->shape = b->variant;
+    if (b->own_shape && b->precision == LBFSI_FP32) {
+        // as the mesh handle (step_shape): 16 rows if they give every SM two
+        // tiles, else 8
+        long long n = 0;
+        for (const Slot& s : b->slots)
+            if (active(s, 0)) n += (long long)b->meshes[s.mesh].host.ntj * ((b->meshes[s.mesh].host.nr + 15) / 16);
+        b->shape = n >= 304 ? 1 : 0;
+    }
     b->tile_rows = lbfsi::tile_rows(b->precision, b->shape);
     e = update_counts(b);
     if (e != cudaSuccess) return cuda_err(e, "solve record upload");
@@ -499,7 +508,7 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
     b->precision = precision;
     b->esize = precision == LBFSI_FP64 ? sizeof(double) : sizeof(float);
     b->stream = static_cast<cudaStream_t>(cuda_stream);
-    if (precision == LBFSI_FP64) b->variant = 0;   // 8-row tiles
+    if (precision == LBFSI_FP64) b->variant = 0;
     b->shape = b->variant;
     b->tile_rows = lbfsi::tile_rows(precision, b->shape);
     int rc = b->pool.init(pool_bytes);
@@ -783,8 +792,9 @@ int lbfsi_batch_set_schedule(lbfsi_batch b, int variant, int order) {
     if (!b) return lbfsi::set_error(LBFSI_EINVAL, "null batch");
     if (variant < 0 || variant >= lbfsi::step_variants(b->precision) || (order != 0 && order != 1))
         return lbfsi::set_error(LBFSI_EINVAL, "variant or order out of range");
-    if (variant == b->variant && order == b->order) return LBFSI_OK;
+    if (!b->own_shape && variant == b->variant && order == b->order) return LBFSI_OK;
     drop_graph(b);
+    b->own_shape = false;
     b->variant = variant;
     b->order = order;
     b->dirty = true;   // (rebuild_tiles: the tile shape, the per-solve CTA counts, the tables)
