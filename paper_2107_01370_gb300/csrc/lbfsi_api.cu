@@ -82,6 +82,11 @@ struct lbfsi_mesh_s {
     int nbatch = 0, precision = 0, variant = 4, order = 1, tile_rows = 16, tiles_per_solve = 0;
     bool own_shape = true;               // no schedule asked for: the shape follows the size
     int shape = 4;                       // tile shape launched (step_shape)
+    // the step whose correction field (float64: and post-collision populations)
+    // the last call left behind its last step, or -1; not once a field's device
+    // address has been handed out (what is written there between calls counts)
+    long long fields_of = -1;
+    bool handed_out = false;
     int nbody = 1;                       // bodies per solve (independent bodies of a C-grid)
     size_t slots() const { return (size_t)nbatch * (size_t)nbody; }   // body records
     size_t esize = 8;
@@ -95,6 +100,10 @@ struct lbfsi_mesh_s {
     void* d_dep = nullptr;               // general meshes, float64: cached static departures ((xi, eta)
                                          // [9][Nx], then codes [Nx]; see SolveDev::dep_xe)
     double* d_stage = nullptr;  // [nbatch][4][N] float64 staging
+    // pinned copies of the records and the status word for the small reads
+    // between steps (null: could not be had, the reads go to pageable memory)
+    StepMaps* h_maps = nullptr;
+    unsigned* h_status = nullptr;
     StepMaps* d_maps[2] = {nullptr, nullptr};  // [nbatch][nbody] each
     BodyStateDev* d_state_a = nullptr;          // host-given states staging
     BodyStateDev* d_state_b = nullptr;
@@ -139,12 +148,7 @@ cudaError_t dalloc(T** p, size_t count) {
     return cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T));
 }
 
-int check_status(lbfsi_mesh m) {
-    cudaError_t e = cudaStreamSynchronize(m->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "stream synchronize");
-    unsigned st = 0;
-    e = cudaMemcpy(&st, m->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "status read");
+int status_code(unsigned st) {
     if (st & lbfsi::ST_BOUNDS)
         return lbfsi::set_error(LBFSI_EBOUNDS, "an index of the step outside its buffer (bounds-checked build)");
     if (st & lbfsi::ST_TMA)
@@ -155,6 +159,16 @@ int check_status(lbfsi_mesh m) {
         return fail(LBFSI_EDEPARTURE, "wall or outlet target point B outside the cells next to its node");
     if (st & lbfsi::ST_NONPHYS) return fail(LBFSI_ENONPHYS, "non-physical state (rho<=0, T<=0 or NaN)");
     return LBFSI_OK;
+}
+
+// The status word behind the stream's work (and the records, whose copy was
+// enqueued before): one copy into pinned memory, one wait.
+int check_status(lbfsi_mesh m) {
+    unsigned own = 0, *st = m->h_status ? m->h_status : &own;
+    cudaError_t e = cudaMemcpyAsync(st, m->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, m->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "status read");
+    return status_code(*st);
 }
 
 void to_double(const void* src, double* dst, size_t n, int precision) {
@@ -265,9 +279,10 @@ cudaError_t launch_fields(lbfsi_mesh m, const lbfsi::StepArgs& a, int loads, int
 
 // n coupled steps of every solve on stream s, two launches per step: the
 // fields of the current state; then per step the step launch and the field
-// launch behind it (the step's loads and bodies, and the next step's fields;
-// behind the last step the loads alone).  The fields are formed anew from the
-// moments by every call, so that moments written between two calls count.
+// launch behind it (the step's loads and bodies, and the next step's fields).
+// The next call takes the fields over, one launch less, unless what they were
+// formed from was changed in between; with a field's address handed out every
+// call forms them anew and the last launch is the loads alone.
 // rec: device history of the steps' records, or null.
 // host_step < 0: the step numbers come from the device counters.
 cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, cudaStream_t s, int64_t* launches) {
@@ -275,7 +290,9 @@ cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, 
     lbfsi::StepArgs a = make_args(m);
     const bool host = host_step >= 0;
     cudaError_t e = cudaSuccess;
-    if (!host || host_step > 0) {   // (the initial state is streamed without colliding)
+    const bool carry = host && !m->handed_out, have = carry && m->fields_of == host_step;
+    m->fields_of = -1;
+    if (!have && (!host || host_step > 0)) {   // (the initial state is streamed without colliding)
         e = launch_fields(m, a, 0, 1, host ? (int)host_step : -1, nullptr, s);
         ++*launches;
     }
@@ -283,10 +300,11 @@ cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, 
         a.ustep = host ? (int)(host_step + k) : -1;
         e = lbfsi::launch_step_uniform(a, m->precision, m->shape, m->nbatch, s);
         if (e == cudaSuccess)
-            e = launch_fields(m, a, 1, k + 1 < n, host ? (int)(host_step + k + 1) : -1,
+            e = launch_fields(m, a, 1, carry || k + 1 < n, host ? (int)(host_step + k + 1) : -1,
                               rec ? rec + (size_t)k * m->slots() * 7 : nullptr, s);
         *launches += 2;
     }
+    if (carry && e == cudaSuccess) m->fields_of = host_step + n;
     return e;
 }
 
@@ -299,6 +317,7 @@ void free_all(lbfsi_mesh m) {
     if (m->graph) cudaGraphExecDestroy(m->graph);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
     if (m->h_rec) cudaFreeHost(m->h_rec);
+    if (m->h_maps) cudaFreeHost(m->h_maps);
     if (m->d_rec) cudaFree(m->d_rec);
     lbfsi::release_mesh(m->dmesh, m->mem);
 }
@@ -548,6 +567,12 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
 #define LB_ALLOC(ptr, cnt) \
     if (e == cudaSuccess) e = dalloc(&(ptr), (cnt));
     LB_ALLOC(m->d_stage, nb * 4 * N);
+    if (cudaMallocHost((void**)&m->h_maps, ns * sizeof(StepMaps) + sizeof(unsigned)) == cudaSuccess) {
+        m->h_status = reinterpret_cast<unsigned*>(m->h_maps + ns);
+    } else {
+        m->h_maps = nullptr;
+        cudaGetLastError();
+    }
     LB_ALLOC(m->d_maps[0], ns);
     LB_ALLOC(m->d_maps[1], ns);
     LB_ALLOC(m->d_state_a, ns);
@@ -652,6 +677,7 @@ int lbfsi_init_fields(lbfsi_mesh m, const lbfsi_flow_params* p, const double* rh
     if (e == cudaSuccess) e = cudaMemsetAsync(m->d_counter, 0, 4 * nb * sizeof(unsigned), m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "init_fields upload");
     m->host_k = 0;
+    m->fields_of = -1;
     rc = upload_solves(m);
     if (rc) return rc;
     e = lbfsi::launch_init(m->precision, m->d_stage, m->d_p[0], m->d_M[0], m->host.Nx, m->nbatch,
@@ -687,6 +713,7 @@ int lbfsi_blend_mesh(lbfsi_mesh m, const lbfsi_body_state* state, const lbfsi_bo
     const size_t nb = m->slots();
     static_assert(sizeof(lbfsi_body_state) == sizeof(BodyStateDev), "layout");
     const lbfsi_body_state* pv = prev ? prev : state;
+    m->fields_of = -1;
     cudaError_t e = cudaMemcpyAsync(m->d_state_a, state, nb * sizeof(BodyStateDev), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->d_state_b, pv, nb * sizeof(BodyStateDev), cudaMemcpyHostToDevice, m->stream);
@@ -712,6 +739,7 @@ int lbfsi_step(lbfsi_mesh m, int nsteps) {
             const int rc = capture_graph(m);
             if (rc) return rc;
         }
+        m->fields_of = -1;
         for (; nsteps - s >= m->graph_steps; s += m->graph_steps) {
             const cudaError_t e = cudaGraphLaunch(m->graph, m->stream);
             if (e != cudaSuccess) return cuda_fail(e, "graph launch");
@@ -730,6 +758,7 @@ int lbfsi_field_ptr(lbfsi_mesh m, int which, void** ptr, int64_t* slots, int64_t
     if (which != LBFSI_FIELD_MOMENTS && which != LBFSI_FIELD_POPULATIONS)
         return fail(LBFSI_EINVAL, "which must be LBFSI_FIELD_MOMENTS or LBFSI_FIELD_POPULATIONS");
     if (!m->initialized) return fail(LBFSI_ESTATE, "init_fields first");
+    m->handed_out = true;
     *ptr = which == LBFSI_FIELD_MOMENTS ? m->d_M[m->cur()] : m->d_p[m->cur()];
     if (slots) *slots = (int64_t)m->host.Nx;
     if (row0) *row0 = (int64_t)m->host.G * m->host.nt;
@@ -743,10 +772,13 @@ int lbfsi_synchronize(lbfsi_mesh m) {
 
 static int download_maps(lbfsi_mesh m, std::vector<StepMaps>& out) {
     out.resize(m->slots());
-    cudaError_t e = cudaMemcpyAsync(out.data(), m->d_maps[m->cur()], out.size() * sizeof(StepMaps),
+    StepMaps* to = m->h_maps ? m->h_maps : out.data();
+    cudaError_t e = cudaMemcpyAsync(to, m->d_maps[m->cur()], out.size() * sizeof(StepMaps),
                                     cudaMemcpyDeviceToHost, m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "maps copy");
-    return check_status(m);
+    const int rc = check_status(m);
+    if (!rc && m->h_maps) std::memcpy(out.data(), m->h_maps, out.size() * sizeof(StepMaps));
+    return rc;
 }
 
 int lbfsi_step_record(lbfsi_mesh m, int nsteps, double* loads_out, lbfsi_body_state* states_out) {
@@ -820,6 +852,7 @@ int lbfsi_advance_bodies(lbfsi_mesh m, const double* loads, double dt) {
         for (size_t b = 0; b < nb; ++b)
             for (int c = 0; c < 3; ++c) ld[b * 3 + c] = mp[b].loads[c];
     }
+    m->fields_of = -1;
     cudaError_t e = cudaMemcpyAsync(m->d_loads_tmp, ld.data(), ld.size() * sizeof(double), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
         e = lbfsi::launch_advance(m->d_bodies, m->d_loads_tmp, dt, (long long)m->host_k, (int)nb,
@@ -847,15 +880,20 @@ int lbfsi_get_body_state(lbfsi_mesh m, lbfsi_body_state* out) {
 int lbfsi_get_fields(lbfsi_mesh m, double* rho_u_T) {
     if (!m || !rho_u_T) return fail(LBFSI_EINVAL, "null argument");
     if (!m->initialized) return fail(LBFSI_ESTATE, "init_fields first");
-    int rc;
-    if (m->host.G) {
-        std::vector<double> all((size_t)m->nbatch * 4 * m->host.Nx);
-        rc = download(m, m->d_M[m->cur()], all.data(), all.size());
-        if (!rc) compact_rows(m->host, all.data(), rho_u_T, (size_t)m->nbatch * 4, 1);
+    // rows 0 .. nr-1 of each component (Nx slots apart) straight into the
+    // caller's array, float values widened on the device first
+    const size_t N = (size_t)m->host.N, Nx = (size_t)m->host.Nx, rows = (size_t)m->nbatch * 4, w = sizeof(double);
+    const char* src = (const char*)m->d_M[m->cur()] + (size_t)m->host.G * m->host.nt * m->esize;
+    cudaError_t e;
+    if (m->precision == LBFSI_FP64) {
+        e = cudaMemcpy2DAsync(rho_u_T, N * w, src, Nx * w, N * w, rows, cudaMemcpyDeviceToHost, m->stream);
     } else {
-        rc = download(m, m->d_M[m->cur()], rho_u_T, (size_t)m->nbatch * 4 * m->host.N);
+        e = lbfsi::launch_read(m->precision, src, Nx, nullptr, m->d_stage, (int)N, rows, m->stream);
+        m->launches++;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(rho_u_T, m->d_stage, rows * N * w, cudaMemcpyDeviceToHost, m->stream);
     }
-    if (rc) return rc;
+    if (e != cudaSuccess) return cuda_fail(e, "fields download");
     return check_status(m);
 }
 
@@ -905,6 +943,7 @@ int lbfsi_set_populations(lbfsi_mesh m, const double* f, const double* g, const 
     if (!m->initialized) return fail(LBFSI_ESTATE, "init_fields first");
     const size_t cnt = (size_t)m->nbatch * 9 * m->host.N;
     const int c = m->cur();
+    m->fields_of = -1;
     std::vector<double> pairs(2 * cnt);
     for (size_t k = 0; k < cnt; ++k) {
         pairs[2 * k] = f[k];
@@ -1001,6 +1040,7 @@ int lbfsi_restore(lbfsi_mesh m, const void* buf, size_t bytes) {
         h.esize != (int32_t)m->esize || (h.nbody > 1 ? (int)h.nbody : 1) != m->nbody)
         return fail(LBFSI_EINVAL, "checkpoint of a different mesh, batch or precision");
     drop_graph(m);
+    m->fields_of = -1;
     m->host_k = h.step;
     const size_t N = (size_t)m->host.Nx, nb = (size_t)m->nbatch;
     const char* p = static_cast<const char*>(buf) + sizeof(h);

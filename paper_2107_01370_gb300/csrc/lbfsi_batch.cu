@@ -149,6 +149,14 @@ struct lbfsi_batch_s {
     Pool pool;
     Workspace work;
     int precision = LBFSI_FP32, variant = 4, order = 0, tile_rows = 16;
+    // reading a solve back: float64 staging of the largest read so far, and
+    // pinned copies of its record and the status word (null: could not be had)
+    double* d_read = nullptr;
+    size_t read_count = 0;
+    struct Small {
+        StepMaps maps;
+        unsigned status;
+    }* h_get = nullptr;
     bool own_shape = true;   // no schedule asked for: the shape follows the active solves' sizes
     int shape = 4;           // tile shape launched (rebuild_tiles)
     size_t esize = 4;
@@ -406,12 +414,13 @@ int rebuild_tiles(lbfsi_batch b) {
     return LBFSI_OK;
 }
 
+// (one copy behind the stream's work, one wait)
 int check_status(lbfsi_batch b) {
-    cudaError_t e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return cuda_err(e, "stream synchronize");
-    unsigned st = 0;
-    e = cudaMemcpy(&st, b->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost);
+    unsigned own = 0, *hs = b->h_get ? &b->h_get->status : &own;
+    cudaError_t e = cudaMemcpyAsync(hs, b->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return cuda_err(e, "status read");
+    const unsigned st = *hs;
     if (st & lbfsi::ST_BOUNDS)
         return lbfsi::set_error(LBFSI_EBOUNDS, "an index of the step outside its buffer (bounds-checked build)");
     if (st & (lbfsi::ST_DEPARTURE | lbfsi::ST_BPOINT))
@@ -530,6 +539,10 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
         lbfsi_batch_destroy(b);
         return lbfsi::set_error(LBFSI_ENOMEM, std::string("batch allocation: ") + cudaGetErrorString(e));
     }
+    if (cudaMallocHost((void**)&b->h_get, sizeof(*b->h_get)) != cudaSuccess) {
+        b->h_get = nullptr;
+        cudaGetLastError();
+    }
     *out = b;
     return LBFSI_OK;
 }
@@ -537,8 +550,9 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
 int lbfsi_batch_destroy(lbfsi_batch b) {
     if (!b) return lbfsi::set_error(LBFSI_EINVAL, "null batch");
     cudaStreamSynchronize(b->stream);
+    if (b->h_get) cudaFreeHost(b->h_get);
     void* ptrs[] = {b->d_meshes, b->d_solves, b->d_tiles, b->d_ftiles, b->d_status, b->d_zero_state,
-                    b->d_zero_loads, b->d_tmaps};
+                    b->d_zero_loads, b->d_tmaps, b->d_read};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (b->graph) cudaGraphExecDestroy(b->graph);
@@ -886,24 +900,38 @@ int lbfsi_batch_get(lbfsi_batch b, int slot, double* rho_u_T, double* loads, lbf
     const size_t N = (size_t)b->meshes[s.mesh].host.N, Nx = (size_t)b->meshes[s.mesh].host.Nx;
     cudaError_t e = cudaSuccess;
     std::vector<unsigned char> raw;
-    if (rho_u_T) {
-        // rows 0 .. nr-1 of the four components (Nx slots apart)
-        raw.resize(4 * N * b->esize);
-        e = cudaMemcpy2DAsync(raw.data(), N * b->esize, s.dev.M[cur], Nx * b->esize, N * b->esize, 4,
-                              cudaMemcpyDeviceToHost, b->stream);
-    }
-    StepMaps mp{};
-    if (e == cudaSuccess && (loads || state))
-        e = cudaMemcpyAsync(&mp, s.dev.maps[cur], sizeof(StepMaps), cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return cuda_err(e, "batch results copy");
-    if (rho_u_T) {
-        if (b->precision == LBFSI_FP64) {
-            std::memcpy(rho_u_T, raw.data(), raw.size());
+    if (rho_u_T && b->precision == LBFSI_FP32 && b->read_count < 4 * N) {
+        // float64 staging of the largest solve read so far
+        if (b->d_read) cudaFree(b->d_read);   // (waits for its last copy)
+        b->read_count = 0;
+        if (cudaMalloc(&b->d_read, 4 * N * sizeof(double)) == cudaSuccess) {
+            b->read_count = 4 * N;
         } else {
-            const float* f = reinterpret_cast<const float*>(raw.data());
-            for (size_t n = 0; n < 4 * N; ++n) rho_u_T[n] = (double)f[n];
+            b->d_read = nullptr;   // no room: widened on the host
+            cudaGetLastError();
         }
+    }
+    // rows 0 .. nr-1 of the four components (Nx slots apart) straight into the
+    // caller's array, float values widened on the device first
+    const bool direct = rho_u_T && (b->precision == LBFSI_FP64 || b->d_read);
+    if (rho_u_T && b->precision == LBFSI_FP32 && b->d_read) {
+        e = lbfsi::launch_read(b->precision, s.dev.M[cur], Nx, nullptr, b->d_read, (int)N, 4, b->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(rho_u_T, b->d_read, 4 * N * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+    } else if (rho_u_T) {
+        if (!direct) raw.resize(4 * N * b->esize);
+        e = cudaMemcpy2DAsync(direct ? (void*)rho_u_T : raw.data(), N * b->esize, s.dev.M[cur], Nx * b->esize,
+                              N * b->esize, 4, cudaMemcpyDeviceToHost, b->stream);
+    }
+    StepMaps own{}, *rec = b->h_get ? &b->h_get->maps : &own;
+    if (e == cudaSuccess && (loads || state))
+        e = cudaMemcpyAsync(rec, s.dev.maps[cur], sizeof(StepMaps), cudaMemcpyDeviceToHost, b->stream);
+    if (e != cudaSuccess) return cuda_err(e, "batch results copy");
+    const int rc = check_status(b);
+    const StepMaps& mp = *rec;
+    if (rho_u_T && !direct) {
+        const float* f = reinterpret_cast<const float*>(raw.data());
+        for (size_t n = 0; n < 4 * N; ++n) rho_u_T[n] = (double)f[n];
     }
     if (loads)
         for (int c = 0; c < 3; ++c) loads[c] = mp.loads[c];
@@ -913,7 +941,7 @@ int lbfsi_batch_get(lbfsi_batch b, int slot, double* rho_u_T, double* loads, lbf
         state->hdot = mp.S_next.hdot;
         state->adot = mp.S_next.adot;
     }
-    return check_status(b);
+    return rc;
 }
 
 int lbfsi_batch_remove(lbfsi_batch b, int slot) {

@@ -1,6 +1,7 @@
 // Internal declarations shared by the kernels and the C-ABI layer.
 #pragma once
 
+#include <utility>
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -288,6 +289,10 @@ cudaError_t launch_init(int precision, const double* M, void* P, void* Mout, int
                         double Cv, cudaStream_t s);
 // Build the maps record from explicit states: S_cur (collision), S_next and
 // S_vgprev (stream); loads copied from 'loads' if non-null.
+// rows x N values of the path's type, rows stride apart, as float64 [rows][N] in
+// the order given (null: as they lie)
+cudaError_t launch_read(int precision, const void* src, size_t stride, const int* order, double* dst, int N, size_t rows,
+                        cudaStream_t s);
 cudaError_t launch_prepare(const BodyDev* bodies, const BodyStateDev* S_cur,
                            const BodyStateDev* S_next, const BodyStateDev* S_vgprev,
                            const double* loads, double dt, int nbatch, StepMaps* maps,
