@@ -69,6 +69,14 @@ struct Macro {
     R rho, ux, uy, T, E;
 };
 
+// The end of the kernel before in the stream, with its writes visible (nothing
+// of a kernel launched by launch_behind may read or write global memory
+// before); then the kernel behind may start (and wait in turn).
+__device__ __forceinline__ void wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // rho = sum f, rho u = sum f c, 2 rho E = sum g, T = (E - u^2/2) / Cv.
 template <typename R>
 __device__ __forceinline__ Macro<R> moments(const R* f, const R* g, R iCv) {

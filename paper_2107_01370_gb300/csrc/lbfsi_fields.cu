@@ -22,18 +22,10 @@
 // the step launch.
 #include <algorithm>
 
+#include "lbfsi_record.cuh"
 #include "lbfsi_stencil.cuh"
 
 namespace lbfsi {
-
-constexpr unsigned FULL = 0xffffffffu;
-
-// Sum over the warp's lanes (the same tree for every caller).
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    return v;
-}
 
 // (double)x of a normal float in integer instructions: a conversion runs at
 // the float64 rate, and a wall node has 18.
@@ -120,38 +112,9 @@ __device__ __forceinline__ void wall_loads(const FieldArgs& a, const SolveDev& S
     // the bodies' steps, four lanes per body: lane r of a group state entry
     // r.  What they need besides the loads is read before the count below, so
     // that the solve's last block does not wait for it in turn
-    const int bo = min(l >> 2, nb - 1), r = l & 3;
+    const int bo = min(l >> 2, nb - 1);
     const size_t sbo = (size_t)sb * nb + bo;
-    const BodyDev& bd = S.body[sbo];
-    const BodyStateDev Sn = prev[bo].S_next;
-    const BodyMap<double> ms = prev[bo].Sd;
-    const double t1 = (double)kk * S.dt;
-    const bool forced = bd.dof == 2 && t1 <= bd.t_forced;
-    double pr[6], sv[4] = {Sn.h, Sn.alpha, Sn.hdot, Sn.adot};
-    {
-        const double* p = forced ? S.prop[sbo].forced[r >> 1] : S.prop[sbo].free[r];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) pr[c] = p[c];
-    }
-    double y = 0.0;   // the part of the step that does not depend on the loads
-    if (forced) {
-        // forced pitching (Sec. IV D): alpha = amp sin(w t) prescribed, its
-        // acceleration at the step's start, middle and end
-        const double ww = bd.w_a, amp = bd.pitch_amp;
-        const double ang = ww * (r == 0 ? t1 - S.dt : r == 1 ? ((double)kk - 0.5) * S.dt : t1);
-        const double sn = amp * (r == 3 ? cos(ang) : sin(ang));
-        const unsigned grp = __activemask();
-        const int g4 = l & ~3;
-        const double a0 = __shfl_sync(grp, sn, g4), ah = __shfl_sync(grp, sn, g4 + 1), a1 = __shfl_sync(grp, sn, g4 + 2);
-        const double c1 = __shfl_sync(grp, sn, g4 + 3);
-        if (r == 1) y = a1;
-        else if (r == 3) y = ww * c1;
-        else y = fm(-ww * ww, fm(pr[3], a0, fm(pr[4], ah, pr[5] * a1)), fm(pr[0], sv[0], pr[1] * sv[2]));
-        pr[4] = (r & 1) ? 0.0 : pr[2];
-        pr[5] = 0.0;
-    } else {
-        y = fm(pr[0], sv[0], pr[1] * sv[1]) + fm(pr[2], sv[2], pr[3] * sv[3]);
-    }
+    const BodyLane bl = body_lane(S.body[sbo], S.prop[sbo], prev[bo], S.dt, kk, l);
     // the acquire-release count publishes this block's partials and makes
     // every other block's visible to the solve's last
     if (nblk > 1) {
@@ -173,51 +136,7 @@ __device__ __forceinline__ void wall_loads(const FieldArgs& a, const SolveDev& S
             if (b == bo) F[c] = t;
         }
     }
-    y = fm(pr[4], F[1], fm(pr[5], F[2], y));
-    const int g4 = bo * 4;
-    const double h = __shfl_sync(FULL, y, g4), al = __shfl_sync(FULL, y, g4 + 1);
-    const double hd = __shfl_sync(FULL, y, g4 + 2), ad = __shfl_sync(FULL, y, g4 + 3);
-    // sin(alpha) and cos(alpha) - 1 = -2 sin^2(alpha / 2) (body_rot)
-    double sn = (r & 1) ? al : 0.5 * al;
-    if (al != 0.0) sn = sin(sn);
-    const double hs = __shfl_sync(FULL, sn, g4), sa = __shfl_sync(FULL, sn, g4 + 1), cm = -2.0 * hs * hs;
-    for (int b = 0; b < nb; ++b) {
-        // the record (build_maps): the collision map is the streamed map at
-        // rest, the stream map the new state's with the rates from the last
-        if (l == 4 * b) {
-            s_rec.S_cur = s_rec.S_vgprev = Sn;
-            s_rec.S_next = BodyStateDev{h, al, hd, ad};
-            for (int c = 0; c < 3; ++c) s_rec.loads[c] = F[c];
-            BodyMap<double> m = ms;
-            m.va00 = m.va01 = m.va10 = m.va11 = m.vtx = m.vty = 0.0;
-            s_rec.Kd = m;
-            m.va00 = m.va11 = (cm - ms.a00) * S.idt;
-            m.va10 = (sa - ms.a10) * S.idt;
-            m.va01 = -m.va10;
-            m.vty = (h - Sn.h) * S.idt;
-            m.a00 = m.a11 = cm;
-            m.a01 = -sa;
-            m.a10 = sa;
-            m.ty = h;
-            s_rec.Sd = m;
-        }
-        __syncwarp();
-        // their float copies, an entry per lane
-        constexpr int ND = (int)((sizeof(BodyMap<double>) - offsetof(BodyMap<double>, xc)) / 8);
-        for (int t = l; t < 2 * ND; t += 32) {
-            const BodyMap<double>& d = t < ND ? s_rec.Sd : s_rec.Kd;
-            BodyMap<float>& f = t < ND ? s_rec.Sf : s_rec.Kf;
-            const int c = t < ND ? t : t - ND;
-            (&f.xc)[c] = (float)(&d.xc)[c];
-            if (c == 0) f.active = d.active;
-        }
-        __syncwarp();
-        const size_t sbb = (size_t)sb * nb + b;
-        unsigned* out = reinterpret_cast<unsigned*>(S.maps[cur] + sbb);
-        for (int t = l; t < (int)(sizeof(StepMaps) / 4); t += 32) out[t] = reinterpret_cast<const unsigned*>(&s_rec)[t];
-        if (a.rec && l < 7) a.rec[sbb * 7 + l] = l < 3 ? s_rec.loads[l] : (&s_rec.S_next.h)[l - 3];
-        __syncwarp();
-    }
+    body_records(bl, F, S.idt, nb, l, s_rec, S.maps[cur] + (size_t)sb * nb, a.rec ? a.rec + (size_t)sb * nb * 7 : nullptr);
     if (l == 0) {
         ctr[1] = kk;
         ctr[2] = 0u;
@@ -599,6 +518,7 @@ __device__ __forceinline__ void fields_tile(const FieldArgs& a, const SolveDev& 
 template <typename R, bool GEN, int TI, bool UNIFORM>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 32 * MARCH_WARPS : 64 * TI, sizeof(R) == 4 ? 5 : 4)
     k_fields(const __grid_constant__ FieldArgs a) {
+    wait_previous();
     __shared__ BodyMap<R> smap[GEN ? MAX_BODIES : 1];
     int sb = 0, blk = (int)blockIdx.x;
     bool loads;
@@ -681,8 +601,8 @@ __global__ void k_post(const SolveDev S, const MeshDev G, int cur, int nbatch) {
 template <typename R, bool GEN, bool UNIFORM>
 static cudaError_t launch_t(const FieldArgs& a, unsigned blocks, cudaStream_t s) {
     constexpr int TI = sizeof(R) == 4 ? 0 : FIELD_ROWS_FP64;
-    k_fields<R, GEN, TI, UNIFORM><<<blocks, sizeof(R) == 4 ? 32 * MARCH_WARPS : 64 * FIELD_ROWS_FP64, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_behind(k_fields<R, GEN, TI, UNIFORM>, blocks, sizeof(R) == 4 ? 32 * MARCH_WARPS : 64 * FIELD_ROWS_FP64, 0,
+                         s, sizeof(R) == 4 || blocks <= OVERLAP_BLOCKS_FP64, a);
 }
 
 template <bool UNIFORM>

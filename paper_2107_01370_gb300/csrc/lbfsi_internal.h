@@ -289,6 +289,35 @@ cudaError_t launch_init(int precision, const double* M, void* P, void* Mout, int
                         double Cv, cudaStream_t s);
 // Build the maps record from explicit states: S_cur (collision), S_next and
 // S_vgprev (stream); loads copied from 'loads' if non-null.
+// The kernels of a step are launched while the one before still runs
+// (programmatic stream serialization) and wait for its end and its writes
+// themselves, first thing (wait_previous): a launch's start -- some 2 to 3 us
+// behind the end of the last, a tenth to a quarter of a small mesh's step --
+// then overlaps the previous kernel's last wave.  Float: every launch (measured
+// per step: 256 x 128 one solve 25.1 -> 22.1 us, 201 x 150 x 5 32.4 -> 29.2,
+// ellipse 512 x 256 x 8 132 -> 127).  Float64: launches of few blocks only, which
+// find SMs of their own (24 x 32: 91.5 -> 87.9 us); more of them are packed
+// beside the running kernel's on some SMs, whose float64 rate then bounds the
+// step while others idle (128 x 64: 46.5 -> 54.7 us, a 97 x 161 C-grid 106 -> 120).
+constexpr unsigned OVERLAP_BLOCKS_FP64 = 76;   // half the SMs
+template <typename... P, typename... A>
+cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap,
+                          A&&... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = overlap ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 // rows x N values of the path's type, rows stride apart, as float64 [rows][N] in
 // the order given (null: as they lie)
 cudaError_t launch_read(int precision, const void* src, size_t stride, const int* order, double* dst, int N, size_t rows,

@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
     // tile nodes streamed per thread
     constexpr int NPT = (TI * TJ + NT - 1) / NT;
     constexpr bool RAGGED = NPT * NT != TI * TJ;
+    wait_previous();
     extern __shared__ __align__(128) unsigned char smraw[];
     R2* sp = reinterpret_cast<R2*>(smraw);                        // [9][PH][PWS] (f_q, g_q) pairs
     R* sY = reinterpret_cast<R*>(sp + 9 * T::PSS);                // [2][PH][PWS] Y_x, Y_y
@@ -915,8 +916,7 @@ struct StepKernel {
         const dim3 grid = !UNIFORM   ? dim3(a.ntiles)
                           : a.uorder ? dim3(nbatch, a.umesh.ntj, nti)
                                      : dim3(a.umesh.ntj, nti, nbatch);
-        k_step<TI, TJ, NT, MINB, UNIFORM, GEN><<<grid, NT, step_smem_bytes<TI, TJ, GEN>(), s>>>(a);
-        return cudaGetLastError();
+        return launch_behind(k_step<TI, TJ, NT, MINB, UNIFORM, GEN>, grid, NT, step_smem_bytes<TI, TJ, GEN>(), s, true, a);
     }
 };
 

@@ -28,6 +28,7 @@ constexpr int S64_WARPS = 4, S64_THREADS = 32 * S64_WARPS;
 template <bool GEN, bool UNIFORM>
 __global__ void __launch_bounds__(S64_THREADS, 4) k_stream64(const __grid_constant__ StepArgs a, int nbatch, int rows) {
     constexpr int TJ = TILE_J;
+    wait_previous();
     __shared__ BodyMap<double> mapS[GEN ? MAX_BODIES : 1];
     __shared__ double s_sum[4][S64_WARPS][TJ];   // rho, rho u_x, rho u_y, 2 rho E of each warp's directions
     __shared__ double s_far[4][TJ];
@@ -354,10 +355,9 @@ __global__ void __launch_bounds__(S64_THREADS, 4) k_stream64(const __grid_consta
 cudaError_t launch_stream64(const StepArgs& a, bool uniform, bool general, int rows, int nbatch, cudaStream_t s) {
     const int nti = (a.umesh.nr + rows - 1) / rows;
     const unsigned grid = uniform ? (unsigned)nbatch * a.umesh.ntj * nti : (unsigned)a.ntiles;
-    auto go = [&](auto kernel) { kernel<<<grid, S64_THREADS, 0, s>>>(a, nbatch, rows); };
-    if (uniform) general ? go(k_stream64<true, true>) : go(k_stream64<false, true>);
-    else general ? go(k_stream64<true, false>) : go(k_stream64<false, false>);
-    return cudaGetLastError();
+    auto go = [&](auto kernel) { return launch_behind(kernel, grid, S64_THREADS, 0, s, grid <= OVERLAP_BLOCKS_FP64, a, nbatch, rows); };
+    if (uniform) return general ? go(k_stream64<true, true>) : go(k_stream64<false, true>);
+    return general ? go(k_stream64<true, false>) : go(k_stream64<false, false>);
 }
 
 }  // namespace lbfsi
