@@ -230,10 +230,8 @@ typedef struct {
 int lbfsi_create_mesh_cgrid_walls(const lbfsi_mesh_cgrid_walls_desc* d, void* cuda_stream, lbfsi_mesh* out);
 
 /* Create a mesh handle on a C-grid; otherwise as lbfsi_create_mesh_xy (one
- * tile shape).  A step is two launches here: the collision of step k of the
- * 16 rows next to the cut into a post-collision buffer, then one launch in
- * which the tiles next to the cut stream step k + 1 from it and the others
- * collide and stream.
+ * tile shape): the tiles next to the cut stage the mirrored rows of its other
+ * side.
  * LBFSI_EINVAL for an even ntheta, a bad n_cut, cut nodes that do not
  * coincide, or a mesh that is not subparametric or not positively oriented. */
 int lbfsi_create_mesh_cgrid(const lbfsi_mesh_cgrid_desc* d, void* cuda_stream, lbfsi_mesh* out);
@@ -391,7 +389,7 @@ int lbfsi_wall_loads_noalloc(int nr, int ntheta, int nbatch, int precision, cons
                              double* loads, void* cuda_stream);
 
 /* ---- Batch runtime: many solves on meshes of different sizes, admitted and
- * retired while others run, advanced together (one launch per step for all
+ * retired while others run, advanced together (two launches per step for all
  * active solves).  Device memory comes from one pool allocated at creation;
  * a solve is admitted only if the pool can hold it (continuous batching with
  * memory-based admission).  Solves on identical O-grids share one device copy
@@ -441,8 +439,8 @@ typedef struct {
 
 /* Admit a solve on a general O-grid (same contract as lbfsi_batch_add).
  * Identical coordinate sets share one device copy.  These solves run on the
- * general-geometry kernel with its one tile shape, in a second launch of
- * every lbfsi_batch_step; lbfsi_batch_set_schedule and the autotuner change
+ * general-geometry kernel with its one tile shape, in launches of their own
+ * in every lbfsi_batch_step; lbfsi_batch_set_schedule and the autotuner change
  * the tiles of the separable-mesh solves only. */
 int lbfsi_batch_add_xy(lbfsi_batch b, const lbfsi_solve_xy_desc* d, int* slot);
 
@@ -460,13 +458,11 @@ typedef struct {
 } lbfsi_solve_cgrid_desc;
 
 /* Admit a solve on a C-grid (same contract as lbfsi_batch_add).  Its tiles
- * form a third part of every lbfsi_batch_step: the collision of the rows next
- * to the cut, then the launch that streams the tiles next to the cut from its
- * output and collides and streams the others. */
+ * join the general-mesh part of every lbfsi_batch_step. */
 int lbfsi_batch_add_cgrid(lbfsi_batch b, const lbfsi_solve_cgrid_desc* d, int* slot);
 
-/* Advance every active solve by up to nsteps coupled steps (one launch per
- * step covering all active solves; a solve stops when it reaches its step
+/* Advance every active solve by up to nsteps coupled steps (two launches
+ * per step covering all active solves of a mesh kind; a solve stops when it reaches its step
  * count).  *active_after (nullable) receives the number of unfinished solves.
  * Asynchronous except when the set of active solves changes. */
 int lbfsi_batch_step(lbfsi_batch b, int nsteps, int* active_after);
@@ -517,17 +513,18 @@ int64_t lbfsi_launch_count(lbfsi_mesh m);
 
 /* Number of tile shapes ("step variants") of the step kernel for a
  * precision (LBFSI_FP32: 5, LBFSI_FP64: 3), or LBFSI_EINVAL.  Float shapes,
- * radial x angular nodes per CTA: 0: 8 x 32, 256 threads, 2 CTAs/SM;
- * 1: 16 x 32, 256 threads; 2: 8 x 32, 3 CTAs/SM; 3: 12 x 32, 384 threads;
- * 4: 16 x 32, 512 threads (default of new mesh handles, with order 1, and of
- * new batches, with order 0).  Float64 shapes (separable O-grids; 256
- * threads, one CTA per SM): 0: 8 x 32 (default), 1: 4 x 32, 2: 2 x 32 -- the
- * smaller tiles spread a small mesh over more SMs, whose float64 rate bounds
- * the step.  Meshes given by node coordinates have one shape (0).
- * Staging (every shape): in a float mesh handle whose Ntheta is a multiple
- * of 4, and for the float solves of a batch on separable O-grids whose Ntheta
- * is a multiple of 4, the moments and populations of each tile whose angular
- * range does not wrap are moved into shared memory by two tensor copies
+ * radial x angular nodes per CTA: 0: 8 x 32, 256 threads, 3 CTAs/SM;
+ * 1: 16 x 32, 256 threads, 3 CTAs/SM; 2: 12 x 32, 192 threads, 4 CTAs/SM;
+ * 3: 12 x 32, 384 threads; 4: 16 x 32, 512 threads (what lbfsi_get_schedule
+ * reports for new mesh handles, with order 1, and new batches, with order 0;
+ * until a schedule is set they launch shape 1 where 16 rows give at least 304
+ * tiles and shape 0 elsewhere).  Float64 shapes (128 threads per row of 32
+ * nodes): 0: one row per CTA (default), 1: two, 2: four.  Meshes given by node
+ * coordinates have one shape (0).
+ * Staging (every float shape): in a float mesh handle whose Ntheta is a
+ * multiple of 4, and for the float solves of a batch on separable O-grids
+ * whose Ntheta is a multiple of 4, the populations and the correction field of
+ * each tile whose angular range does not wrap are moved into shared memory by two tensor copies
  * (TMA), the other tiles by per-thread copies; LBFSI_TMA=0 in the environment
  * when a handle first steps (when a batch rebuilds its tile table) stages
  * every tile by per-thread copies.  Both give the same bits. */
@@ -540,8 +537,8 @@ int lbfsi_step_variants(int precision);
 int lbfsi_set_schedule(lbfsi_mesh m, int variant, int order);
 int lbfsi_get_schedule(lbfsi_mesh m, int* variant, int* order);
 
-/* graph_steps > 0: lbfsi_step replays a CUDA graph of graph_steps step
- * launches (captured at first use on a private stream, recaptured after a
+/* graph_steps > 0: lbfsi_step replays a CUDA graph of the launches of
+ * graph_steps steps (captured at first use on a private stream, recaptured after a
  * schedule change; its launches read the step number from the device),
  * plain launches for the remainder; 0 (default): plain launches only. */
 int lbfsi_set_graph_steps(lbfsi_mesh m, int graph_steps);
@@ -560,8 +557,8 @@ int lbfsi_autotune(lbfsi_mesh m, int steps_per_trial, int* best_variant, int* be
  * cases this way).  A separate handle: the step on an element list runs as
  * four launches per step over node lists (correction field D, collision into
  * a post-collision buffer, stream, load reduction and body update) with the
- * Q2 gathers read from global memory, instead of the structured meshes'
- * one-launch tiled kernel.
+ * Q2 gathers of a block of nodes read from the populations of its elements in
+ * shared memory, instead of the structured meshes' tiled kernels.
  *
  * Mesh: N nodes, elements of 3 x 3 node indices [a][b] (entry (a, b) at
  * reference coordinates (a - 1, b - 1)), subparametric (each element's mid

@@ -30,7 +30,8 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
 
 # the step kernels' instantiations (tile shapes, launch forms) have to round
 # alike: no contraction but the fused operations written out in their sources
-SOURCE_FLAGS = {s: ["-fmad=false"] for s in ("lbfsi_step.cu", "lbfsi_fields.cu", "lbfsi_stream64.cu")}
+SOURCE_FLAGS = {s: ["-fmad=false"] for s in ("lbfsi_step.cu", "lbfsi_fields.cu", "lbfsi_stream64.cu",
+                                              "lbfsi_elements.cu")}
 
 
 def nvcc() -> str:

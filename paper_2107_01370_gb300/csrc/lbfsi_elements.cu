@@ -39,6 +39,8 @@
 #include "lbfsi_device.cuh"
 #include "lbfsi_host.h"
 #include "lbfsi_internal.h"
+#include "lbfsi_record.cuh"
+#include "lbfsi_stencil.cuh"
 
 namespace lbfsi {
 namespace {
@@ -51,13 +53,27 @@ constexpr int EN_STRIDE = 12;
 struct EArgs {
     int N, nbatch, nblk, kstep, collide;
     const void* X;        // [N][2] node coordinates (element type of the path)
-    const int* E;         // [Ne][EN_STRIDE] element nodes, entry a * 3 + b (then padding, so
+    // a block's nodes lie in a few elements: the tables of each block's own
+    // copy of them, block blk's elements eptr[blk] .. eptr[blk + 1)
+    const int* eptr;      // [nblk + 1]
+    const int* E;         // [.][EN_STRIDE] element nodes, entry a * 3 + b (then padding, so
                           // that a gather reads an element's nodes in three 16-byte loads)
-    const void* ecoef;    // [Ne][6] bilinear map: (b_x, b_y, c_x, c_y, d_x, d_y)
+    const void* ecoef;    // [.][8] bilinear map: (b_x, b_y, c_x, c_y, d_x, d_y, 0, 0)
     const int* hptr;      // [N + 1] holding elements of each node
-    const int* hold;      // [.] element * 16 + the node's entry in it
-    const int* gptr;      // [N + 1] gradient operator rows
-    const int* gcol;      // [.] neighbour node
+    const int* hold;      // [.] (block's) element * 16 + 4 a + b, (a, b) the node's entry in it
+    // staged gathers (k_em_stream): the nodes of block blk's elements
+    // nlist[nptr[blk] .. nptr[blk + 1]), in increasing order, and the elements'
+    // nodes as byte offsets of pairs into that list; rows of snode pairs
+    const int* nptr;
+    const int* nlist;
+    const unsigned short* lnode;   // [.][EN_STRIDE]
+    int snode;
+    // gradient operator in slices of 32 nodes (a warp's): slice s holds
+    // gptr[s + 1] - gptr[s] entries per node, entry k of lane l at gptr[s] * 32 +
+    // 32 k + l, rows shorter than their slice padded by zero weights on the node
+    // itself -- so that a warp's reads of an entry are consecutive
+    const int* gptr;      // [slices + 1] entries per lane before the slice
+    const int* gcol;      // neighbour node
     const void* gw;       // [.][2] weights of d/dX and d/dY
     const int* kind;      // [N]
     const double* xw;     // [nwall][2] wall node coordinates
@@ -66,9 +82,9 @@ struct EArgs {
     const double* nfar;   // [nfar][2] outward directions of the far field
     // departures of the interior nodes for a node the blend does not move
     // (the displacement of direction q is then -dt c_q at every step),
-    // solved once for the flow's dt: the position in hold of the holding
-    // element [9][N] (-1: none holds the point) and (xi, eta) [9][N]; null:
-    // solved every step
+    // solved once for the flow's dt: the entry of hold of the holding element
+    // [9][N] (-1: none holds the point) and (xi, eta) [9][N]; null: solved
+    // every step
     int* dep_e;
     void* dep_xe;
     const void* p_in;     // [nbatch][9][N] pairs: pre-collision state of step k
@@ -76,13 +92,20 @@ struct EArgs {
     void* p_out;          // [nbatch][9][N] pairs: pre-collision state of step k + 1
     const void* M_in;     // [nbatch][4][N] moments of step k
     void* M_out;          // [nbatch][4][N] moments of step k + 1
-    void* D;              // [nbatch][2][N]
-    void* dQ;             // [nbatch][2][N] dQ of the moments the stream writes (the next
+    void* D;              // [nbatch][N] pairs
+    void* dQ;             // [nbatch][N] pairs: dQ of the moments the stream writes (the next
                           // step's correction field reads it at every neighbour)
     const StepMaps* maps_in;   // [nbatch]
     StepMaps* maps_out;        // [nbatch]
     const BodyDev* bodies;     // [nbatch]
-    double* part;         // [nbatch][nblk][3]
+    const BodyProp* prop;      // [nbatch]
+    // the order the stream takes the blocks in: those with wall nodes, then those
+    // with nodes a blend may move (their departures are solved), then the rest,
+    // so that the long blocks do not come last
+    const int* border;    // [nblk]
+    const int* wblk;      // [nblk] a block's slot among those with wall nodes, or -1
+    int nwblk;
+    double* part;         // [nbatch][nwblk][3] load partials
     SolveDev flow;        // flow parameters (buffers unused)
     unsigned* status;
 };
@@ -133,32 +156,44 @@ __device__ __forceinline__ bool inv_map(const BodyMap<R>& bm, R X, R Y, R& i00, 
 
 // Newton's method for the point (dx, dy) relative to a node at reference
 // position (xi0, eta0) of an element with bilinear map X0 + b xi + c eta +
-// d xi eta, c = (b_x, b_y, c_x, c_y, d_x, d_y): (b + d eta0) u + (c + d xi0) v
-// + d u v = (dx, dy).  Returns the point's reference coordinates.  Written
+// d xi eta, ce = (b_x, b_y, c_x, c_y, d_x, d_y): (b + d eta0) u + (c + d xi0) v
+// + d u v = (dx, dy).  Gives the point's reference coordinates; false where the
+// first iterate already shows that the element does not hold it: with (p, q)
+// the solution of the linear part for d, the iterate is u (1 + p v), and
+// 1 + p v, the ratio of the map's determinants at the node and at (xi0, eta0 +
+// v), is positive in an element, so u and its iterate have one sign.  Written
 // with fixed rounding (fma_rn, mul_rn, add_rn) so that the departures cached
 // by k_em_record equal, bit for bit, the ones k_em_stream solves.
 template <typename R>
-__device__ __forceinline__ void em_newton(const R* c, R xi0, R et0, R dx, R dy, R& x, R& y) {
-    const R Bx = fma_rn(c[4], et0, c[0]), By = fma_rn(c[5], et0, c[1]);
-    const R Cx = fma_rn(c[4], xi0, c[2]), Cy = fma_rn(c[5], xi0, c[3]);
-    R u = R(0), v = R(0);
+__device__ __forceinline__ bool em_newton(const R* __restrict__ ce, R xi0, R et0, R dx, R dy, R& x, R& y) {
+    using V = typename EVec<R>::T2;
+    const V* cv = reinterpret_cast<const V*>(ce);
+    const V cb = __ldg(cv), cc = __ldg(cv + 1), cd = __ldg(cv + 2);
+    const R Bx = fma_rn(cd.x, et0, cb.x), By = fma_rn(cd.y, et0, cb.y);
+    const R Cx = fma_rn(cd.x, xi0, cc.x), Cy = fma_rn(cd.y, xi0, cc.y);
+    R idet = rcp_(fma_rn(Bx, Cy, -mul_rn(Cx, By)));
+    R u = mul_rn(fma_rn(Cy, dx, -mul_rn(Cx, dy)), idet);
+    R v = mul_rn(fma_rn(Bx, dy, -mul_rn(By, dx)), idet);
+    if (mul_rn(xi0, u) > R(1e-3) || mul_rn(et0, v) > R(1e-3)) return false;
     constexpr int ITS = sizeof(R) == 4 ? 4 : 20;
 #pragma unroll 1
-    for (int it = 0; it < ITS; ++it) {
+    for (int it = 1; it < ITS; ++it) {
         const R uv = mul_rn(u, v);
-        const R rx = fma_rn(c[4], uv, fma_rn(Cx, v, fma_rn(Bx, u, -dx)));
-        const R ry = fma_rn(c[5], uv, fma_rn(Cy, v, fma_rn(By, u, -dy)));
-        const R a11 = fma_rn(c[4], v, Bx), a12 = fma_rn(c[4], u, Cx);
-        const R a21 = fma_rn(c[5], v, By), a22 = fma_rn(c[5], u, Cy);
-        const R idet = rcp_(fma_rn(a11, a22, -mul_rn(a12, a21)));
+        const R rx = fma_rn(cd.x, uv, fma_rn(Cx, v, fma_rn(Bx, u, -dx)));
+        const R ry = fma_rn(cd.y, uv, fma_rn(Cy, v, fma_rn(By, u, -dy)));
+        const R a11 = fma_rn(cd.x, v, Bx), a12 = fma_rn(cd.x, u, Cx);
+        const R a21 = fma_rn(cd.y, v, By), a22 = fma_rn(cd.y, u, Cy);
+        idet = rcp_(fma_rn(a11, a22, -mul_rn(a12, a21)));
         const R du = mul_rn(fma_rn(a22, rx, -mul_rn(a12, ry)), idet);
         const R dv = mul_rn(fma_rn(a11, ry, -mul_rn(a21, rx)), idet);
         u = add_rn(u, -du);
         v = add_rn(v, -dv);
-        if (sizeof(R) == 8 && abs_(du) + abs_(dv) < R(1e-15)) break;
+        // (the next correction is of the order of this one's square)
+        if (abs_(du) + abs_(dv) < (sizeof(R) == 8 ? R(1e-15) : R(1e-4))) break;
     }
     x = add_rn(xi0, u);
     y = add_rn(et0, v);
+    return true;
 }
 
 // Containment tolerance of pass 0 / 1 (reading R8): 1e-12 of the element
@@ -174,60 +209,65 @@ __host__ __device__ constexpr int em_passes() {
 
 // Departure point of node n displaced by (dx, dy): the first element holding
 // the node (increasing index) that contains it (Eq. depPnt; readings R8, R9).
+// guess: the entry of hold of the element to try first, or -1: a point well
+// inside an element is in no other, so that the order does not matter.
 template <typename R>
-__device__ bool em_locate(const EArgs& a, int n, R dx, R dy, int& elem, R& xi, R& eta) {
+__device__ __forceinline__ bool em_locate(const EArgs& a, int n, R dx, R dy, int& code, R& xi, R& eta, int guess = -1) {
     const R* ec = static_cast<const R*>(a.ecoef);
-    const int h0 = a.hptr[n], h1 = a.hptr[n + 1];
+    const int h0 = __ldg(a.hptr + n), h1 = __ldg(a.hptr + n + 1);
+    // one copy of the solve for the first try and the search
+    int pass = guess >= 0 ? -1 : 0, h = h0;
 #pragma unroll 1
-    for (int pass = 0; pass < em_passes<R>(); ++pass) {
-        const R tin = em_tol<R>(pass);
-#pragma unroll 1
-        for (int h = h0; h < h1; ++h) {
-            const int code = __ldg(a.hold + h), e = code >> 4, ent = code & 15;
-            R x, y;
-            em_newton<R>(ec + 6 * (size_t)e, R(ent / 3 - 1), R(ent % 3 - 1), dx, dy, x, y);
-            if (abs_(x) <= tin && abs_(y) <= tin) {
-                elem = e;
-                xi = x;
-                eta = y;
-                return true;
-            }
+    while (true) {
+        code = pass < 0 ? guess : __ldg(a.hold + h);
+        const R tin = pass < 0 ? R(0.99) : em_tol<R>(pass);
+        if (em_newton<R>(ec + 8 * (size_t)(code >> 4), R(((code >> 2) & 3) - 1), R((code & 3) - 1), dx, dy, xi, eta) &&
+            abs_(xi) <= tin && abs_(eta) <= tin)
+            return true;
+        if (pass < 0 || ++h == h1) {
+            h = h0;
+            if (++pass == em_passes<R>()) return false;
         }
     }
-    return false;
 }
 
-// The nodal gradient operator applied to two fields in one pass over the
-// operator's row: fld(m, v0, v1) gives both at node m.  Each field's sums
-// run in the same order as in em_grad.
+// The nodal gradient operator of node n applied to a field given by a functor.
 template <typename R, typename Fn>
-__device__ __forceinline__ void em_grad2(const EArgs& a, int n, Fn fld, R& g0X, R& g0Y, R& g1X, R& g1Y) {
-    const R* w = static_cast<const R*>(a.gw);
-    g0X = R(0);
-    g0Y = R(0);
-    g1X = R(0);
-    g1Y = R(0);
-    for (int k = a.gptr[n]; k < a.gptr[n + 1]; ++k) {
-        R v0, v1;
-        fld(a.gcol[k], v0, v1);
-        const R wX = w[2 * k], wY = w[2 * k + 1];
-        g0X += wX * v0;
-        g0Y += wY * v0;
-        g1X += wX * v1;
-        g1Y += wY * v1;
+__device__ __forceinline__ void em_grad(const EArgs& a, int n, Fn fld, R& gX, R& gY) {
+    using R2 = typename EVec<R>::T2;
+    const int s = n >> 5, l = n & 31, p0 = __ldg(a.gptr + s), len = __ldg(a.gptr + s + 1) - p0;
+    const int* col = a.gcol + 32 * (size_t)p0 + l;
+    const R2* w = static_cast<const R2*>(a.gw) + 32 * (size_t)p0 + l;
+    gX = R(0);
+    gY = R(0);
+    for (int k = 0; k < len; ++k) {
+        const R v = fld(__ldg(col + 32 * k));
+        const R2 wk = __ldg(w + 32 * k);
+        gX = fm(wk.x, v, gX);
+        gY = fm(wk.y, v, gY);
     }
 }
 
-// The nodal gradient operator applied to a field given by a functor.
-template <typename R, typename Fn>
-__device__ __forceinline__ void em_grad(const EArgs& a, int n, Fn fld, R& gX, R& gY) {
-    const R* w = static_cast<const R*>(a.gw);
-    gX = R(0);
-    gY = R(0);
-    for (int k = a.gptr[n]; k < a.gptr[n + 1]; ++k) {
-        const R v = fld(a.gcol[k]);
-        gX += w[2 * k] * v;
-        gY += w[2 * k + 1] * v;
+// The same on both components of a field of pairs for NS solves at once (one
+// read of the operator): gx_[s] = d/dX of (v.x, v.y), gy_[s] = d/dY; fld(m, s)
+// gives the pair of solve s at node m.
+template <typename R, int NS, typename Fn>
+__device__ __forceinline__ void em_grad2(const EArgs& a, int n, Fn fld, typename EVec<R>::T2* gx_, typename EVec<R>::T2* gy_) {
+    using R2 = typename EVec<R>::T2;
+    const int s = n >> 5, l = n & 31, p0 = __ldg(a.gptr + s), len = __ldg(a.gptr + s + 1) - p0;
+    const int* col = a.gcol + 32 * (size_t)p0 + l;
+    const R2* w = static_cast<const R2*>(a.gw) + 32 * (size_t)p0 + l;
+#pragma unroll
+    for (int b = 0; b < NS; ++b) gx_[b] = gy_[b] = pair(R(0), R(0));
+    for (int k = 0; k < len; ++k) {
+        const int m = __ldg(col + 32 * k);
+        const R2 wk = __ldg(w + 32 * k);
+#pragma unroll
+        for (int b = 0; b < NS; ++b) {
+            const R2 v = fld(m, b);
+            gx_[b] = pfma(pair(wk.x, wk.x), v, gx_[b]);
+            gy_[b] = pfma(pair(wk.y, wk.y), v, gy_[b]);
+        }
     }
 }
 
@@ -244,76 +284,91 @@ __device__ __forceinline__ typename EVec<R>::T2 ref_pair(const SolveDev& s, int 
     return r;
 }
 
+// Solves per thread: the mesh's tables (operator, departures, element nodes)
+// are read once for all of them.  (float64 is bound by its arithmetic, which
+// the solves do not share.)
+template <typename R>
+__host__ __device__ constexpr int em_solves() {
+    return sizeof(R) == 4 ? 2 : 1;
+}
+
 // ---- launch 1: D = (mu/p) grad dQ (Sec. II C), dQ_a = rho u_a (1 - 3T) - rho u_a^3
 // (dQ written with the moments by the previous stream launch, em_dq)
-template <typename R>
+template <typename R, int NS>
 __global__ void __launch_bounds__(EM_THREADS) k_em_D(const EArgs a) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+    wait_previous();
+    using R2 = typename EVec<R>::T2;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, b0 = blockIdx.y * NS;
     if (n >= a.N) return;
     const size_t N = (size_t)a.N;
-    const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
-    const R* X = static_cast<const R*>(a.X);
-    R i00, i01, i10, i11, vx, vy;
-    inv_map(kmap<R>(a.maps_in[b]), X[2 * n], X[2 * n + 1], i00, i01, i10, i11, vx, vy);
-    const R* Q = static_cast<const R*>(a.dQ) + (size_t)b * 2 * N;
-    R xX, xY, yX, yY;
-    em_grad2<R>(a, n, [&](int m, R& v0, R& v1) {
-        v0 = Q[m];
-        v1 = Q[N + m];
-    }, xX, xY, yX, yY);
-    const R mup = flowv<R>(a.flow, a.flow.mu, a.flow.mu_f) * rcp_(M[n] * M[3 * N + n]);
-    R* D = static_cast<R*>(a.D) + (size_t)b * 2 * N;
-    D[n] = mup * (i00 * xX + i10 * xY);
-    D[N + n] = mup * (i01 * yX + i11 * yY);
+    const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
+    const R2* Q = static_cast<const R2*>(a.dQ);
+    R2 gx[NS], gy[NS];
+    em_grad2<R, NS>(a, n, [&](int m, int s) { return Q[(size_t)min(b0 + s, a.nbatch - 1) * N + m]; }, gx, gy);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const int b = b0 + s;
+        if (b >= a.nbatch) break;
+        const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
+        R i00, i01, i10, i11, vx, vy;
+        inv_map(kmap<R>(a.maps_in[b]), x.x, x.y, i00, i01, i10, i11, vx, vy);
+        const R mup = flowv<R>(a.flow, a.flow.mu, a.flow.mu_f) * rcp_(M[n] * M[3 * N + n]);
+        static_cast<R2*>(a.D)[(size_t)b * N + n] = pair(mup * fm(i00, gx[s].x, i10 * gy[s].x), mup * fm(i01, gx[s].y, i11 * gy[s].y));
+    }
 }
 
 // dQ_a = rho u_a (1 - 3T) - rho u_a^3 of a node's moments (Sec. II C).
 template <typename R>
-__device__ __forceinline__ void em_dq(R* Q, size_t N, int n, R rho, R ux, R uy, R T) {
-    Q[n] = rho * ux * (R(1) - R(3) * T) - rho * ux * ux * ux;
-    Q[N + n] = rho * uy * (R(1) - R(3) * T) - rho * uy * uy * uy;
+__device__ __forceinline__ typename EVec<R>::T2 em_dq(R rho, R ux, R uy, R T) {
+    const R t = fm(R(-3), T, R(1));
+    return pair(rho * ux * fm(-ux, ux, t), rho * uy * fm(-uy, uy, t));
 }
 
 // ---- launch 2: Y = grad D and the collision (Eq. f_boltz) into ppost;
 // step 0 only copies the initial state
-template <typename R>
+template <typename R, int NS>
 __global__ void __launch_bounds__(EM_THREADS) k_em_collide(const EArgs a) {
+    wait_previous();
     using R2 = typename EVec<R>::T2;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, b0 = blockIdx.y * NS;
     if (n >= a.N) return;
     const size_t N = (size_t)a.N;
-    const R2* pin = static_cast<const R2*>(a.p_in) + (size_t)b * 9 * N;
-    R2* pout = static_cast<R2*>(a.ppost) + (size_t)b * 9 * N;
-    R2 pq[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) pq[q] = pin[q * N + n];
-    if (a.collide) {
-        const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
-        const R Cv = flowv<R>(a.flow, a.flow.Cv, a.flow.Cv_f);
-        if (a.kind[n] < 0) {
-            R f[9], g[9];
-            f_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], f);
-            g_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], Cv, g);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) pq[q] = pair(f[q], g[q]);
-        } else {
-            const R* X = static_cast<const R*>(a.X);
-            R i00, i01, i10, i11, vx, vy;
-            inv_map(kmap<R>(a.maps_in[b]), X[2 * n], X[2 * n + 1], i00, i01, i10, i11, vx, vy);
-            const R* D = static_cast<const R*>(a.D) + (size_t)b * 2 * N;
-            R xX, xY, yX, yY;
-            em_grad2<R>(a, n, [&](int m, R& v0, R& v1) {
-                v0 = D[m];
-                v1 = D[N + m];
-            }, xX, xY, yX, yY);
-            const R Yx = i00 * xX + i10 * xY, Yy = i01 * yX + i11 * yY;
-            collide_pairs(pq, Yx, Yy, flowv<R>(a.flow, a.flow.mu, a.flow.mu_f),
-                          flowv<R>(a.flow, a.flow.muP, a.flow.muP_f), flowv<R>(a.flow, a.flow.dt, a.flow.dt_f),
-                          flowv<R>(a.flow, a.flow.iCv, a.flow.iCv_f));
-        }
+    const bool far = a.kind[n] < 0;
+    const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
+    R2 gx[NS], gy[NS];
+    if (a.collide && !far) {
+        const R2* D = static_cast<const R2*>(a.D);
+        em_grad2<R, NS>(a, n, [&](int m, int s) { return D[(size_t)min(b0 + s, a.nbatch - 1) * N + m]; }, gx, gy);
     }
 #pragma unroll
-    for (int q = 0; q < 9; ++q) pout[q * N + n] = psub(pq[q], ref_pair<R>(a.flow, q));
+    for (int s = 0; s < NS; ++s) {
+        const int b = b0 + s;
+        if (b >= a.nbatch) break;
+        const R2* pin = static_cast<const R2*>(a.p_in) + (size_t)b * 9 * N;
+        R2* pout = static_cast<R2*>(a.ppost) + (size_t)b * 9 * N;
+        R2 pq[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) pq[q] = pin[q * N + n];
+        if (a.collide) {
+            if (far) {
+                const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
+                R f[9], g[9];
+                f_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], f);
+                g_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], flowv<R>(a.flow, a.flow.Cv, a.flow.Cv_f), g);
+#pragma unroll
+                for (int q = 0; q < 9; ++q) pq[q] = pair(f[q], g[q]);
+            } else {
+                R i00, i01, i10, i11, vx, vy;
+                inv_map(kmap<R>(a.maps_in[b]), x.x, x.y, i00, i01, i10, i11, vx, vy);
+                const R Yx = fm(i00, gx[s].x, i10 * gy[s].x), Yy = fm(i01, gx[s].y, i11 * gy[s].y);
+                collide_pairs(pq, Yx, Yy, flowv<R>(a.flow, a.flow.mu, a.flow.mu_f),
+                              flowv<R>(a.flow, a.flow.muP, a.flow.muP_f), flowv<R>(a.flow, a.flow.dt, a.flow.dt_f),
+                              flowv<R>(a.flow, a.flow.iCv, a.flow.iCv_f));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 9; ++q) pout[q * N + n] = psub(pq[q], ref_pair<R>(a.flow, q));
+    }
 }
 
 // Q2 interpolation of direction q's post-collision pairs over element e.
@@ -322,12 +377,12 @@ __device__ __forceinline__ typename EVec<R>::T2 em_gather(const EArgs& a, const 
                                                           R xi, R eta) {
     using R2 = typename EVec<R>::T2;
     R Lx[3], Ly[3];
-    Lx[0] = xi * (R(0.5) * xi - R(0.5));
-    Lx[1] = R(1) - xi * xi;
-    Lx[2] = xi * (R(0.5) * xi + R(0.5));
-    Ly[0] = eta * (R(0.5) * eta - R(0.5));
-    Ly[1] = R(1) - eta * eta;
-    Ly[2] = eta * (R(0.5) * eta + R(0.5));
+    Lx[0] = xi * fm(R(0.5), xi, R(-0.5));
+    Lx[1] = fm(-xi, xi, R(1));
+    Lx[2] = xi * fm(R(0.5), xi, R(0.5));
+    Ly[0] = eta * fm(R(0.5), eta, R(-0.5));
+    Ly[1] = fm(-eta, eta, R(1));
+    Ly[2] = eta * fm(R(0.5), eta, R(0.5));
     const int4* e4 = reinterpret_cast<const int4*>(a.E + EN_STRIDE * (size_t)e);
     const int4 n0 = __ldg(e4), n1 = __ldg(e4 + 1), n2 = __ldg(e4 + 2);
     const int nd[9] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w, n2.x};
@@ -342,6 +397,32 @@ __device__ __forceinline__ typename EVec<R>::T2 em_gather(const EArgs& a, const 
     return acc;
 }
 
+// The same from the block's staged populations: row is direction q's, nd the
+// element's nodes as byte offsets into it.
+__device__ __forceinline__ float2 em_gather_staged(const unsigned char* row, const unsigned short* nd, float xi, float eta) {
+    float Lx[3], Ly[3];
+    Lx[0] = xi * fm(0.5f, xi, -0.5f);
+    Lx[1] = fm(-xi, xi, 1.0f);
+    Lx[2] = xi * fm(0.5f, xi, 0.5f);
+    Ly[0] = eta * fm(0.5f, eta, -0.5f);
+    Ly[1] = fm(-eta, eta, 1.0f);
+    Ly[2] = eta * fm(0.5f, eta, 0.5f);
+    const uint2* w = reinterpret_cast<const uint2*>(nd);
+    const uint2 w0 = w[0], w1 = w[1], w2 = w[2];
+    const unsigned o[9] = {w0.x & 0xffffu, w0.x >> 16, w0.y & 0xffffu, w0.y >> 16, w1.x & 0xffffu,
+                           w1.x >> 16,     w1.y & 0xffffu, w1.y >> 16, w2.x & 0xffffu};
+    auto at = [&](int k) { return *reinterpret_cast<const float2*>(row + o[k]); };
+    float2 acc = pair(0.0f, 0.0f);
+#pragma unroll
+    for (int aa = 0; aa < 3; ++aa) {
+        float2 t = pmul(pair(Ly[0], Ly[0]), at(3 * aa));
+        t = pfma(pair(Ly[1], Ly[1]), at(3 * aa + 1), t);
+        t = pfma(pair(Ly[2], Ly[2]), at(3 * aa + 2), t);
+        acc = pfma(pair(Lx[aa], Lx[aa]), t, acc);
+    }
+    return acc;
+}
+
 // Moments rho, u, T at a point of element e: the node's own values plus the
 // Q2-weighted differences from them (the weights' round-off then acts on
 // small differences).
@@ -349,12 +430,12 @@ template <typename R>
 __device__ __forceinline__ void em_interp_M(const EArgs& a, const R* M, size_t N, int n, int e, R xi, R eta,
                                             R* out) {
     R Lx[3], Ly[3];
-    Lx[0] = xi * (R(0.5) * xi - R(0.5));
-    Lx[1] = R(1) - xi * xi;
-    Lx[2] = xi * (R(0.5) * xi + R(0.5));
-    Ly[0] = eta * (R(0.5) * eta - R(0.5));
-    Ly[1] = R(1) - eta * eta;
-    Ly[2] = eta * (R(0.5) * eta + R(0.5));
+    Lx[0] = xi * fm(R(0.5), xi, R(-0.5));
+    Lx[1] = fm(-xi, xi, R(1));
+    Lx[2] = xi * fm(R(0.5), xi, R(0.5));
+    Ly[0] = eta * fm(R(0.5), eta, R(-0.5));
+    Ly[1] = fm(-eta, eta, R(1));
+    Ly[2] = eta * fm(R(0.5), eta, R(0.5));
     const int* en = a.E + EN_STRIDE * (size_t)e;
     R d[4] = {R(0), R(0), R(0), R(0)};
     R own[4];
@@ -365,43 +446,74 @@ __device__ __forceinline__ void em_interp_M(const EArgs& a, const R* M, size_t N
         const R w = Lx[s / 3] * Ly[s % 3];
         const int m = en[s];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) d[c] += w * (M[c * N + m] - own[c]);
+        for (int c = 0; c < 4; ++c) d[c] = fm(w, M[c * N + m] - own[c], d[c]);
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c) out[c] = own[c] + d[c];
 }
 
-// ---- launch 3: stream step k + 1.  Bound by the latency of its dependent
-// loads: the float kernel is held to 40 registers so that six blocks (48
-// warps) share an SM (measured: 64 registers and four blocks 2506 MLUPS,
-// 48 and five 2635, 40 and six 2700)
-template <typename R>
-__global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_stream(const EArgs a) {
+// ---- launch 3: stream step k + 1.  The float kernel is bound by the gathers'
+// loads and their instructions: a block first stages the populations of all
+// the nodes its own nodes' elements have (nlist: measured 1.8 times its 256
+// nodes on a stretched ring) and those elements' node offsets into shared
+// memory, and the 81 gathers of a node read there.  STAGED = false reads
+// global memory instead: lists whose numbering scatters so much that a
+// block's nodes would not fit (EM_STAGE_MAX), and float64, bound by its
+// arithmetic.
+constexpr size_t EM_STAGE_MAX = 75 * 1024;   // three blocks per SM
+__host__ __device__ constexpr size_t em_stage_bytes(int snode, int selem) {
+    const size_t a = 9 * (size_t)snode * sizeof(float2) + (size_t)selem * EN_STRIDE * sizeof(unsigned short);
+    return a > 3 * EM_THREADS * sizeof(double) ? a : 3 * EM_THREADS * sizeof(double);
+}
+
+template <typename R, bool STAGED>
+__global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_stream(const EArgs a) {
+    wait_previous();
     using R2 = typename EVec<R>::T2;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+    extern __shared__ __align__(16) unsigned char smem[];
+    // (a block of all solves side by side: they share its tables in L2)
+    const int blk = __ldg(a.border + blockIdx.x / a.nbatch), b = blockIdx.x % a.nbatch;
+    const int n = blk * EM_THREADS + threadIdx.x;
     const size_t N = (size_t)a.N;
+    const R2* pp = static_cast<const R2*>(a.ppost) + (size_t)b * 9 * N;
+    const int e0 = __ldg(a.eptr + blk);
+    [[maybe_unused]] const unsigned short* ln = nullptr;
+    if constexpr (STAGED) {
+        const int l0 = __ldg(a.nptr + blk), nn = __ldg(a.nptr + blk + 1) - l0;
+        for (int i = threadIdx.x; i < nn; i += EM_THREADS) {
+            const int m = __ldg(a.nlist + l0 + i);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) cp_async8(smem + 8 * ((size_t)q * a.snode + i), pp + q * N + m);
+        }
+        unsigned char* lb = smem + 72 * (size_t)a.snode;
+        const int ne = __ldg(a.eptr + blk + 1) - e0;
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(a.lnode + (size_t)EN_STRIDE * e0);
+        for (int i = threadIdx.x; i < 3 * ne; i += EM_THREADS) cp_async8(lb + 8 * i, src + 8 * i);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        ln = reinterpret_cast<const unsigned short*>(lb);
+    }
     double fcx = 0.0, fcy = 0.0, fcm = 0.0;
     bool wallnode = false;
     if (n < a.N) {
         const SolveDev& fl = a.flow;
         const R dt = flowv<R>(fl, fl.dt, fl.dt_f), Cv = flowv<R>(fl, fl.Cv, fl.Cv_f);
         const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
-        const R2* pp = static_cast<const R2*>(a.ppost) + (size_t)b * 9 * N;
         R2* po = static_cast<R2*>(a.p_out) + (size_t)b * 9 * N;
         R* Mo = static_cast<R*>(a.M_out) + (size_t)b * 4 * N;
-        R* Qo = static_cast<R*>(a.dQ) + (size_t)b * 2 * N;
-        const R* X = static_cast<const R*>(a.X);
-        const int kd = a.kind[n];
+        R2* Qo = static_cast<R2*>(a.dQ) + (size_t)b * N;
+        const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
+        const int kd = __ldg(a.kind + n);
         wallnode = kd > 0;
         if (kd < 0) {
             // far field: targets at B = A - dt n_out; the inlet prescribes the
             // free stream's u and T (reading R20)
             const double* nf = a.nfar + 2 * (size_t)(-kd - 1);
             R t[4];
-            int e;
+            int code;
             R xi, eta;
-            if (em_locate<R>(a, n, -dt * (R)nf[0], -dt * (R)nf[1], e, xi, eta)) {
-                em_interp_M<R>(a, M, N, n, e, xi, eta, t);
+            if (em_locate<R>(a, n, -dt * (R)nf[0], -dt * (R)nf[1], code, xi, eta)) {
+                em_interp_M<R>(a, M, N, n, code >> 4, xi, eta, t);
             } else {
                 atomicOr(a.status, ST_BPOINT);
                 for (int c = 0; c < 4; ++c) t[c] = M[c * N + n];
@@ -418,15 +530,15 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
             for (int q = 0; q < 9; ++q) po[q * N + n] = pair(f[q], g[q]);
 #pragma unroll
             for (int c = 0; c < 4; ++c) Mo[c * N + n] = t[c];
-            em_dq<R>(Qo, N, n, t[0], t[1], t[2], t[3]);
+            Qo[n] = em_dq<R>(t[0], t[1], t[2], t[3]);
         } else {
             const StepMaps& mp = a.maps_in[b];
             R i00, i01, i10, i11, vx, vy;
-            const bool moved = inv_map(smap<R>(mp), X[2 * n], X[2 * n + 1], i00, i01, i10, i11, vx, vy);
+            const bool moved = inv_map(smap<R>(mp), x.x, x.y, i00, i01, i10, i11, vx, vy);
             // an interior node the blend does not move takes its cached
-            // departures (the same solves, made once for the flow's dt)
-            const bool cached = a.dep_e != nullptr && kd == 0 && !moved;
-            const R2* dxe = static_cast<const R2*>(a.dep_xe);
+            // departures (the same solves, made once for the flow's dt); one
+            // that it moves tries their elements first
+            const bool dep = a.dep_e != nullptr && kd == 0;
             unsigned missing = 0u;
             const int w = kd - 1;
             if (kd > 0) {
@@ -443,37 +555,43 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
                     if (hx * n0x + hy * n0y > 1e-12) missing |= 1u << q;
                 }
             }
-            R f[9], g[9];
+            // moments summed as the populations come (no array of them: one
+            // copy of the solve for the nine directions)
+            R rho = R(0), jx = R(0), jy = R(0), s2 = R(0);
+            auto put = [&](int q, R cx, R cy, R2 v) {
+                po[q * N + n] = v;
+                rho += v.x;
+                jx = fm(cx, v.x, jx);
+                jy = fm(cy, v.x, jy);
+                s2 += v.y;
+            };
             bool lost = false;
 #pragma unroll 1
             for (int q = 0; q < 9; ++q) {
-                f[q] = R(0);
-                g[q] = R(0);
                 if (missing & (1u << q)) continue;
                 const R cx = (R)cxq(q), cy = (R)cyq(q);
-                const R hx = i00 * cx + i01 * cy - vx, hy = i10 * cx + i11 * cy - vy;
-                int e;
+                int code = dep ? __ldg(a.dep_e + (size_t)q * N + n) : -1;
                 R xi, eta;
-                R2 v;
                 bool found;
-                if (cached) {
-                    e = __ldg(a.dep_e + (size_t)q * N + n);
-                    found = e >= 0;
-                    const R2 xe = __ldg(dxe + (size_t)q * N + n);
+                if (dep && !moved) {
+                    const R2 xe = __ldg(static_cast<const R2*>(a.dep_xe) + (size_t)q * N + n);
                     xi = xe.x;
                     eta = xe.y;
+                    found = code >= 0;
                 } else {
-                    found = em_locate<R>(a, n, -dt * hx, -dt * hy, e, xi, eta);
+                    const R hx = fm(i00, cx, fm(i01, cy, -vx)), hy = fm(i10, cx, fm(i11, cy, -vy));
+                    found = em_locate<R>(a, n, -dt * hx, -dt * hy, code, xi, eta, code);
                 }
+                R2 v;
+                if (found) found = in_bounds((code >> 4) >= e0 && (code >> 4) < __ldg(a.eptr + blk + 1), a.status);
                 if (found) {
-                    v = em_gather<R>(a, pp + (size_t)q * N, e, xi, eta);
+                    if constexpr (STAGED) v = em_gather_staged(smem + 8 * (size_t)q * a.snode, ln + EN_STRIDE * ((code >> 4) - e0), xi, eta);
+                    else v = em_gather<R>(a, pp + (size_t)q * N, code >> 4, xi, eta);
                 } else {
                     lost = true;
                     v = pp[q * N + n];
                 }
-                v = padd(v, ref_pair<R>(fl, q));
-                f[q] = v.x;
-                g[q] = v.y;
+                put(q, cx, cy, padd(v, ref_pair<R>(fl, q)));
             }
             if (lost) atomicOr(a.status, ST_DEPARTURE);
             if (missing) {
@@ -481,51 +599,44 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
                 // wall velocity, gradients at the node; Grad's approximation
                 // of the missing populations (Sec. III A)
                 R t[4];
-                int e;
+                int code;
                 R xi, eta;
-                if (em_locate<R>(a, n, dt * (R)a.n0[2 * w], dt * (R)a.n0[2 * w + 1], e, xi, eta)) {
-                    em_interp_M<R>(a, M, N, n, e, xi, eta, t);
+                if (em_locate<R>(a, n, dt * (R)a.n0[2 * w], dt * (R)a.n0[2 * w + 1], code, xi, eta)) {
+                    em_interp_M<R>(a, M, N, n, code >> 4, xi, eta, t);
                 } else {
                     atomicOr(a.status, ST_BPOINT);
                     for (int c = 0; c < 4; ++c) t[c] = M[c * N + n];
                 }
-                R gr[3][2];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    R gX, gY;
-                    em_grad<R>(a, n, [&](int m) { return M[(1 + c) * N + m]; }, gX, gY);
-                    gr[c][0] = i00 * gX + i10 * gY;
-                    gr[c][1] = i01 * gX + i11 * gY;
-                }
+                R2 gX, gY;
+                R gTX, gTY;
+                em_grad2<R, 1>(a, n, [&](int m, int) { return pair(M[N + m], M[2 * N + m]); }, &gX, &gY);
+                em_grad<R>(a, n, [&](int m) { return M[3 * N + m]; }, gTX, gTY);
                 R fw[9], gw[9];
-                grad_populations(t[0], vx, vy, t[3], gr[0][0], gr[0][1], gr[1][0], gr[1][1], gr[2][0], gr[2][1],
-                                 flowv<R>(fl, fl.mu, fl.mu_f), dt, Cv, flowv<R>(fl, fl.iCv, fl.iCv_f),
-                                 flowv<R>(fl, fl.iPr, fl.iPr_f), fw, gw);
+                grad_populations(t[0], vx, vy, t[3], fm(i00, gX.x, i10 * gY.x), fm(i01, gX.x, i11 * gY.x),
+                                 fm(i00, gX.y, i10 * gY.y), fm(i01, gX.y, i11 * gY.y), fm(i00, gTX, i10 * gTY),
+                                 fm(i01, gTX, i11 * gTY), flowv<R>(fl, fl.mu, fl.mu_f), dt, Cv,
+                                 flowv<R>(fl, fl.iCv, fl.iCv_f), flowv<R>(fl, fl.iPr, fl.iPr_f), fw, gw);
 #pragma unroll
                 for (int q = 0; q < 9; ++q)
-                    if (missing & (1u << q)) {
-                        f[q] = fw[q];
-                        g[q] = gw[q];
-                    }
+                    if (missing & (1u << q)) put(q, (R)cxq(q), (R)cyq(q), pair(fw[q], gw[q]));
             }
-            const Macro<R> mc = moments(f, g, flowv<R>(fl, fl.iCv, fl.iCv_f));
-            if (!(mc.rho > R(0)) || !(mc.T > R(0)) || !isfinite(mc.ux) || !isfinite(mc.uy))
-                atomicOr(a.status, ST_NONPHYS);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) po[q * N + n] = pair(f[q], g[q]);
-            Mo[n] = mc.rho;
-            Mo[N + n] = mc.ux;
-            Mo[2 * N + n] = mc.uy;
-            Mo[3 * N + n] = mc.T;
-            em_dq<R>(Qo, N, n, mc.rho, mc.ux, mc.uy, mc.T);
+            const R ir = rcp_(rho), ux = jx * ir, uy = jy * ir;
+            const R T = fm(R(-0.5), fm(ux, ux, uy * uy), R(0.5) * s2 * ir) * flowv<R>(fl, fl.iCv, fl.iCv_f);
+            if (!(rho > R(0)) || !(T > R(0)) || !isfinite(ux) || !isfinite(uy)) atomicOr(a.status, ST_NONPHYS);
+            Mo[n] = rho;
+            Mo[N + n] = ux;
+            Mo[2 * N + n] = uy;
+            Mo[3 * N + n] = T;
+            Qo[n] = em_dq<R>(rho, ux, uy, T);
             if (kd > 0) {
                 // wall stress sigma = -p I - (1 - omega/2) sum (f - f^eq) c c
                 // (Sec. III) in float64, this node's Simpson shares
                 double fd[9], gd[9], feq[9];
 #pragma unroll
                 for (int q = 0; q < 9; ++q) {
-                    fd[q] = (double)f[q];
-                    gd[q] = (double)g[q];
+                    const R2 v = po[q * N + n];   // (this thread's own writes)
+                    fd[q] = (double)v.x;
+                    gd[q] = (double)v.y;
                 }
                 const Macro<double> md = moments(fd, gd, fl.iCv);
                 f_equilibrium(md.rho, md.ux, md.uy, md.T, feq);
@@ -558,29 +669,22 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 6 : 2) k_em_strea
             }
         }
     }
-    // this block's share of the load, summed in thread order (a block with
-    // no wall node writes the zeros that sum would give)
-    __shared__ double red[3][EM_THREADS];
-    double* pt0 = a.part + ((size_t)b * a.nblk + blockIdx.x) * 3;
-    if (!__syncthreads_or(wallnode)) {
-        if (threadIdx.x == 0) pt0[0] = pt0[1] = pt0[2] = 0.0;
-        return;
+    // this block's share of the load: a tree per warp, then the warps in order
+    // (blocks with no wall node have none)
+    const int slot = __ldg(a.wblk + blk);
+    if (slot < 0) return;
+    __shared__ double red[3][EM_THREADS / 32];
+    const double v0 = warp_sum(fcx), v1 = warp_sum(fcy), v2 = warp_sum(fcm);
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = v0;
+        red[1][threadIdx.x >> 5] = v1;
+        red[2][threadIdx.x >> 5] = v2;
     }
-    red[0][threadIdx.x] = fcx;
-    red[1][threadIdx.x] = fcy;
-    red[2][threadIdx.x] = fcm;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        for (int t = 0; t < EM_THREADS; ++t) {
-            s0 += red[0][t];
-            s1 += red[1][t];
-            s2 += red[2][t];
-        }
-        double* pt = a.part + ((size_t)b * a.nblk + blockIdx.x) * 3;
-        pt[0] = s0;
-        pt[1] = s1;
-        pt[2] = s2;
+    if (threadIdx.x < 3) {
+        double s = 0.0;
+        for (int t = 0; t < EM_THREADS / 32; ++t) s += red[threadIdx.x][t];
+        a.part[((size_t)b * a.nwblk + slot) * 3 + threadIdx.x] = s;
     }
 }
 
@@ -594,56 +698,44 @@ __global__ void __launch_bounds__(EM_THREADS) k_em_record(const EArgs a) {
     if (n >= a.N) return;
     const size_t N = (size_t)a.N;
     R2* dxe = static_cast<R2*>(a.dep_xe);
-    if (a.kind[n] != 0) {
-        for (int q = 0; q < 9; ++q) {
-            a.dep_e[q * N + n] = -1;
-            dxe[q * N + n] = pair(R(0), R(0));
-        }
-        return;
-    }
+    const bool inner = a.kind[n] == 0;
     const SolveDev& fl = a.flow;
     const R dt = flowv<R>(fl, fl.dt, fl.dt_f);
-    const R* X = static_cast<const R*>(a.X);
+    const R2 x = static_cast<const R2*>(a.X)[n];
     BodyMap<R> still{};
     still.active = 0;
     R i00, i01, i10, i11, vx, vy;
-    inv_map(still, X[2 * n], X[2 * n + 1], i00, i01, i10, i11, vx, vy);
+    inv_map(still, x.x, x.y, i00, i01, i10, i11, vx, vy);
 #pragma unroll 1
     for (int q = 0; q < 9; ++q) {
         const R cx = (R)cxq(q), cy = (R)cyq(q);
-        const R hx = i00 * cx + i01 * cy - vx, hy = i10 * cx + i11 * cy - vy;
-        int e;
-        R xi, eta;
-        if (em_locate<R>(a, n, -dt * hx, -dt * hy, e, xi, eta)) {
-            a.dep_e[q * N + n] = e;
-            dxe[q * N + n] = pair(xi, eta);
-        } else {
-            a.dep_e[q * N + n] = -1;
-            dxe[q * N + n] = pair(R(0), R(0));
+        const R hx = fm(i00, cx, fm(i01, cy, -vx)), hy = fm(i10, cx, fm(i11, cy, -vy));
+        int code = -1;
+        R xi = R(0), eta = R(0);
+        if (!inner || !em_locate<R>(a, n, -dt * hx, -dt * hy, code, xi, eta)) {
+            code = -1;
+            xi = eta = R(0);
         }
+        a.dep_e[q * N + n] = code;
+        dxe[q * N + n] = pair(xi, eta);
     }
 }
 
-// ---- launch 4: one warp per solve: the load from the block partials in a
-// fixed order (lane t sums blocks t, t + 32, ...; then the lanes in order),
-// RK4 (Sec. III B) and the next step's blended maps
+// ---- launch 4: one warp per solve: the load from the partials of the blocks
+// with wall nodes, in a fixed order, the body's step (Sec. III B) and the next
+// step's blended maps
 __global__ void k_em_finish(const EArgs a) {
+    wait_previous();
+    __shared__ StepMaps s_rec;
     const int b = blockIdx.x, l = threadIdx.x;
-    const double* pt = a.part + (size_t)b * a.nblk * 3;
-    double v[3] = {0.0, 0.0, 0.0};
-    for (int k = l; k < a.nblk; k += 32)
-        for (int c = 0; c < 3; ++c) v[c] += pt[3 * k + c];
+    const double* pt = a.part + (size_t)b * a.nwblk * 3;
+    const BodyLane bl = body_lane(a.bodies[b], a.prop[b], a.maps_in[b], a.flow.dt, (unsigned)a.kstep + 1u, l);
     double F[3] = {0.0, 0.0, 0.0};
-    for (int t = 0; t < 32; ++t)
-        for (int c = 0; c < 3; ++c) F[c] += __shfl_sync(0xffffffffu, v[c], t);
-    if (l != 0) return;
-    const BodyDev bd = a.bodies[b];
-    const BodyStateDev Sn = a.maps_in[b].S_next;
-    const BodyStateDev Snew = rk4_body(bd, Sn, F[1], F[2], a.flow.dt, (long long)a.kstep);
-    StepMaps mo;
-    build_maps(bd, Sn, Snew, Sn, a.flow.dt, mo);
-    for (int c = 0; c < 3; ++c) mo.loads[c] = F[c];
-    a.maps_out[b] = mo;
+    for (int k = l; k < a.nwblk; k += 32)
+        for (int c = 0; c < 3; ++c) F[c] += pt[3 * k + c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) F[c] = warp_sum(F[c]);
+    body_records(bl, F, a.flow.idt, 1, l, s_rec, a.maps_out + b, nullptr);
 }
 
 }  // namespace
@@ -655,21 +747,24 @@ using lbfsi::SolveDev;
 using lbfsi::StepMaps;
 
 struct lbfsi_emesh_s {
-    int N = 0, Ne = 0, nwall = 0, nfarn = 0, nbatch = 0, precision = 0, nblk = 0;
+    int N = 0, Ne = 0, nwall = 0, nfarn = 0, nbatch = 0, precision = 0, nblk = 0, nwblk = 0;
+    size_t stage_bytes = 0;   // shared memory of the staged stream, 0: not staged
+    int snode = 0;
     size_t es = 8;   // element size of the path
     cudaStream_t stream = nullptr;
     std::vector<lbfsi_body_desc> bodies;
     std::vector<void*> blocks;   // every device allocation
     // mesh
     void* X = nullptr;
-    int* E = nullptr;
+    int *E = nullptr, *eptr = nullptr, *nptr = nullptr, *nlist = nullptr, *border = nullptr, *wblk = nullptr;
+    unsigned short* lnode = nullptr;
     void* ecoef = nullptr;
     int *hptr = nullptr, *hold = nullptr, *gptr = nullptr, *gcol = nullptr, *kind = nullptr;
     void* gw = nullptr;
     double *xw = nullptr, *n0 = nullptr, *wgeo = nullptr, *nfar = nullptr;
     // cached departures of the interior nodes the blend does not move
-    // ([9][N] position in hold of the holding element, [9][N] (xi, eta)),
-    // or null
+    // ([9][N] entry of hold of the holding element, [9][N] (xi, eta)), or
+    // null
     int* dep_e = nullptr;
     void* dep_xe = nullptr;
     // solves
@@ -677,11 +772,13 @@ struct lbfsi_emesh_s {
     void* ppost = nullptr;
     void* M[2] = {nullptr, nullptr};
     void* D = nullptr;
-    void* dQ = nullptr;   // [nbatch][2][N] dQ of the last streamed moments
+    void* dQ = nullptr;   // [nbatch][N] pairs: dQ of the last streamed moments
     StepMaps* maps[2] = {nullptr, nullptr};
     BodyDev* dbodies = nullptr;
+    lbfsi::BodyProp* dprop = nullptr;
     double* part = nullptr;
     double* stage = nullptr;   // [nbatch][4][N] float64 staging
+    int* inv = nullptr;        // [N] the caller's node i is library node inv[i]
     BodyStateDev *st_a = nullptr, *st_b = nullptr;
     double* zl = nullptr;
     unsigned* status = nullptr;
@@ -897,7 +994,12 @@ lbfsi::EArgs make_eargs(lbfsi_emesh m) {
     a.kstep = (int)m->k;
     a.collide = m->k > 0u;
     a.X = m->X;
+    a.eptr = m->eptr;
     a.E = m->E;
+    a.nptr = m->nptr;
+    a.nlist = m->nlist;
+    a.lnode = m->lnode;
+    a.snode = m->snode;
     a.ecoef = m->ecoef;
     a.hptr = m->hptr;
     a.hold = m->hold;
@@ -922,6 +1024,10 @@ lbfsi::EArgs make_eargs(lbfsi_emesh m) {
     a.maps_in = m->maps[c];
     a.maps_out = m->maps[c ^ 1];
     a.bodies = m->dbodies;
+    a.prop = m->dprop;
+    a.border = m->border;
+    a.wblk = m->wblk;
+    a.nwblk = m->nwblk;
     a.part = m->part;
     a.flow = m->flow;
     a.status = m->status;
@@ -933,14 +1039,20 @@ lbfsi::EArgs make_eargs(lbfsi_emesh m) {
 template <typename R>
 cudaError_t launch_em_collide(lbfsi_emesh m) {
     const lbfsi::EArgs a = make_eargs<R>(m);
-    const dim3 grid((unsigned)m->nblk, (unsigned)m->nbatch);
+    cudaError_t e = cudaSuccess;
+    constexpr int NS = lbfsi::em_solves<R>();
+    const bool multi = NS > 1 && m->nbatch > 1;
+    const dim3 grid((unsigned)m->nblk, (unsigned)(multi ? (m->nbatch + NS - 1) / NS : m->nbatch));
     if (a.collide) {
-        lbfsi::k_em_D<R><<<grid, lbfsi::EM_THREADS, 0, m->stream>>>(a);
+        if (multi) e = lbfsi::launch_behind(lbfsi::k_em_D<R, NS>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
+        else e = lbfsi::launch_behind(lbfsi::k_em_D<R, 1>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
         m->launches++;
     }
-    lbfsi::k_em_collide<R><<<grid, lbfsi::EM_THREADS, 0, m->stream>>>(a);
+    if (e != cudaSuccess) return e;
+    if (multi) e = lbfsi::launch_behind(lbfsi::k_em_collide<R, NS>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
+    else e = lbfsi::launch_behind(lbfsi::k_em_collide<R, 1>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
     m->launches++;
-    return cudaGetLastError();
+    return e;
 }
 
 template <typename R>
@@ -948,11 +1060,16 @@ cudaError_t launch_em_step(lbfsi_emesh m) {
     cudaError_t e = launch_em_collide<R>(m);
     if (e != cudaSuccess) return e;
     const lbfsi::EArgs a = make_eargs<R>(m);
-    const dim3 grid((unsigned)m->nblk, (unsigned)m->nbatch);
-    lbfsi::k_em_stream<R><<<grid, lbfsi::EM_THREADS, 0, m->stream>>>(a);
-    lbfsi::k_em_finish<<<m->nbatch, 32, 0, m->stream>>>(a);
+    const dim3 grid((unsigned)m->nblk * (unsigned)m->nbatch);
+    if constexpr (sizeof(R) == 4) {
+        if (m->stage_bytes) e = lbfsi::launch_behind(lbfsi::k_em_stream<R, true>, grid, lbfsi::EM_THREADS, m->stage_bytes, m->stream, sizeof(R) == 4, a);
+        else e = lbfsi::launch_behind(lbfsi::k_em_stream<R, false>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
+    } else {
+        e = lbfsi::launch_behind(lbfsi::k_em_stream<R, false>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
+    }
+    if (e == cudaSuccess) e = lbfsi::launch_behind(lbfsi::k_em_finish, m->nbatch, 32, 0, m->stream, sizeof(R) == 4, a);
     m->launches += 2;
-    return cudaGetLastError();
+    return e;
 }
 
 int em_status(lbfsi_emesh m) {
@@ -965,6 +1082,7 @@ int em_status(lbfsi_emesh m) {
         return efail(LBFSI_EDEPARTURE, "departure point outside the elements holding its node (CFL)");
     if (st & lbfsi::ST_BPOINT)
         return efail(LBFSI_EDEPARTURE, "wall or far-field target point B outside the elements holding its node");
+    if (st & lbfsi::ST_BOUNDS) return efail(LBFSI_EBOUNDS, "element outside its block's tables (bounds-checked build)");
     if (st & lbfsi::ST_NONPHYS) return efail(LBFSI_ENONPHYS, "non-physical state (rho<=0, T<=0 or NaN)");
     return LBFSI_OK;
 }
@@ -1032,7 +1150,7 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
         }
     }
     // subparametric elements: every node at the bilinear position of the corners
-    std::vector<double> ecoef(6 * (size_t)Ne);
+    std::vector<double> ecoef(8 * (size_t)Ne, 0.0);
     for (int e = 0; e < Ne; ++e) {
         const int* en = &E[9 * (size_t)e];
         for (int c = 0; c < 2; ++c) {
@@ -1047,9 +1165,9 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
                         return efail(LBFSI_EINVAL, "elements must be subparametric (mid nodes at the bilinear "
                                                    "positions of the corners)");
                 }
-            ecoef[6 * (size_t)e + c] = 0.25 * (-c00 + c10 - c01 + c11);
-            ecoef[6 * (size_t)e + 2 + c] = 0.25 * (-c00 - c10 + c01 + c11);
-            ecoef[6 * (size_t)e + 4 + c] = 0.25 * (c00 - c10 - c01 + c11);
+            ecoef[8 * (size_t)e + c] = 0.25 * (-c00 + c10 - c01 + c11);
+            ecoef[8 * (size_t)e + 2 + c] = 0.25 * (-c00 - c10 + c01 + c11);
+            ecoef[8 * (size_t)e + 4 + c] = 0.25 * (c00 - c10 - c01 + c11);
         }
     }
     // node -> holding elements, in increasing element index
@@ -1073,24 +1191,79 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
     int rc = d->grid_ij ? gradient_r18(N, ijr.data(), d->grid_nr, d->grid_nt, X, gptr, gcol, gw)
                         : gradient_r33(N, E, X, hptr, hold, gptr, gcol, gw);
     if (rc) return rc;
-    // elements stored in the order of their centre nodes (so along the same
-    // curve as the nodes); each node's list of holding elements keeps the
-    // caller's element order, the order of the departure search
-    std::vector<int> eperm((size_t)Ne), einv((size_t)Ne);
-    for (int e2 = 0; e2 < Ne; ++e2) eperm[e2] = e2;
-    std::stable_sort(eperm.begin(), eperm.end(),
-                     [&](int a, int b) { return E[9 * (size_t)a + 4] < E[9 * (size_t)b + 4]; });
-    for (int k = 0; k < Ne; ++k) einv[eperm[k]] = k;
+    // each stream block's own copy of the tables of the elements that hold its
+    // nodes, in the order of their centre nodes (so along the same curve as
+    // the nodes), and the list of those elements' nodes; each node's list of
+    // holding elements keeps the caller's element order, the order of the
+    // departure search
+    const int nblk = (N + lbfsi::EM_THREADS - 1) / lbfsi::EM_THREADS;
+    std::vector<int> eptr((size_t)nblk + 1, 0), nptr((size_t)nblk + 1, 0), nlist, Ep;
+    std::vector<double> ecb;
+    std::vector<unsigned short> lnode;
+    int snode = 0, selem = 0;
     {
-        std::vector<int> Es(E.size());
-        std::vector<double> cs(ecoef.size());
-        for (int k = 0; k < Ne; ++k) {
-            std::copy_n(&E[9 * (size_t)eperm[k]], 9, &Es[9 * (size_t)k]);
-            std::copy_n(&ecoef[6 * (size_t)eperm[k]], 6, &cs[6 * (size_t)k]);
+        std::vector<int> eperm((size_t)Ne), einv((size_t)Ne), slot((size_t)Ne, -1), at((size_t)N, 0), be;
+        for (int e2 = 0; e2 < Ne; ++e2) eperm[e2] = e2;
+        std::stable_sort(eperm.begin(), eperm.end(),
+                         [&](int a, int b) { return E[9 * (size_t)a + 4] < E[9 * (size_t)b + 4]; });
+        for (int k = 0; k < Ne; ++k) einv[eperm[k]] = k;
+        for (int blk = 0; blk < nblk; ++blk) {
+            const int n0 = blk * lbfsi::EM_THREADS, n1 = std::min(N, n0 + lbfsi::EM_THREADS);
+            be.clear();
+            for (int h = hptr[n0]; h < hptr[n1]; ++h) be.push_back(einv[hold[h] >> 4]);
+            std::sort(be.begin(), be.end());
+            be.erase(std::unique(be.begin(), be.end()), be.end());
+            if (Ep.size() / lbfsi::EN_STRIDE + be.size() > (1u << 27) - 1u) return efail(LBFSI_EINVAL, "mesh too large");
+            const size_t nl0 = nlist.size();
+            for (int k : be)
+                for (int s = 0; s < 9; ++s) nlist.push_back(E[9 * (size_t)eperm[k] + s]);
+            std::sort(nlist.begin() + nl0, nlist.end());
+            nlist.erase(std::unique(nlist.begin() + nl0, nlist.end()), nlist.end());
+            const int nn = (int)(nlist.size() - nl0);
+            for (int k = 0; k < nn; ++k) at[nlist[nl0 + k]] = k;
+            for (size_t k = 0; k < be.size(); ++k) {
+                const int e2 = eperm[be[k]];
+                slot[e2] = eptr[blk] + (int)k;
+                for (int s = 0; s < lbfsi::EN_STRIDE; ++s) {
+                    Ep.push_back(s < 9 ? E[9 * (size_t)e2 + s] : 0);
+                    // (past the staged sizes the offsets are not used)
+                    lnode.push_back(s < 9 ? (unsigned short)(at[E[9 * (size_t)e2 + s]] * 8) : 0);
+                }
+                ecb.insert(ecb.end(), &ecoef[8 * (size_t)e2], &ecoef[8 * (size_t)e2] + 8);
+            }
+            for (int h = hptr[n0]; h < hptr[n1]; ++h) hold[h] = slot[hold[h] >> 4] * 16 + (hold[h] & 15) / 3 * 4 + (hold[h] & 15) % 3;
+            eptr[blk + 1] = eptr[blk] + (int)be.size();
+            nptr[blk + 1] = (int)nlist.size();
+            snode = std::max(snode, nn);
+            selem = std::max(selem, (int)be.size());
         }
-        E.swap(Es);
-        ecoef.swap(cs);
-        for (int& h : hold) h = einv[h >> 4] * 16 + (h & 15);
+    }
+    // gradient operator rows in slices of 32 nodes
+    {
+        const int ns = (N + 31) / 32;
+        std::vector<int> sp((size_t)ns + 1, 0), sc;
+        for (int k = 0; k < ns; ++k) {
+            int len = 0;
+            for (int n = 32 * k; n < std::min(N, 32 * k + 32); ++n) len = std::max(len, gptr[n + 1] - gptr[n]);
+            sp[k + 1] = sp[k] + len;
+        }
+        sc.resize(32 * (size_t)sp[ns]);
+        std::vector<double> sw(2 * sc.size(), 0.0);
+        for (int n = 0; n < 32 * ns; ++n) {
+            const int k = n / 32;
+            for (int c = 0; c < sp[k + 1] - sp[k]; ++c) {
+                const size_t to = 32 * ((size_t)sp[k] + c) + (size_t)(n % 32);
+                const bool in = n < N && c < gptr[n + 1] - gptr[n];
+                sc[to] = in ? gcol[gptr[n] + c] : std::min(n, N - 1);
+                if (in) {
+                    sw[2 * to] = gw[2 * ((size_t)gptr[n] + c)];
+                    sw[2 * to + 1] = gw[2 * ((size_t)gptr[n] + c) + 1];
+                }
+            }
+        }
+        gptr.swap(sp);
+        gcol.swap(sc);
+        gw.swap(sw);
     }
     // chains
     std::vector<int> kind(N, 0);
@@ -1109,6 +1282,20 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
         pf[2 * f] = X[2 * n];
         pf[2 * f + 1] = X[2 * n + 1];
     }
+    std::vector<int> wblk((size_t)nblk, -1);
+    int nwblk = 0;
+    for (int n = 0; n < N; ++n)
+        if (kind[n] > 0 && wblk[n / lbfsi::EM_THREADS] < 0) wblk[n / lbfsi::EM_THREADS] = nwblk++;
+    std::vector<int> border((size_t)nblk), weight((size_t)nblk, 0);
+    for (int n = 0; n < N; ++n) {
+        int& w = weight[n / lbfsi::EM_THREADS];
+        if (kind[n] > 0) w = 2;
+        for (int b = 0; b < d->nbatch && w == 0; ++b)
+            if (d->bodies[b].dof != 0 && std::hypot(X[2 * n] - d->bodies[b].xc, X[2 * n + 1] - d->bodies[b].yc) < d->bodies[b].r_out)
+                w = 1;
+    }
+    for (int k = 0; k < nblk; ++k) border[k] = k;
+    std::stable_sort(border.begin(), border.end(), [&](int a, int b) { return weight[a] > weight[b]; });
     std::vector<double> n0, wgeo, nfar, fgeo;
     lbfsi::chain_geometry(pw, n0, wgeo);
     lbfsi::chain_geometry(pf, nfar, fgeo);
@@ -1131,7 +1318,11 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
     m->nbatch = d->nbatch;
     m->precision = d->precision;
     m->es = d->precision == LBFSI_FP64 ? sizeof(double) : sizeof(float);
-    m->nblk = (N + lbfsi::EM_THREADS - 1) / lbfsi::EM_THREADS;
+    m->nblk = nblk;
+    m->nwblk = nwblk;
+    m->snode = (snode + 1) & ~1;
+    m->stage_bytes = lbfsi::em_stage_bytes(m->snode, selem);
+    if (d->precision != LBFSI_FP32 || m->stage_bytes > lbfsi::EM_STAGE_MAX) m->stage_bytes = 0;
     m->stream = static_cast<cudaStream_t>(cuda_stream);
     m->bodies.assign(d->bodies, d->bodies + d->nbatch);
     m->perm = perm;
@@ -1144,12 +1335,20 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
         *dst = q;
         return e;
     };
-    const std::vector<unsigned char> Xt = typed(Xv, d->precision), ect = typed(ecoef, d->precision),
+    const std::vector<unsigned char> Xt = typed(Xv, d->precision), ect = typed(ecb, d->precision),
                                      gwt = typed(gw, d->precision);
     cudaError_t e = put(&m->X, Xt.data(), Xt.size());
-    std::vector<int> Ep((size_t)Ne * lbfsi::EN_STRIDE, 0);
-    for (size_t k = 0; k < (size_t)Ne; ++k)
-        for (int s = 0; s < 9; ++s) Ep[k * lbfsi::EN_STRIDE + s] = E[9 * k + s];
+    if (e == cudaSuccess) e = put((void**)&m->eptr, eptr.data(), eptr.size() * sizeof(int));
+    if (e == cudaSuccess) e = put((void**)&m->border, border.data(), border.size() * sizeof(int));
+    if (e == cudaSuccess) e = put((void**)&m->wblk, wblk.data(), wblk.size() * sizeof(int));
+    if (e == cudaSuccess && m->stage_bytes) {
+        e = put((void**)&m->nptr, nptr.data(), nptr.size() * sizeof(int));
+        if (e == cudaSuccess) e = put((void**)&m->nlist, nlist.data(), nlist.size() * sizeof(int));
+        if (e == cudaSuccess) e = put((void**)&m->lnode, lnode.data(), lnode.size() * sizeof(unsigned short));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute((const void*)lbfsi::k_em_stream<float, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbfsi::EM_STAGE_MAX);
+    }
     if (e == cudaSuccess) e = put((void**)&m->E, Ep.data(), Ep.size() * sizeof(int));
     if (e == cudaSuccess) e = put(&m->ecoef, ect.data(), ect.size());
     if (e == cudaSuccess) e = put((void**)&m->hptr, hptr.data(), hptr.size() * sizeof(int));
@@ -1157,6 +1356,7 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
     if (e == cudaSuccess) e = put((void**)&m->gptr, gptr.data(), gptr.size() * sizeof(int));
     if (e == cudaSuccess) e = put((void**)&m->gcol, gcol.data(), std::max<size_t>(gcol.size(), 1) * sizeof(int));
     if (e == cudaSuccess) e = put(&m->gw, gwt.data(), std::max<size_t>(gwt.size(), 1));
+    if (e == cudaSuccess) e = put((void**)&m->inv, inv.data(), inv.size() * sizeof(int));
     if (e == cudaSuccess) e = put((void**)&m->kind, kind.data(), kind.size() * sizeof(int));
     if (e == cudaSuccess) e = put((void**)&m->xw, pw.data(), pw.size() * sizeof(double));
     if (e == cudaSuccess) e = put((void**)&m->n0, n0.data(), n0.size() * sizeof(double));
@@ -1177,7 +1377,8 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
     if (e == cudaSuccess) e = ealloc(m, &q, nb * 2 * N * es);
     m->dQ = q;
     if (e == cudaSuccess) e = ealloc(m, &m->dbodies, nb);
-    if (e == cudaSuccess) e = ealloc(m, &m->part, nb * m->nblk * 3);
+    if (e == cudaSuccess) e = ealloc(m, &m->dprop, nb);
+    if (e == cudaSuccess) e = ealloc(m, &m->part, nb * (size_t)m->nwblk * 3);
     if (e == cudaSuccess) e = ealloc(m, &m->stage, nb * 4 * N);
     if (e == cudaSuccess) e = ealloc(m, &m->st_a, nb);
     if (e == cudaSuccess) e = ealloc(m, &m->st_b, nb);
@@ -1222,6 +1423,8 @@ int lbfsi_emesh_init_fields(lbfsi_emesh m, const lbfsi_flow_params* p, const dou
     const size_t N = (size_t)m->N, nb = (size_t)m->nbatch;
     std::vector<BodyDev> bd(nb);
     for (size_t b = 0; b < nb; ++b) bd[b] = lbfsi::body_dev(m->bodies[b], proto.rho_inf, proto.uinf_x);
+    std::vector<lbfsi::BodyProp> prop(nb);
+    for (size_t b = 0; b < nb; ++b) prop[b] = lbfsi::body_prop(bd[b], proto.dt);
     std::vector<double> Mh;
     if (rho_u_T) {
         // the caller's node order -> the library's
@@ -1241,6 +1444,8 @@ int lbfsi_emesh_init_fields(lbfsi_emesh m, const lbfsi_flow_params* p, const dou
     std::vector<BodyStateDev> zero(nb, BodyStateDev{0.0, 0.0, 0.0, 0.0});
     std::vector<double> zl(nb * 3, 0.0);
     cudaError_t e = cudaMemcpyAsync(m->dbodies, bd.data(), nb * sizeof(BodyDev), cudaMemcpyHostToDevice, m->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m->dprop, prop.data(), nb * sizeof(lbfsi::BodyProp), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->stage, Mh.data(), nb * 4 * N * sizeof(double), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
@@ -1335,13 +1540,14 @@ int lbfsi_emesh_get_body_state(lbfsi_emesh m, lbfsi_body_state* out) {
 
 int lbfsi_emesh_get_fields(lbfsi_emesh m, double* rho_u_T) {
     if (!m || !rho_u_T) return efail(LBFSI_EINVAL, "null argument");
+    // widened and put into the caller's node order on the device
     const size_t N = (size_t)m->N, rows = (size_t)m->nbatch * 4;
-    std::vector<double> v(rows * N);
-    const int rc = download(m, m->M[m->cur()], v.data(), rows * N);
-    if (rc) return rc;
-    for (size_t r = 0; r < rows; ++r)
-        for (size_t i = 0; i < N; ++i) rho_u_T[r * N + (size_t)m->perm[i]] = v[r * N + i];
-    return LBFSI_OK;
+    cudaError_t e = lbfsi::launch_read(m->precision, m->M[m->cur()], N, m->inv, m->stage, m->N, rows, m->stream);
+    m->launches++;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(rho_u_T, m->stage, rows * N * sizeof(double), cudaMemcpyDeviceToHost, m->stream);
+    if (e != cudaSuccess) return ecuda(e, "fields download");
+    return em_status(m);
 }
 
 int lbfsi_emesh_get_populations(lbfsi_emesh m, int which, double* f, double* g) {
