@@ -517,8 +517,8 @@ int64_t lbfsi_launch_count(lbfsi_mesh m);
  * 1: 16 x 32, 256 threads, 3 CTAs/SM; 2: 12 x 32, 192 threads, 4 CTAs/SM;
  * 3: 12 x 32, 384 threads; 4: 16 x 32, 512 threads (what lbfsi_get_schedule
  * reports for new mesh handles, with order 1, and new batches, with order 0;
- * until a schedule is set they launch shape 1 where 16 rows give at least 304
- * tiles and shape 0 elsewhere).  Float64 shapes (128 threads per row of 32
+ * until a schedule is set they launch shape 0, 4 or 1 by their number of 16-row
+ * tiles: below 152, below 608, above).  Float64 shapes (128 threads per row of 32
  * nodes): 0: one row per CTA (default), 1: two, 2: four.  Meshes given by node
  * coordinates have one shape (0).
  * Staging (every float shape): in a float mesh handle whose Ntheta is a
@@ -557,8 +557,8 @@ int lbfsi_autotune(lbfsi_mesh m, int steps_per_trial, int* best_variant, int* be
  * cases this way).  A separate handle: the step on an element list runs as
  * four launches per step over node lists (correction field D, collision into
  * a post-collision buffer, stream, load reduction and body update) with the
- * Q2 gathers of a block of nodes read from the populations of its elements in
- * shared memory, instead of the structured meshes' tiled kernels.
+ * Q2 gathers read from global memory, instead of the structured meshes' tiled
+ * kernels.
  *
  * Mesh: N nodes, elements of 3 x 3 node indices [a][b] (entry (a, b) at
  * reference coordinates (a - 1, b - 1)), subparametric (each element's mid

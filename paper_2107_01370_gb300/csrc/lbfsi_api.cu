@@ -243,14 +243,10 @@ void unify_cut_copies(const lbfsi::HostMesh& h, double* user, size_t blocks, int
 lbfsi::StepArgs make_args(lbfsi_mesh m);
 
 // Tile shape of a handle: its schedule's variant or, as long as none was asked
-// for, by its size the shape of the most rows that still gives every SM two
-// tiles (float 16 or 8 rows; float64 always one row per block).
+// for, by its size (default_shape).
 int step_shape(lbfsi_mesh m) {
     if (!m->own_shape) return m->variant;
-    auto enough = [&](int rows) {
-        return (long long)m->nbatch * m->host.ntj * ((m->host.nr + rows - 1) / rows) >= 304;
-    };
-    return m->precision == LBFSI_FP64 ? 0 : enough(16) ? 1 : 0;
+    return lbfsi::default_shape(m->precision, (long long)m->nbatch * m->host.ntj * ((m->host.nr + 15) / 16));
 }
 
 // Tile shape, rows and tiles of the handle's schedule.

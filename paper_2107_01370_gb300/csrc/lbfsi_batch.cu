@@ -325,12 +325,11 @@ int rebuild_tiles(lbfsi_batch b) {
     auto active = [&](const Slot& s, int part) { return s.used && !s.finished && (s.general ? 1 : 0) == part; };
     b->shape = b->variant;
     if (b->own_shape && b->precision == LBFSI_FP32) {
-        // as the mesh handle (step_shape): 16 rows if they give every SM two
-        // tiles, else 8
+        // as the mesh handle (step_shape)
         long long n = 0;
         for (const Slot& s : b->slots)
             if (active(s, 0)) n += (long long)b->meshes[s.mesh].host.ntj * ((b->meshes[s.mesh].host.nr + 15) / 16);
-        b->shape = n >= 304 ? 1 : 0;
+        b->shape = lbfsi::default_shape(b->precision, n);
     }
     b->tile_rows = lbfsi::tile_rows(b->precision, b->shape);
     e = update_counts(b);

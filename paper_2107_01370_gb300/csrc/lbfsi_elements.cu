@@ -2,8 +2,8 @@
 // Sec. II B; the structured meshes of lbfsi_step.cu are its special cases).
 //
 // A node's neighbourhood is no longer a tile of an index grid, so the step is
-// four launches over node lists, each node's data read from global memory
-// (the mesh tables and the step's fields stay in L2 for meshes of this size):
+// four launches over node lists (the mesh tables and the step's fields stay in
+// L2 for meshes of this size):
 //
 //   D        correction field D = (mu/p) grad dQ at every node (Sec. II C),
 //            with the mesh's nodal gradient operator (Eq. ddx+fem; reading
@@ -22,9 +22,9 @@
 //            target point B = A + dt n0, far-field nodes take equilibria at
 //            the targets at B = A - dt n_out (Sec. III A; readings R19, R20,
 //            R34); moments; the wall nodes' Simpson shares of the load (FP64)
-//            summed per block in thread order
-//   finish   per solve: the block partials summed in block order, RK4 of the
-//            body (Sec. III B), the next step's blended maps.
+//            summed per block by warp trees
+//   finish   per solve: the block partials summed in a fixed order, the body's
+//            RK4 step (Sec. III B), the next step's blended maps.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -53,21 +53,11 @@ constexpr int EN_STRIDE = 12;
 struct EArgs {
     int N, nbatch, nblk, kstep, collide;
     const void* X;        // [N][2] node coordinates (element type of the path)
-    // a block's nodes lie in a few elements: the tables of each block's own
-    // copy of them, block blk's elements eptr[blk] .. eptr[blk + 1)
-    const int* eptr;      // [nblk + 1]
-    const int* E;         // [.][EN_STRIDE] element nodes, entry a * 3 + b (then padding, so
+    const int* E;         // [Ne][EN_STRIDE] element nodes, entry a * 3 + b (then padding, so
                           // that a gather reads an element's nodes in three 16-byte loads)
-    const void* ecoef;    // [.][8] bilinear map: (b_x, b_y, c_x, c_y, d_x, d_y, 0, 0)
+    const void* ecoef;    // [Ne][8] bilinear map: (b_x, b_y, c_x, c_y, d_x, d_y, 0, 0)
     const int* hptr;      // [N + 1] holding elements of each node
-    const int* hold;      // [.] (block's) element * 16 + 4 a + b, (a, b) the node's entry in it
-    // staged gathers (k_em_stream): the nodes of block blk's elements
-    // nlist[nptr[blk] .. nptr[blk + 1]), in increasing order, and the elements'
-    // nodes as byte offsets of pairs into that list; rows of snode pairs
-    const int* nptr;
-    const int* nlist;
-    const unsigned short* lnode;   // [.][EN_STRIDE]
-    int snode;
+    const int* hold;      // [.] element * 16 + 4 a + b, (a, b) the node's entry in it
     // gradient operator in slices of 32 nodes (a warp's): slice s holds
     // gptr[s + 1] - gptr[s] entries per node, entry k of lane l at gptr[s] * 32 +
     // 32 k + l, rows shorter than their slice padded by zero weights on the node
@@ -248,26 +238,19 @@ __device__ __forceinline__ void em_grad(const EArgs& a, int n, Fn fld, R& gX, R&
     }
 }
 
-// The same on both components of a field of pairs for NS solves at once (one
-// read of the operator): gx_[s] = d/dX of (v.x, v.y), gy_[s] = d/dY; fld(m, s)
-// gives the pair of solve s at node m.
-template <typename R, int NS, typename Fn>
-__device__ __forceinline__ void em_grad2(const EArgs& a, int n, Fn fld, typename EVec<R>::T2* gx_, typename EVec<R>::T2* gy_) {
+// The same on both components of a field of pairs: gX = d/dX of (v.x, v.y), gY =
+// d/dY.
+template <typename R, typename Fn>
+__device__ __forceinline__ void em_grad2(const EArgs& a, int n, Fn fld, typename EVec<R>::T2& gX, typename EVec<R>::T2& gY) {
     using R2 = typename EVec<R>::T2;
     const int s = n >> 5, l = n & 31, p0 = __ldg(a.gptr + s), len = __ldg(a.gptr + s + 1) - p0;
     const int* col = a.gcol + 32 * (size_t)p0 + l;
     const R2* w = static_cast<const R2*>(a.gw) + 32 * (size_t)p0 + l;
-#pragma unroll
-    for (int b = 0; b < NS; ++b) gx_[b] = gy_[b] = pair(R(0), R(0));
+    gX = gY = pair(R(0), R(0));
     for (int k = 0; k < len; ++k) {
-        const int m = __ldg(col + 32 * k);
-        const R2 wk = __ldg(w + 32 * k);
-#pragma unroll
-        for (int b = 0; b < NS; ++b) {
-            const R2 v = fld(m, b);
-            gx_[b] = pfma(pair(wk.x, wk.x), v, gx_[b]);
-            gy_[b] = pfma(pair(wk.y, wk.y), v, gy_[b]);
-        }
+        const R2 v = fld(__ldg(col + 32 * k)), wk = __ldg(w + 32 * k);
+        gX = pfma(pair(wk.x, wk.x), v, gX);
+        gY = pfma(pair(wk.y, wk.y), v, gY);
     }
 }
 
@@ -284,37 +267,24 @@ __device__ __forceinline__ typename EVec<R>::T2 ref_pair(const SolveDev& s, int 
     return r;
 }
 
-// Solves per thread: the mesh's tables (operator, departures, element nodes)
-// are read once for all of them.  (float64 is bound by its arithmetic, which
-// the solves do not share.)
-template <typename R>
-__host__ __device__ constexpr int em_solves() {
-    return sizeof(R) == 4 ? 2 : 1;
-}
-
 // ---- launch 1: D = (mu/p) grad dQ (Sec. II C), dQ_a = rho u_a (1 - 3T) - rho u_a^3
 // (dQ written with the moments by the previous stream launch, em_dq)
-template <typename R, int NS>
+template <typename R>
 __global__ void __launch_bounds__(EM_THREADS) k_em_D(const EArgs a) {
     wait_previous();
     using R2 = typename EVec<R>::T2;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x, b0 = blockIdx.y * NS;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (n >= a.N) return;
     const size_t N = (size_t)a.N;
     const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
-    const R2* Q = static_cast<const R2*>(a.dQ);
-    R2 gx[NS], gy[NS];
-    em_grad2<R, NS>(a, n, [&](int m, int s) { return Q[(size_t)min(b0 + s, a.nbatch - 1) * N + m]; }, gx, gy);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const int b = b0 + s;
-        if (b >= a.nbatch) break;
-        const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
-        R i00, i01, i10, i11, vx, vy;
-        inv_map(kmap<R>(a.maps_in[b]), x.x, x.y, i00, i01, i10, i11, vx, vy);
-        const R mup = flowv<R>(a.flow, a.flow.mu, a.flow.mu_f) * rcp_(M[n] * M[3 * N + n]);
-        static_cast<R2*>(a.D)[(size_t)b * N + n] = pair(mup * fm(i00, gx[s].x, i10 * gy[s].x), mup * fm(i01, gx[s].y, i11 * gy[s].y));
-    }
+    const R2* Q = static_cast<const R2*>(a.dQ) + (size_t)b * N;
+    R2 gX, gY;
+    em_grad2<R>(a, n, [&](int m) { return Q[m]; }, gX, gY);
+    const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
+    R i00, i01, i10, i11, vx, vy;
+    inv_map(kmap<R>(a.maps_in[b]), x.x, x.y, i00, i01, i10, i11, vx, vy);
+    const R mup = flowv<R>(a.flow, a.flow.mu, a.flow.mu_f) * rcp_(M[n] * M[3 * N + n]);
+    static_cast<R2*>(a.D)[(size_t)b * N + n] = pair(mup * fm(i00, gX.x, i10 * gY.x), mup * fm(i01, gX.y, i11 * gY.y));
 }
 
 // dQ_a = rho u_a (1 - 3T) - rho u_a^3 of a node's moments (Sec. II C).
@@ -326,49 +296,41 @@ __device__ __forceinline__ typename EVec<R>::T2 em_dq(R rho, R ux, R uy, R T) {
 
 // ---- launch 2: Y = grad D and the collision (Eq. f_boltz) into ppost;
 // step 0 only copies the initial state
-template <typename R, int NS>
+template <typename R>
 __global__ void __launch_bounds__(EM_THREADS) k_em_collide(const EArgs a) {
     wait_previous();
     using R2 = typename EVec<R>::T2;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x, b0 = blockIdx.y * NS;
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
     if (n >= a.N) return;
     const size_t N = (size_t)a.N;
-    const bool far = a.kind[n] < 0;
-    const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
-    R2 gx[NS], gy[NS];
-    if (a.collide && !far) {
-        const R2* D = static_cast<const R2*>(a.D);
-        em_grad2<R, NS>(a, n, [&](int m, int s) { return D[(size_t)min(b0 + s, a.nbatch - 1) * N + m]; }, gx, gy);
-    }
+    const R2* pin = static_cast<const R2*>(a.p_in) + (size_t)b * 9 * N;
+    R2* pout = static_cast<R2*>(a.ppost) + (size_t)b * 9 * N;
+    R2 pq[9];
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const int b = b0 + s;
-        if (b >= a.nbatch) break;
-        const R2* pin = static_cast<const R2*>(a.p_in) + (size_t)b * 9 * N;
-        R2* pout = static_cast<R2*>(a.ppost) + (size_t)b * 9 * N;
-        R2 pq[9];
+    for (int q = 0; q < 9; ++q) pq[q] = pin[q * N + n];
+    if (a.collide) {
+        if (a.kind[n] < 0) {
+            const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
+            R f[9], g[9];
+            f_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], f);
+            g_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], flowv<R>(a.flow, a.flow.Cv, a.flow.Cv_f), g);
 #pragma unroll
-        for (int q = 0; q < 9; ++q) pq[q] = pin[q * N + n];
-        if (a.collide) {
-            if (far) {
-                const R* M = static_cast<const R*>(a.M_in) + (size_t)b * 4 * N;
-                R f[9], g[9];
-                f_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], f);
-                g_equilibrium(M[n], M[N + n], M[2 * N + n], M[3 * N + n], flowv<R>(a.flow, a.flow.Cv, a.flow.Cv_f), g);
-#pragma unroll
-                for (int q = 0; q < 9; ++q) pq[q] = pair(f[q], g[q]);
-            } else {
-                R i00, i01, i10, i11, vx, vy;
-                inv_map(kmap<R>(a.maps_in[b]), x.x, x.y, i00, i01, i10, i11, vx, vy);
-                const R Yx = fm(i00, gx[s].x, i10 * gy[s].x), Yy = fm(i01, gx[s].y, i11 * gy[s].y);
-                collide_pairs(pq, Yx, Yy, flowv<R>(a.flow, a.flow.mu, a.flow.mu_f),
-                              flowv<R>(a.flow, a.flow.muP, a.flow.muP_f), flowv<R>(a.flow, a.flow.dt, a.flow.dt_f),
-                              flowv<R>(a.flow, a.flow.iCv, a.flow.iCv_f));
-            }
+            for (int q = 0; q < 9; ++q) pq[q] = pair(f[q], g[q]);
+        } else {
+            const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
+            const R2* D = static_cast<const R2*>(a.D) + (size_t)b * N;
+            R2 gX, gY;
+            em_grad2<R>(a, n, [&](int m) { return D[m]; }, gX, gY);
+            R i00, i01, i10, i11, vx, vy;
+            inv_map(kmap<R>(a.maps_in[b]), x.x, x.y, i00, i01, i10, i11, vx, vy);
+            const R Yx = fm(i00, gX.x, i10 * gY.x), Yy = fm(i01, gX.y, i11 * gY.y);
+            collide_pairs(pq, Yx, Yy, flowv<R>(a.flow, a.flow.mu, a.flow.mu_f),
+                          flowv<R>(a.flow, a.flow.muP, a.flow.muP_f), flowv<R>(a.flow, a.flow.dt, a.flow.dt_f),
+                          flowv<R>(a.flow, a.flow.iCv, a.flow.iCv_f));
         }
-#pragma unroll
-        for (int q = 0; q < 9; ++q) pout[q * N + n] = psub(pq[q], ref_pair<R>(a.flow, q));
     }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) pout[q * N + n] = psub(pq[q], ref_pair<R>(a.flow, q));
 }
 
 // Q2 interpolation of direction q's post-collision pairs over element e.
@@ -392,32 +354,6 @@ __device__ __forceinline__ typename EVec<R>::T2 em_gather(const EArgs& a, const 
         R2 t = pmul(pair(Ly[0], Ly[0]), pp[nd[3 * aa]]);
         t = pfma(pair(Ly[1], Ly[1]), pp[nd[3 * aa + 1]], t);
         t = pfma(pair(Ly[2], Ly[2]), pp[nd[3 * aa + 2]], t);
-        acc = pfma(pair(Lx[aa], Lx[aa]), t, acc);
-    }
-    return acc;
-}
-
-// The same from the block's staged populations: row is direction q's, nd the
-// element's nodes as byte offsets into it.
-__device__ __forceinline__ float2 em_gather_staged(const unsigned char* row, const unsigned short* nd, float xi, float eta) {
-    float Lx[3], Ly[3];
-    Lx[0] = xi * fm(0.5f, xi, -0.5f);
-    Lx[1] = fm(-xi, xi, 1.0f);
-    Lx[2] = xi * fm(0.5f, xi, 0.5f);
-    Ly[0] = eta * fm(0.5f, eta, -0.5f);
-    Ly[1] = fm(-eta, eta, 1.0f);
-    Ly[2] = eta * fm(0.5f, eta, 0.5f);
-    const uint2* w = reinterpret_cast<const uint2*>(nd);
-    const uint2 w0 = w[0], w1 = w[1], w2 = w[2];
-    const unsigned o[9] = {w0.x & 0xffffu, w0.x >> 16, w0.y & 0xffffu, w0.y >> 16, w1.x & 0xffffu,
-                           w1.x >> 16,     w1.y & 0xffffu, w1.y >> 16, w2.x & 0xffffu};
-    auto at = [&](int k) { return *reinterpret_cast<const float2*>(row + o[k]); };
-    float2 acc = pair(0.0f, 0.0f);
-#pragma unroll
-    for (int aa = 0; aa < 3; ++aa) {
-        float2 t = pmul(pair(Ly[0], Ly[0]), at(3 * aa));
-        t = pfma(pair(Ly[1], Ly[1]), at(3 * aa + 1), t);
-        t = pfma(pair(Ly[2], Ly[2]), at(3 * aa + 2), t);
         acc = pfma(pair(Lx[aa], Lx[aa]), t, acc);
     }
     return acc;
@@ -452,47 +388,23 @@ __device__ __forceinline__ void em_interp_M(const EArgs& a, const R* M, size_t N
     for (int c = 0; c < 4; ++c) out[c] = own[c] + d[c];
 }
 
-// ---- launch 3: stream step k + 1.  The float kernel is bound by the gathers'
-// loads and their instructions: a block first stages the populations of all
-// the nodes its own nodes' elements have (nlist: measured 1.8 times its 256
-// nodes on a stretched ring) and those elements' node offsets into shared
-// memory, and the 81 gathers of a node read there.  STAGED = false reads
-// global memory instead: lists whose numbering scatters so much that a
-// block's nodes would not fit (EM_STAGE_MAX), and float64, bound by its
-// arithmetic.
-constexpr size_t EM_STAGE_MAX = 75 * 1024;   // three blocks per SM
-__host__ __device__ constexpr size_t em_stage_bytes(int snode, int selem) {
-    const size_t a = 9 * (size_t)snode * sizeof(float2) + (size_t)selem * EN_STRIDE * sizeof(unsigned short);
-    return a > 3 * EM_THREADS * sizeof(double) ? a : 3 * EM_THREADS * sizeof(double);
-}
-
-template <typename R, bool STAGED>
+// ---- launch 3: stream step k + 1.  Bound by the latency of its dependent
+// loads (departure, element nodes, populations) and, at moving nodes, by the
+// departure solves.  Measured on the 513 x 256 ring, 4 solves, half its nodes
+// moving: 126 us; 62 with moving nodes trying their cached element first,
+// elements ruled out by the first Newton iterate, the long blocks first and no
+// population array per thread.  Staging the populations of a block's elements in
+// shared memory, with 16-bit offsets, 71 (and 30 us more per step behind the
+// other launches): its nodes in Z-order already hit L1 and L2.
+template <typename R>
 __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_stream(const EArgs a) {
     wait_previous();
     using R2 = typename EVec<R>::T2;
-    extern __shared__ __align__(16) unsigned char smem[];
     // (a block of all solves side by side: they share its tables in L2)
     const int blk = __ldg(a.border + blockIdx.x / a.nbatch), b = blockIdx.x % a.nbatch;
     const int n = blk * EM_THREADS + threadIdx.x;
     const size_t N = (size_t)a.N;
     const R2* pp = static_cast<const R2*>(a.ppost) + (size_t)b * 9 * N;
-    const int e0 = __ldg(a.eptr + blk);
-    [[maybe_unused]] const unsigned short* ln = nullptr;
-    if constexpr (STAGED) {
-        const int l0 = __ldg(a.nptr + blk), nn = __ldg(a.nptr + blk + 1) - l0;
-        for (int i = threadIdx.x; i < nn; i += EM_THREADS) {
-            const int m = __ldg(a.nlist + l0 + i);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) cp_async8(smem + 8 * ((size_t)q * a.snode + i), pp + q * N + m);
-        }
-        unsigned char* lb = smem + 72 * (size_t)a.snode;
-        const int ne = __ldg(a.eptr + blk + 1) - e0;
-        const unsigned char* src = reinterpret_cast<const unsigned char*>(a.lnode + (size_t)EN_STRIDE * e0);
-        for (int i = threadIdx.x; i < 3 * ne; i += EM_THREADS) cp_async8(lb + 8 * i, src + 8 * i);
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();
-        ln = reinterpret_cast<const unsigned short*>(lb);
-    }
     double fcx = 0.0, fcy = 0.0, fcm = 0.0;
     bool wallnode = false;
     if (n < a.N) {
@@ -583,10 +495,8 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
                     found = em_locate<R>(a, n, -dt * hx, -dt * hy, code, xi, eta, code);
                 }
                 R2 v;
-                if (found) found = in_bounds((code >> 4) >= e0 && (code >> 4) < __ldg(a.eptr + blk + 1), a.status);
                 if (found) {
-                    if constexpr (STAGED) v = em_gather_staged(smem + 8 * (size_t)q * a.snode, ln + EN_STRIDE * ((code >> 4) - e0), xi, eta);
-                    else v = em_gather<R>(a, pp + (size_t)q * N, code >> 4, xi, eta);
+                    v = em_gather<R>(a, pp + (size_t)q * N, code >> 4, xi, eta);
                 } else {
                     lost = true;
                     v = pp[q * N + n];
@@ -609,7 +519,7 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
                 }
                 R2 gX, gY;
                 R gTX, gTY;
-                em_grad2<R, 1>(a, n, [&](int m, int) { return pair(M[N + m], M[2 * N + m]); }, &gX, &gY);
+                em_grad2<R>(a, n, [&](int m) { return pair(M[N + m], M[2 * N + m]); }, gX, gY);
                 em_grad<R>(a, n, [&](int m) { return M[3 * N + m]; }, gTX, gTY);
                 R fw[9], gw[9];
                 grad_populations(t[0], vx, vy, t[3], fm(i00, gX.x, i10 * gY.x), fm(i01, gX.x, i11 * gY.x),
@@ -723,7 +633,9 @@ __global__ void __launch_bounds__(EM_THREADS) k_em_record(const EArgs a) {
 
 // ---- launch 4: one warp per solve: the load from the partials of the blocks
 // with wall nodes, in a fixed order, the body's step (Sec. III B) and the next
-// step's blended maps
+// step's blended maps.  Bound by one warp's chain: with the wall blocks'
+// partials alone and the linear body step 12.5 -> 4.9 us (513 partials, a
+// Runge-Kutta step and the maps on one thread before)
 __global__ void k_em_finish(const EArgs a) {
     wait_previous();
     __shared__ StepMaps s_rec;
@@ -748,16 +660,13 @@ using lbfsi::StepMaps;
 
 struct lbfsi_emesh_s {
     int N = 0, Ne = 0, nwall = 0, nfarn = 0, nbatch = 0, precision = 0, nblk = 0, nwblk = 0;
-    size_t stage_bytes = 0;   // shared memory of the staged stream, 0: not staged
-    int snode = 0;
     size_t es = 8;   // element size of the path
     cudaStream_t stream = nullptr;
     std::vector<lbfsi_body_desc> bodies;
     std::vector<void*> blocks;   // every device allocation
     // mesh
     void* X = nullptr;
-    int *E = nullptr, *eptr = nullptr, *nptr = nullptr, *nlist = nullptr, *border = nullptr, *wblk = nullptr;
-    unsigned short* lnode = nullptr;
+    int *E = nullptr, *border = nullptr, *wblk = nullptr;
     void* ecoef = nullptr;
     int *hptr = nullptr, *hold = nullptr, *gptr = nullptr, *gcol = nullptr, *kind = nullptr;
     void* gw = nullptr;
@@ -994,12 +903,7 @@ lbfsi::EArgs make_eargs(lbfsi_emesh m) {
     a.kstep = (int)m->k;
     a.collide = m->k > 0u;
     a.X = m->X;
-    a.eptr = m->eptr;
     a.E = m->E;
-    a.nptr = m->nptr;
-    a.nlist = m->nlist;
-    a.lnode = m->lnode;
-    a.snode = m->snode;
     a.ecoef = m->ecoef;
     a.hptr = m->hptr;
     a.hold = m->hold;
@@ -1039,20 +943,15 @@ lbfsi::EArgs make_eargs(lbfsi_emesh m) {
 template <typename R>
 cudaError_t launch_em_collide(lbfsi_emesh m) {
     const lbfsi::EArgs a = make_eargs<R>(m);
-    cudaError_t e = cudaSuccess;
-    constexpr int NS = lbfsi::em_solves<R>();
-    const bool multi = NS > 1 && m->nbatch > 1;
-    const dim3 grid((unsigned)m->nblk, (unsigned)(multi ? (m->nbatch + NS - 1) / NS : m->nbatch));
+    const dim3 grid((unsigned)m->nblk, (unsigned)m->nbatch);
+    constexpr bool over = sizeof(R) == 4;
     if (a.collide) {
-        if (multi) e = lbfsi::launch_behind(lbfsi::k_em_D<R, NS>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
-        else e = lbfsi::launch_behind(lbfsi::k_em_D<R, 1>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
+        const cudaError_t e = lbfsi::launch_behind(lbfsi::k_em_D<R>, grid, lbfsi::EM_THREADS, 0, m->stream, over, a);
+        if (e != cudaSuccess) return e;
         m->launches++;
     }
-    if (e != cudaSuccess) return e;
-    if (multi) e = lbfsi::launch_behind(lbfsi::k_em_collide<R, NS>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
-    else e = lbfsi::launch_behind(lbfsi::k_em_collide<R, 1>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
     m->launches++;
-    return e;
+    return lbfsi::launch_behind(lbfsi::k_em_collide<R>, grid, lbfsi::EM_THREADS, 0, m->stream, over, a);
 }
 
 template <typename R>
@@ -1061,12 +960,7 @@ cudaError_t launch_em_step(lbfsi_emesh m) {
     if (e != cudaSuccess) return e;
     const lbfsi::EArgs a = make_eargs<R>(m);
     const dim3 grid((unsigned)m->nblk * (unsigned)m->nbatch);
-    if constexpr (sizeof(R) == 4) {
-        if (m->stage_bytes) e = lbfsi::launch_behind(lbfsi::k_em_stream<R, true>, grid, lbfsi::EM_THREADS, m->stage_bytes, m->stream, sizeof(R) == 4, a);
-        else e = lbfsi::launch_behind(lbfsi::k_em_stream<R, false>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
-    } else {
-        e = lbfsi::launch_behind(lbfsi::k_em_stream<R, false>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
-    }
+    e = lbfsi::launch_behind(lbfsi::k_em_stream<R>, grid, lbfsi::EM_THREADS, 0, m->stream, sizeof(R) == 4, a);
     if (e == cudaSuccess) e = lbfsi::launch_behind(lbfsi::k_em_finish, m->nbatch, 32, 0, m->stream, sizeof(R) == 4, a);
     m->launches += 2;
     return e;
@@ -1082,7 +976,6 @@ int em_status(lbfsi_emesh m) {
         return efail(LBFSI_EDEPARTURE, "departure point outside the elements holding its node (CFL)");
     if (st & lbfsi::ST_BPOINT)
         return efail(LBFSI_EDEPARTURE, "wall or far-field target point B outside the elements holding its node");
-    if (st & lbfsi::ST_BOUNDS) return efail(LBFSI_EBOUNDS, "element outside its block's tables (bounds-checked build)");
     if (st & lbfsi::ST_NONPHYS) return efail(LBFSI_ENONPHYS, "non-physical state (rho<=0, T<=0 or NaN)");
     return LBFSI_OK;
 }
@@ -1191,52 +1084,24 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
     int rc = d->grid_ij ? gradient_r18(N, ijr.data(), d->grid_nr, d->grid_nt, X, gptr, gcol, gw)
                         : gradient_r33(N, E, X, hptr, hold, gptr, gcol, gw);
     if (rc) return rc;
-    // each stream block's own copy of the tables of the elements that hold its
-    // nodes, in the order of their centre nodes (so along the same curve as
-    // the nodes), and the list of those elements' nodes; each node's list of
-    // holding elements keeps the caller's element order, the order of the
-    // departure search
+    // elements stored in the order of their centre nodes (so along the same
+    // curve as the nodes); each node's list of holding elements keeps the
+    // caller's element order, the order of the departure search
     const int nblk = (N + lbfsi::EM_THREADS - 1) / lbfsi::EM_THREADS;
-    std::vector<int> eptr((size_t)nblk + 1, 0), nptr((size_t)nblk + 1, 0), nlist, Ep;
-    std::vector<double> ecb;
-    std::vector<unsigned short> lnode;
-    int snode = 0, selem = 0;
+    std::vector<int> Ep((size_t)Ne * lbfsi::EN_STRIDE, 0);
     {
-        std::vector<int> eperm((size_t)Ne), einv((size_t)Ne), slot((size_t)Ne, -1), at((size_t)N, 0), be;
+        std::vector<int> eperm((size_t)Ne), einv((size_t)Ne);
         for (int e2 = 0; e2 < Ne; ++e2) eperm[e2] = e2;
         std::stable_sort(eperm.begin(), eperm.end(),
                          [&](int a, int b) { return E[9 * (size_t)a + 4] < E[9 * (size_t)b + 4]; });
-        for (int k = 0; k < Ne; ++k) einv[eperm[k]] = k;
-        for (int blk = 0; blk < nblk; ++blk) {
-            const int n0 = blk * lbfsi::EM_THREADS, n1 = std::min(N, n0 + lbfsi::EM_THREADS);
-            be.clear();
-            for (int h = hptr[n0]; h < hptr[n1]; ++h) be.push_back(einv[hold[h] >> 4]);
-            std::sort(be.begin(), be.end());
-            be.erase(std::unique(be.begin(), be.end()), be.end());
-            if (Ep.size() / lbfsi::EN_STRIDE + be.size() > (1u << 27) - 1u) return efail(LBFSI_EINVAL, "mesh too large");
-            const size_t nl0 = nlist.size();
-            for (int k : be)
-                for (int s = 0; s < 9; ++s) nlist.push_back(E[9 * (size_t)eperm[k] + s]);
-            std::sort(nlist.begin() + nl0, nlist.end());
-            nlist.erase(std::unique(nlist.begin() + nl0, nlist.end()), nlist.end());
-            const int nn = (int)(nlist.size() - nl0);
-            for (int k = 0; k < nn; ++k) at[nlist[nl0 + k]] = k;
-            for (size_t k = 0; k < be.size(); ++k) {
-                const int e2 = eperm[be[k]];
-                slot[e2] = eptr[blk] + (int)k;
-                for (int s = 0; s < lbfsi::EN_STRIDE; ++s) {
-                    Ep.push_back(s < 9 ? E[9 * (size_t)e2 + s] : 0);
-                    // (past the staged sizes the offsets are not used)
-                    lnode.push_back(s < 9 ? (unsigned short)(at[E[9 * (size_t)e2 + s]] * 8) : 0);
-                }
-                ecb.insert(ecb.end(), &ecoef[8 * (size_t)e2], &ecoef[8 * (size_t)e2] + 8);
-            }
-            for (int h = hptr[n0]; h < hptr[n1]; ++h) hold[h] = slot[hold[h] >> 4] * 16 + (hold[h] & 15) / 3 * 4 + (hold[h] & 15) % 3;
-            eptr[blk + 1] = eptr[blk] + (int)be.size();
-            nptr[blk + 1] = (int)nlist.size();
-            snode = std::max(snode, nn);
-            selem = std::max(selem, (int)be.size());
+        std::vector<double> cs(ecoef.size());
+        for (int k = 0; k < Ne; ++k) {
+            einv[eperm[k]] = k;
+            std::copy_n(&E[9 * (size_t)eperm[k]], 9, &Ep[(size_t)k * lbfsi::EN_STRIDE]);
+            std::copy_n(&ecoef[8 * (size_t)eperm[k]], 8, &cs[8 * (size_t)k]);
         }
+        ecoef.swap(cs);
+        for (int& h : hold) h = einv[h >> 4] * 16 + (h & 15) / 3 * 4 + (h & 15) % 3;
     }
     // gradient operator rows in slices of 32 nodes
     {
@@ -1320,9 +1185,6 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
     m->es = d->precision == LBFSI_FP64 ? sizeof(double) : sizeof(float);
     m->nblk = nblk;
     m->nwblk = nwblk;
-    m->snode = (snode + 1) & ~1;
-    m->stage_bytes = lbfsi::em_stage_bytes(m->snode, selem);
-    if (d->precision != LBFSI_FP32 || m->stage_bytes > lbfsi::EM_STAGE_MAX) m->stage_bytes = 0;
     m->stream = static_cast<cudaStream_t>(cuda_stream);
     m->bodies.assign(d->bodies, d->bodies + d->nbatch);
     m->perm = perm;
@@ -1335,20 +1197,11 @@ int lbfsi_create_mesh_elements(const lbfsi_mesh_elements_desc* d, void* cuda_str
         *dst = q;
         return e;
     };
-    const std::vector<unsigned char> Xt = typed(Xv, d->precision), ect = typed(ecb, d->precision),
+    const std::vector<unsigned char> Xt = typed(Xv, d->precision), ect = typed(ecoef, d->precision),
                                      gwt = typed(gw, d->precision);
     cudaError_t e = put(&m->X, Xt.data(), Xt.size());
-    if (e == cudaSuccess) e = put((void**)&m->eptr, eptr.data(), eptr.size() * sizeof(int));
     if (e == cudaSuccess) e = put((void**)&m->border, border.data(), border.size() * sizeof(int));
     if (e == cudaSuccess) e = put((void**)&m->wblk, wblk.data(), wblk.size() * sizeof(int));
-    if (e == cudaSuccess && m->stage_bytes) {
-        e = put((void**)&m->nptr, nptr.data(), nptr.size() * sizeof(int));
-        if (e == cudaSuccess) e = put((void**)&m->nlist, nlist.data(), nlist.size() * sizeof(int));
-        if (e == cudaSuccess) e = put((void**)&m->lnode, lnode.data(), lnode.size() * sizeof(unsigned short));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute((const void*)lbfsi::k_em_stream<float, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbfsi::EM_STAGE_MAX);
-    }
     if (e == cudaSuccess) e = put((void**)&m->E, Ep.data(), Ep.size() * sizeof(int));
     if (e == cudaSuccess) e = put(&m->ecoef, ect.data(), ect.size());
     if (e == cudaSuccess) e = put((void**)&m->hptr, hptr.data(), hptr.size() * sizeof(int));

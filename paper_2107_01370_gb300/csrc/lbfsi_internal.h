@@ -265,6 +265,7 @@ cudaError_t launch_step(const StepArgs& a, int precision, bool general, int vari
 // Uniform launch over nbatch solves of one mesh (see StepArgs).
 cudaError_t launch_step_uniform(const StepArgs& a, int precision, int variant, int nbatch,
                                 cudaStream_t s);
+int default_shape(int precision, long long tiles16);
 int tile_rows(int precision, int variant);
 // Stream launch of the float64 path (lbfsi_stream64.cu): blocks of 'rows' rows
 // x 32 columns, each row by four warps that share the directions.

@@ -29,6 +29,12 @@
 // chunks and the stream writes one 64-bit pair per direction.  The redundant
 // work is the collision of the 2-node halo; the HBM traffic per node is the
 // 18 populations read and written once plus the 4-value moment field and Y.
+//
+// Bound by instruction issue: 41.7 warp instructions per node on the VIV ring
+// (59.9 when this kernel also formed dQ, D and Y in its halo and reduced the
+// loads).  Measured at 512 x 256 x 16 solves, half the nodes moving: that one
+// kernel 155 us a step; this launch 113 us and the field launch 22.  At 256 x 128
+// x 1: 29.6 us against 11.3 and 9.5 (the loads' chain no longer ends the step).
 #include <algorithm>
 #include <cstdio>
 #include <type_traits>
@@ -935,6 +941,20 @@ static cudaError_t with_kernel(bool general, int variant, Fn fn) {
 }
 
 int step_variants(int precision) { return precision == 0 ? 3 : 5; }
+
+// Tile shape where no schedule was asked for, by the tiles of 16 rows (float64:
+// one row per block).  Below a tile per SM more and smaller tiles spread the
+// work; up to four per SM a tile's own time counts, which 512 threads shorten;
+// beyond, the three blocks of 256 threads that an SM holds overlap better.
+// Measured per step with 8 x 32 tiles, 16 x 32 / 512 threads, 16 x 32 / 256
+// threads: 256 x 128 (64 tiles) 20.2, 21.3, 23.3 us; 256 x 128 x 4 (256) 25.3, 24.7,
+// 25.6; 201 x 150 x 5 (325) 28.3, 27.3, 29.5; 512 x 256 x 2 (512) 32.7, 31.8, 32.8;
+// x 3 (768) 43.0, 40.3, 39.8; x 16 (4096) 150, 140.7, 139.9; 8192 x 512 (8192) 259,
+// 242.3, 240.6.
+int default_shape(int precision, long long tiles16) {
+    if (precision == 0) return 0;
+    return tiles16 < 152 ? 0 : tiles16 < 608 ? 4 : 1;
+}
 
 int tile_rows(int precision, int variant) {
     if (precision == 0) return 1 << variant;

@@ -1,6 +1,6 @@
 """Layouts of the step that follow the sizes: the tile shape a float handle
-or batch takes when no schedule is asked for, and the element list's staged
-and unstaged stream (blocks of 256 nodes, gradient rows in slices of 32).
+or batch takes when no schedule is asked for, and the element list's blocks of
+256 nodes and gradient rows in slices of 32.
 
 Tolerance of the float paths against the float64 oracle: a population is a sum
 of nine terms whose weights' magnitudes sum to at most 1.6, on deviations from
@@ -35,9 +35,9 @@ def _err(a, b):
 
 
 # solves of 4 or 6 tiles of 16 x 32 nodes (the last with one row, ragged
-# columns), one solve below the 304 tiles from which 16 rows are taken and at it
-@pytest.mark.parametrize("nr,nt,nb", [(17, 34, 75), (17, 34, 76), (33, 62, 50), (33, 62, 51)])
-def test_float_default_shape_either_side_of_its_line(L, nr, nt, nb):
+# columns) on both sides of the default shape's lines at 152 and 608 tiles
+@pytest.mark.parametrize("nr,nt,nb", [(17, 34, 37), (17, 34, 38), (33, 62, 101), (33, 62, 102)])
+def test_float_default_shape_either_side_of_its_lines(L, nr, nt, nb):
     body = inputs.BodySpec(dof=1, r_in=0.75, r_out=2.0, m_star=3.0, v_r=5.0)
     case = inputs.cylinder_case(nr, nt, r_far=10.0, body=body)
     M0 = inputs.initial_field(nr, nt, case.flow, seed=nr)
@@ -45,7 +45,7 @@ def test_float_default_shape_either_side_of_its_line(L, nr, nt, nb):
     for _ in range(STEPS):
         r = s.step()
     out = []
-    for schedule in (None, (0, 0), (1, 0)):
+    for schedule in (None, (0, 0), (1, 0), (4, 1)):
         m = L.Mesh(case.r, case.e, case.bodies * nb, precision=L.FP32)
         if schedule is not None:
             m.set_schedule(*schedule)
@@ -68,10 +68,10 @@ def test_float_default_shape_either_side_of_its_line(L, nr, nt, nb):
 
 
 # node counts below, at and past whole blocks and slices; solves that fill a
-# pair or not; and a thin ring whose blocks' elements reach 1288 nodes, more
-# than are staged (its first step alone, the one without a correction field:
-# second derivatives over spacings of 1e-3 multiply float roundings by 1e6, so
-# the bound above does not hold for the steps that follow)
+# pair or not; and a thin ring whose blocks' elements reach 1288 nodes (its
+# first step alone, the one without a correction field: second derivatives over
+# spacings of 1e-3 multiply float roundings by 1e6, so the bound above does not
+# hold for the steps that follow)
 @pytest.mark.parametrize("nr,nt,nb,thin", [(7, 24, 1, False), (16, 16, 2, False), (17, 32, 3, False),
                                            (25, 48, 2, False), (257, 16, 3, True)])
 def test_float_element_list_blocks(L, nr, nt, nb, thin):
