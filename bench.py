@@ -5,7 +5,8 @@ Re 100, Ma 0.2) on an O-grid of 512 radial x 256 angular nodes deformed by the
 blending polynomial, FP32 populations with FP64 loads, RK4 and blend
 displacement; a batch of independent solves per GPU (default 16, a
 302 MB ping-pong population set, larger than the 129 MB L2).  A step is one
-coupled time step of every solve of the batch: one launch of the fused kernel.
+coupled time step of every solve of the batch: the step launch and the field
+launch behind it.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--batch B]
   python bench.py --impl reference ...   (the FP64 oracle on the host cores)
@@ -43,7 +44,7 @@ from paper_2107_01370_gb300 import inputs, replicas  # noqa: E402
 METRIC = "fused-step MLUPS"
 UNIT = "MLUPS"
 BYTES_PER_NODE_FP32 = 144   # 18 populations read + 18 written, 4 bytes each
-KERNEL = "k_step<float>"
+KERNEL = "k_step<float> + k_fields<float> (the two launches of a step)"
 
 
 def workload_name(batch):
@@ -51,9 +52,10 @@ def workload_name(batch):
             f"Re 100, Ma 0.2, FP32 populations / FP64 loads+RK4; batch of {batch} solves per GPU")
 
 
-# The sources the step kernel is compiled from (a profile taken on them stays
+# The sources the step's kernels are compiled from (a profile taken on them stays
 # valid while they are unchanged).
-KERNEL_SOURCES = ("lbfsi_device.cuh", "lbfsi_internal.h", "lbfsi_step.cu")
+KERNEL_SOURCES = ("lbfsi_device.cuh", "lbfsi_internal.h", "lbfsi_stencil.cuh", "lbfsi_departure.cuh",
+                  "lbfsi_record.cuh", "lbfsi_step.cu", "lbfsi_fields.cu")
 
 
 def source_sha():
@@ -73,7 +75,7 @@ def measured_peaks():
 
 
 def traffic_per_node():
-    """DRAM bytes per node update of the step kernel from the committed ncu
+    """DRAM bytes per node update of a step's two launches from the committed ncu
     summary, if it was taken on the current kernel source."""
     p = os.path.join(ROOT, "profiles", "k_step_fp32_traffic.json")
     if not os.path.exists(p):
@@ -317,7 +319,7 @@ def small_case_graphs(stream, steps=1000, graph_steps=100):
     for label, g in (("plain", 0), ("graph", graph_steps)):
         m = lbfsi.Mesh(case.r, case.e, case.bodies, precision=lbfsi.FP64, stream=stream.cuda_stream)
         m.init_fields(case.flow, M0[None])
-        # the tile shape (8, 4 or 2 rows: few tiles leave SMs idle) by the tuner
+        # the tile shape (1, 2 or 4 rows per CTA) by the tuner
         v, o, _ = m.autotune(20)
         res["schedule"] = {"variant": v, "order": o}
         m.set_graph_steps(g)
@@ -376,9 +378,8 @@ def general_mesh_cases():
 def general_mesh_throughput(stream, peak, steps=200, warmup=5, batch=(8, 8, 1, 6), only=None):
     """MLUPS of the general-mesh step (Newton departure points, cached for
     the nodes no blend moves; stored metric) on the workloads of
-    general_mesh_cases, timed with CUDA events on the library's stream; the
-    C-grid step is two launches (the collision of the rows next to the cut,
-    then the step).  HBM fraction against the algorithmic 144 B per node
+    general_mesh_cases, timed with CUDA events on the library's stream.
+    HBM fraction against the algorithmic 144 B per node
     update."""
     import torch
     from paper_2107_01370_gb300 import lbfsi
@@ -462,7 +463,7 @@ def element_mesh_throughput(stream, peak, steps=100, warmup=5, batch=8):
 
 
 def issue_roofline(nodes, kernel_s, sm_mhz):
-    """Instruction-issue ceiling of the step kernel: warp instructions per
+    """Instruction-issue ceiling of a step's two launches: warp instructions per
     node from the committed ncu capture (current source only) against one
     warp instruction per scheduler per cycle (152 SMs x 4 schedulers)."""
     p = os.path.join(ROOT, "profiles", "k_step_fp32_traffic.json")
