@@ -470,12 +470,13 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
             // moments summed as the populations come (no array of them: one
             // copy of the solve for the nine directions)
             R rho = R(0), jx = R(0), jy = R(0), s2 = R(0);
-            auto put = [&](int q, R cx, R cy, R2 v) {
+            // (float: summed over the deviations d from the free stream's)
+            auto put = [&](int q, R cx, R cy, R2 v, R2 d) {
                 po[q * N + n] = v;
-                rho += v.x;
-                jx = fm(cx, v.x, jx);
-                jy = fm(cy, v.x, jy);
-                s2 += v.y;
+                rho += d.x;
+                jx = fm(cx, d.x, jx);
+                jy = fm(cy, d.x, jy);
+                s2 += d.y;
             };
             bool lost = false;
 #pragma unroll 1
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
                     lost = true;
                     v = pp[q * N + n];
                 }
-                put(q, cx, cy, padd(v, ref_pair<R>(fl, q)));
+                put(q, cx, cy, padd(v, ref_pair<R>(fl, q)), v);
             }
             if (lost) atomicOr(a.status, ST_DEPARTURE);
             if (missing) {
@@ -528,7 +529,13 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
                                  flowv<R>(fl, fl.iCv, fl.iCv_f), flowv<R>(fl, fl.iPr, fl.iPr_f), fw, gw);
 #pragma unroll
                 for (int q = 0; q < 9; ++q)
-                    if (missing & (1u << q)) put(q, (R)cxq(q), (R)cyq(q), pair(fw[q], gw[q]));
+                    if (missing & (1u << q)) put(q, (R)cxq(q), (R)cyq(q), pair(fw[q], gw[q]), psub(pair(fw[q], gw[q]), ref_pair<R>(fl, q)));
+            }
+            if constexpr (sizeof(R) == 4) {
+                rho += fl.mref[0];
+                jx += fl.mref[1];
+                jy += fl.mref[2];
+                s2 += fl.mref[3];
             }
             const R ir = rcp_(rho), ux = jx * ir, uy = jy * ir;
             const R T = fm(R(-0.5), fm(ux, ux, uy * uy), R(0.5) * s2 * ir) * flowv<R>(fl, fl.iCv, fl.iCv_f);

@@ -717,6 +717,14 @@ int fill_flow(const lbfsi_flow_params& p, SolveDev& s) {
         s.fgref[2 * q] = (float)fr[q];
         s.fgref[2 * q + 1] = (float)gr[q];
     }
+    double mr[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int q = 0; q < 9; ++q) {
+        mr[0] += s.fgref[2 * q];
+        mr[1] += cxq(q) * (double)s.fgref[2 * q];
+        mr[2] += cyq(q) * (double)s.fgref[2 * q];
+        mr[3] += s.fgref[2 * q + 1];
+    }
+    for (int c = 0; c < 4; ++c) s.mref[c] = (float)mr[c];
     return LBFSI_OK;
 }
 

@@ -149,6 +149,7 @@ struct SolveDev {
     // every step at a node that does not move) scales with the deviation, not
     // with the population
     float fgref[18];
+    float mref[4];   // its moments: rho, rho u_x, rho u_y, 2 rho E
     void* p[2];                    // populations, (f_q, g_q) pairs [9][N]
     void* M[2];                    // moments [4][N]
     StepMaps* maps[2];             // [nbody] each

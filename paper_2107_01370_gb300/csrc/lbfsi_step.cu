@@ -678,14 +678,17 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
         // population q of the node: written as it is found, its share added to
         // the moments (in the order of q on every path)
         R rho = R(0), jx = R(0), jy = R(0), s2 = R(0);
-        auto put = [&](int q, R2 v) {
+        // v: the population, d: its deviation from the free stream's.  The moments
+        // are summed over the deviations (nine small numbers), which keeps their
+        // rounding to that of the last addition
+        auto put = [&](int q, R2 v, R2 d) {
             p_out[(size_t)q * N + n] = v;
             if (dup2) p_out[(ptrdiff_t)q * N + n2] = v;
-            rho += v.x;
-            s2 += v.y;
+            rho += d.x;
+            s2 += d.y;
             const int cx = cxq(q), cy = cyq(q);
-            if (cx) jx += cx > 0 ? v.x : -v.x;
-            if (cy) jy += cy > 0 ? v.x : -v.x;
+            if (cx) jx += cx > 0 ? d.x : -d.x;
+            if (cy) jy += cy > 0 ? d.x : -d.x;
         };
         R jn[4] = {R(0), R(0), R(0), R(0)};
         // departure solve of this node for a displacement (dx, dy): the window's
@@ -751,12 +754,12 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
                     lagrange3(xe[q].y, Ly);
                     v = gather9(sp + q * T::PSS + base, T::PWS, Lx, Ly);
                 }
-                put(q, add_ref(q, v));
+                put(q, add_ref(q, v), v);
             }
         } else if (!GEN && !moved && i > 0) {
             // a node the blend does not move: c_hat = c, and the rest
             // population's departure point is the node itself
-            put(0, add_ref(0, sp[own]));
+            put(0, add_ref(0, sp[own]), sp[own]);
             auto pull = [&](auto cxc, auto cyc, int q) {
                 int wa, wb;
                 R xi, eta;
@@ -772,7 +775,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
                     lost = true;
                     v = sp[q * T::PSS + own];
                 }
-                put(q, add_ref(q, v));
+                put(q, add_ref(q, v), v);
             };
             using P1 = std::integral_constant<int, 1>;
             using Z0 = std::integral_constant<int, 0>;
@@ -791,7 +794,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
 #pragma unroll 1
             for (int q = 0; q < 9; ++q) {
                 if (missing & (1u << q)) {
-                    put(q, s_wall(q, tj));   // Grad's approximation
+                    put(q, s_wall(q, tj), psub(s_wall(q, tj), ref_of(q)));   // Grad's approximation
                     continue;
                 }
                 const R cx = (R)cxq(q), cy = (R)cyq(q);
@@ -812,10 +815,14 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
                     lost = true;
                     v = sp[q * T::PSS + own];
                 }
-                put(q, add_ref(q, v));
+                put(q, add_ref(q, v), v);
             }
         }
         if (lost) atomicOr(a.status, ST_DEPARTURE);
+        rho += SD(mref)[0];
+        jx += SD(mref)[1];
+        jy += SD(mref)[2];
+        s2 += SD(mref)[3];
         const R ir = rcp_(rho), ux = jx * ir, uy = jy * ir;
         const R Tn = fm(R(-0.5), fm(ux, ux, uy * uy), R(0.5) * s2 * ir) * iCv;
         if (!(rho > R(0)) || !(Tn > R(0)) || !isfinite(ux) || !isfinite(uy)) atomicOr(a.status, ST_NONPHYS);
