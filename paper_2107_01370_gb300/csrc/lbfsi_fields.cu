@@ -283,9 +283,9 @@ __device__ __forceinline__ void fields_march(const SolveDev& S, const MeshDev& G
         const float4 r = sR[k];
         return make_float4(r.y * c0, -r.z * c1, -r.y * c2, r.z * c3);
     };
-    // derivative along j (one-sided on a C-grid's outlet columns and at a
-    // row-0 junction)
-    const bool edge = cg && (sx == 0 || sx == nsx - 1);
+    // derivative along j (one-sided on a C-grid's outlet columns, which a strip
+    // may hold in its halo alone, and at a row-0 junction)
+    const bool edge = cg && (sx == 0 || sx * W - H + 31 >= nt - 1);
     auto dj = [&](float v, bool row0) -> float {
         const float up = __shfl_down_sync(FULL, v, 1), dn = __shfl_up_sync(FULL, v, 1);
         float d = 0.5f * (up - dn);
