@@ -651,29 +651,56 @@ BodyDev body_dev(const lbfsi_body_desc& d, double rho, double U) {
     return b;
 }
 
-// The RK4 map's columns: the step applied to unit states, loads and
-// accelerations (the step is linear and maps zero to zero).
+// The columns of the RK4 step's increment: the increment for unit states, loads
+// and accelerations (it is linear and maps zero to zero).
 BodyProp body_prop(const BodyDev& b, double dt) {
     BodyProp p{};
-    const long long never_forced = 1ll << 60;
+    const double det = b.m * b.i_a - b.s_a * b.s_a;
     for (int c = 0; c < 6; ++c) {
-        const double e[6] = {c == 0 ? 1.0 : 0.0, c == 1 ? 1.0 : 0.0, c == 2 ? 1.0 : 0.0,
-                             c == 3 ? 1.0 : 0.0, c == 4 ? 1.0 : 0.0, c == 5 ? 1.0 : 0.0};
-        const BodyStateDev s = rk4_body(b, BodyStateDev{e[0], e[1], e[2], e[3]}, e[4], e[5], dt, never_forced);
-        p.free[0][c] = s.h;
-        p.free[1][c] = s.alpha;
-        p.free[2][c] = s.hdot;
-        p.free[3][c] = s.adot;
-        if (b.dof != 2) continue;
-        // m h'' + S_alpha alpha''(t) + k_h h = F_y with alpha'' prescribed
-        auto acc = [&](double a, double h) { return (e[2] - b.k_h * h - b.s_a * a) / b.m; };
-        const double h0 = e[0], v0 = e[1];
-        const double k1h = v0, k1v = acc(e[3], h0);
-        const double k2h = v0 + 0.5 * dt * k1v, k2v = acc(e[4], h0 + 0.5 * dt * k1h);
-        const double k3h = v0 + 0.5 * dt * k2v, k3v = acc(e[4], h0 + 0.5 * dt * k2h);
-        const double k4h = v0 + dt * k3v, k4v = acc(e[5], h0 + dt * k3h);
-        p.forced[0][c] = h0 + dt / 6.0 * (k1h + 2.0 * k2h + 2.0 * k3h + k4h);
-        p.forced[1][c] = v0 + dt / 6.0 * (k1v + 2.0 * k2v + 2.0 * k3v + k4v);
+        double e[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        e[c] = 1.0;
+        // RK4 of (h, alpha, hdot, adot) under accelerations acc(stage, h, alpha, hdot) -> (h'', alpha'')
+        auto increment = [&](auto acc, double* out) {
+            double k[4][4], sum[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int s = 0; s < 4; ++s) {
+                const double f = s == 0 ? 0.0 : s == 3 ? dt : 0.5 * dt, w = s == 0 || s == 3 ? 1.0 : 2.0;
+                double y[4];
+                for (int r = 0; r < 4; ++r) y[r] = e[r] + (s ? f * k[s - 1][r] : 0.0);
+                k[s][0] = y[2];
+                k[s][1] = y[3];
+                acc(s, y, k[s] + 2);
+                for (int r = 0; r < 4; ++r) sum[r] += w * k[s][r];
+            }
+            for (int r = 0; r < 4; ++r) out[r] = dt / 6.0 * sum[r];
+        };
+        double d[4];
+        if (b.dof == 1) {
+            increment([&](int, const double* y, double* a) {
+                a[0] = (e[4] - b.k * y[0] - b.c * y[2]) / b.m;
+                a[1] = 0.0;
+            }, d);
+            p.free[0][c] = d[0];
+            p.free[2][c] = d[2];
+        } else if (b.dof == 2) {
+            increment([&](int, const double* y, double* a) {
+                const double r0 = e[4] - b.k_h * y[0], r1 = e[5] - b.k_a * y[1];
+                a[0] = (b.i_a * r0 - b.s_a * r1) / det;
+                a[1] = (b.m * r1 - b.s_a * r0) / det;
+            }, d);
+            for (int r = 0; r < 4; ++r) p.free[r][c] = d[r];
+            // m h'' + S_alpha alpha''(t) + k_h h = F_y with alpha'' prescribed: the
+            // columns are h, hdot, F_y and alpha'' at the step's start, middle and end
+            const double u[6] = {e[0], e[1], e[2], e[3], e[4], e[5]};
+            e[0] = u[0];
+            e[1] = e[3] = 0.0;
+            e[2] = u[1];
+            increment([&](int s, const double* y, double* a) {
+                a[0] = (u[2] - b.k_h * y[0] - b.s_a * (s == 0 ? u[3] : s == 3 ? u[5] : u[4])) / b.m;
+                a[1] = 0.0;
+            }, d);
+            p.forced[0][c] = d[0];
+            p.forced[1][c] = d[2];
+        }
     }
     return p;
 }

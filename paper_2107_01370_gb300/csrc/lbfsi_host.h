@@ -96,7 +96,7 @@ int validate_bodies(const HostMesh& m, const lbfsi_body_desc* bodies, int n);
 
 // Dimensional ODE coefficients from the nondimensional groups.
 BodyDev body_dev(const lbfsi_body_desc& d, double rho, double U);
-// Its RK4 step over dt as a linear map.
+// The increment of its RK4 step over dt as a linear map.
 BodyProp body_prop(const BodyDev& b, double dt);
 
 // Validate flow parameters and fill the flow fields of a solve descriptor.

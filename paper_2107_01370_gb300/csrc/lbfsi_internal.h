@@ -33,10 +33,13 @@ struct BodyStateDev {
     double h, alpha, hdot, adot;
 };
 
-// One RK4 step of a body over the flow's dt under a held load (Sec. III B) as
-// the linear map it is: row r of free gives state entry r from (h, alpha, hdot,
-// adot, F_y, M); forced gives (h, hdot) of a step in the forcing interval from
-// (h, hdot, F_y, alpha'' at the step's start, middle and end).
+// The increment of one RK4 step of a body over the flow's dt under a held load
+// (Sec. III B) as the linear map it is: row r of free gives that of state entry r
+// from (h, alpha, hdot, adot, F_y, M); forced gives those of (h, hdot) of a step
+// in the forcing interval from (h, hdot, F_y, alpha'' at the step's start, middle
+// and end).  The increment, not the state: it is some hundredths of the state, so
+// the state's own rounding is the addition's alone (as a whole map its products
+// rounded it again, and 1 / dt carries that into the mesh velocity).
 struct BodyProp {
     double free[4][6], forced[2][6];
 };

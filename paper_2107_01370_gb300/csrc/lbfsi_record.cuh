@@ -22,12 +22,13 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Lane r of a body's group of four: its part of state entry r (h, alpha,
-// hdot, adot) that does not depend on the loads, and the weights of F_y and M.
+// Lane r of a body's group of four: state entry r (h, alpha, hdot, adot) before
+// the step (zero where the new one is prescribed), the part of its increment that
+// does not depend on the loads, and the weights of F_y and M.
 struct BodyLane {
     BodyStateDev Sn;
     BodyMap<double> ms;
-    double p4, p5, y;
+    double p4, p5, y, base;
 };
 
 // The step to step kk from the record prev of the step before; whole warp.
@@ -43,7 +44,7 @@ __device__ __forceinline__ BodyLane body_lane(const BodyDev& bd, const BodyProp&
 #pragma unroll
         for (int c = 0; c < 6; ++c) pr[c] = p[c];
     }
-    double y = 0.0;   // the part of the step that does not depend on the loads
+    double y = 0.0, base = r == 0 ? Sn.h : r == 1 ? Sn.alpha : r == 2 ? Sn.hdot : Sn.adot;
     if (forced) {
         // forced pitching (Sec. IV D): alpha = amp sin(w t) prescribed, its
         // acceleration at the step's start, middle and end
@@ -57,12 +58,13 @@ __device__ __forceinline__ BodyLane body_lane(const BodyDev& bd, const BodyProp&
         if (r == 1) y = a1;
         else if (r == 3) y = ww * c1;
         else y = fm(-ww * ww, fm(pr[3], a0, fm(pr[4], ah, pr[5] * a1)), fm(pr[0], sv[0], pr[1] * sv[2]));
+        if (r & 1) base = 0.0;
         pr[4] = (r & 1) ? 0.0 : pr[2];
         pr[5] = 0.0;
     } else {
         y = fm(pr[0], sv[0], pr[1] * sv[1]) + fm(pr[2], sv[2], pr[3] * sv[3]);
     }
-    return BodyLane{Sn, prev.Sd, pr[4], pr[5], y};
+    return BodyLane{Sn, prev.Sd, pr[4], pr[5], y, base};
 }
 
 // The new states from the loads F (x, y, moment of the lane's body) and the
@@ -70,7 +72,7 @@ __device__ __forceinline__ BodyLane body_lane(const BodyDev& bd, const BodyProp&
 __device__ __forceinline__ void body_records(const BodyLane& bl, const double* F, double idt, int nb, int l,
                                              StepMaps& s_rec, StepMaps* maps, double* rec) {
     const int g4 = min(l >> 2, nb - 1) * 4, r = l & 3;
-    const double y = fm(bl.p4, F[1], fm(bl.p5, F[2], bl.y));
+    const double y = bl.base + fm(bl.p4, F[1], fm(bl.p5, F[2], bl.y));
     const BodyStateDev& Sn = bl.Sn;
     const BodyMap<double>& ms = bl.ms;
     const double h = __shfl_sync(FULL, y, g4), al = __shfl_sync(FULL, y, g4 + 1);
