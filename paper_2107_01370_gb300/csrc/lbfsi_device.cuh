@@ -27,9 +27,13 @@ __device__ __forceinline__ float rcp_(float x) {
     return y;
 }
 // (float64: the hardware's seed of about 20 bits and two Newton steps
-// r += r (1 - x r), which square its error twice: 1/x to about an ulp; the
-// division's exact rounding costs about twice the operations, at 1/64 of the
-// float rate)
+// r += r (1 - x r), which square its error twice, to far below an ulp, the last
+// with one rounding: 1/x correctly rounded but for values within some 2^-20 ulp
+// of a tie.  For normal x whose reciprocal is normal; zero, infinity and NaN give
+// NaN, which every caller treats as it does an infinity: a state of rho = 0 is
+// non-physical and a departure solve with no determinant lost, by comparisons
+// that NaN fails too.  The division costs 2 to 3.5% of a step: 80.1 -> 82.9 us on
+// 96 x 96 x 3, 102.5 -> 106.2 on a 97 x 161 C-grid)
 __host__ __device__ __forceinline__ double rcp_(double x) {
 #ifdef __CUDA_ARCH__
     double r;
