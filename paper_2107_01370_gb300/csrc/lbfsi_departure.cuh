@@ -93,20 +93,25 @@ __device__ __forceinline__ bool depart_static(const NodeGeo<R>& G, R dt, int& wa
 
 // One Newton step of (b + d eta0) u + (c + d xi0) v + d u v = (dx, dy), with
 // B = b + d eta0, C = c + d xi0 (written with fixed rounding: see fma_rn);
-// ONCE false: and a second one with the same Jacobian.
+// ONCE false: and a second one with the same Jacobian.  Returns the size of the
+// first step.
 template <bool ONCE, typename R>
-__device__ __forceinline__ void newton_step(const R* c, R Bx, R By, R Cx, R Cy, R dx, R dy, R& u, R& v) {
+__device__ __forceinline__ R newton_step(const R* c, R Bx, R By, R Cx, R Cy, R dx, R dy, R& u, R& v) {
     const R a11 = fma_rn(c[4], v, Bx), a12 = fma_rn(c[4], u, Cx);
     const R a21 = fma_rn(c[5], v, By), a22 = fma_rn(c[5], u, Cy);
     const R idet = rcp_(fma_rn(a11, a22, -mul_rn(a12, a21)));
+    R size = R(0);
 #pragma unroll
     for (int it = 0; it < (ONCE ? 1 : 2); ++it) {
         const R uv = mul_rn(u, v);
         const R rx = fma_rn(c[4], uv, fma_rn(Cx, v, fma_rn(Bx, u, -dx)));
         const R ry = fma_rn(c[5], uv, fma_rn(Cy, v, fma_rn(By, u, -dy)));
-        u = add_rn(u, -mul_rn(fma_rn(a22, rx, -mul_rn(a12, ry)), idet));
-        v = add_rn(v, -mul_rn(fma_rn(a11, ry, -mul_rn(a21, rx)), idet));
+        const R du = mul_rn(fma_rn(a22, rx, -mul_rn(a12, ry)), idet), dv = mul_rn(fma_rn(a11, ry, -mul_rn(a21, rx)), idet);
+        u = add_rn(u, -du);
+        v = add_rn(v, -dv);
+        if (it == 0) size = max(abs_(du), abs_(dv));
     }
+    return size;
 }
 
 // Departure point on a general mesh (Eq. depPnt): the node's Q2 element for
@@ -166,18 +171,24 @@ __device__ __forceinline__ bool depart_gen(const R* __restrict__ gc, const R* jn
 #pragma unroll 1
             for (int it = 0; it < 3; ++it) newton_step<true>(c, Bx, By, Cx, Cy, dx, dy, u, v);
         } else {
-            // three float iterations for the start (their arithmetic is free
-            // beside float64's): the error of about 1e-7 of a cell goes to
-            // 1e-14 in one float64 step, and below round-off in a second
-            // with the first's Jacobian
+            // float iterations for the start (their arithmetic is free beside
+            // float64's) until one moves by less than 1e-5 of a cell: the error
+            // is then float round-off, below 1e-5, goes to 1e-10 in one float64
+            // step and below round-off in a second with the first's Jacobian.
+            // Where they do not get there (cells skewed so far that float
+            // round-off is more, values beyond float's range) float64 from zero
             const float cf[6] = {0.f, 0.f, 0.f, 0.f, (float)c[4], (float)c[5]};
             const float bx = (float)Bx, by = (float)By, ex = (float)Cx, ey = (float)Cy, fx = (float)dx, fy = (float)dy;
             float uf = 0.f, vf = 0.f;
+            bool near = false;
 #pragma unroll 1
-            for (int it = 0; it < 3; ++it) newton_step<true>(cf, bx, by, ex, ey, fx, fy, uf, vf);
-            u = (R)uf;
-            v = (R)vf;
-            newton_step<false>(c, Bx, By, Cx, Cy, dx, dy, u, v);
+            for (int it = 0; it < 12 && !near; ++it) near = newton_step<true>(cf, bx, by, ex, ey, fx, fy, uf, vf) < 1e-5f;
+            if (near) {
+                u = (R)uf;
+                v = (R)vf;
+            }
+#pragma unroll 1
+            for (int it = near ? 15 : 0; it < 16; ++it) newton_step<false>(c, Bx, By, Cx, Cy, dx, dy, u, v);
         }
         const R x = add_rn(xi0, u), e = add_rn(et0, v);
         const R du = max(abs_(u), abs_(v));   // displacement in cells (CFL)
