@@ -467,18 +467,38 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
             // c_hat . n0 > 0, decided in float64.  A wall moves rigidly with
             // its own body (it lies in that body's rigid zone and outside
             // every other's blended region).  A float value beyond its
-            // rounding error (below 1e-6 for |c_hat| <= 2) has the float64
-            // value's sign; the others, the directions along the wall, are
-            // decided below
+            // rounding error has the float64 value's sign; the others, the
+            // directions along the wall, are decided below.  The error: some
+            // ten roundings (2^-24) each of the inverse map's entries, the
+            // velocity and the coordinates that it is formed from; sixteen
+            // times the sum of all of them
             const BodyMap<double>& mw = mapSd[GEN ? (ct >> CT_BODY_SHIFT) & (MAX_BODIES - 1) : 0];
+            const BodyMap<R>& mf = mapS[GEN ? (ct >> CT_BODY_SHIFT) & (MAX_BODIES - 1) : 0];
             const double n0x = MD(n0)[2 * j], n0y = MD(n0)[2 * j + 1];
             const R fx = (R)n0x, fy = (R)n0y;
+            R reach = abs_(i00) + abs_(i01) + abs_(i10) + abs_(i11);
+            if (mw.active) {
+                R X, Y;
+                if constexpr (GEN) {
+                    const R2 x = __ldg(reinterpret_cast<const R2*>(MD(nodex)) + j);
+                    X = x.x;
+                    Y = x.y;
+                } else {
+                    const R r = srow[RT_R];
+                    X = abs_(xm) + abs_(r * scol[tid * CS + CT_E]);
+                    Y = abs_(ym) + abs_(r * scol[tid * CS + CT_E + 1]);
+                }
+                reach += abs_(vx) + abs_(vy) + abs_(mf.vtx) + abs_(mf.vty) +
+                         (abs_(mf.va00) + abs_(mf.va01) + abs_(mf.va10) + abs_(mf.va11)) *
+                             (abs_(X) + abs_(Y) + abs_(mf.xp) + abs_(mf.yp));
+            }
+            const R round = R(16.0 / (1 << 24)) * reach;
             unsigned near = 0u;
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
                 const R v = (i00 * R(cxq(q)) + i01 * R(cyq(q)) - vx) * fx + (i10 * R(cxq(q)) + i11 * R(cyq(q)) - vy) * fy;
-                if (v > R(1e-5)) missing |= 1u << q;
-                else if (!(v < R(-1e-5))) near |= 1u << q;
+                if (v > round) missing |= 1u << q;
+                else if (!(v < -round)) near |= 1u << q;
             }
             if (!mw.active) near &= ~1u;   // (a wall at rest: the rest population's is zero)
             if (near) {
