@@ -306,7 +306,7 @@ enum { LBFSI_FIELD_MOMENTS = 0, LBFSI_FIELD_POPULATIONS = 1 };
  * memory belongs to the handle; the pointer is valid until the handle is
  * destroyed, but the state it holds is the current one only until the next
  * step (the step writes the other buffer of a ping-pong pair and that one
- * becomes current).  Reads must be ordered after the handle's stream
+ * becomes current; the float64 populations of every step stand in one buffer).  Reads must be ordered after the handle's stream
  * (lbfsi_synchronize, or work on the same stream); writes change the next
  * step's input.  LBFSI_EINVAL for a bad 'which' or null ptr,
  * LBFSI_ESTATE before lbfsi_init_fields. */

@@ -92,10 +92,11 @@ struct lbfsi_mesh_s {
     size_t esize = 8;
     cudaStream_t stream = nullptr;
     std::vector<lbfsi_body_desc> bodies;
-    void* d_p[2] = {nullptr, nullptr};   // populations, (f_q, g_q) pairs [nbatch][9][N]
+    void* d_p[2] = {nullptr, nullptr};   // populations, (f_q, g_q) pairs [nbatch][9][N]: float a
+                                         // ping-pong pair; float64 the post-collision ones and the state
     void* d_M[2] = {nullptr, nullptr};
-    void* d_ppost = nullptr;             // post-collision populations, same layout (float64: the
-                                         // step's; float: made when the accessor asks)
+    void* d_ppost = nullptr;             // float: post-collision populations, same layout (made when
+                                         // the accessor asks)
     void* d_Y = nullptr;                 // float: correction field [nbatch][2][N]
     void* d_dep = nullptr;               // general meshes, float64: cached static departures ((xi, eta)
                                          // [9][Nx], then codes [Nx]; see SolveDev::dep_xe)
@@ -139,6 +140,7 @@ struct lbfsi_mesh_s {
 
     int cur() const { return (int)(host_k & 1u); }
     bool first() const { return host_k == 0u; }
+    void* pops() const { return d_p[precision == LBFSI_FP64 ? 1 : cur()]; }   // the state's populations
     void changed() { fields_of = ended_at = -1; }   // the state, other than by steps
 };
 
@@ -292,7 +294,8 @@ cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, 
     cudaError_t e = cudaSuccess;
     const bool carry = host && !m->handed_out && m->ended_at == host_step, have = carry && m->fields_of == host_step;
     m->changed();
-    if (!have && (!host || host_step > 0)) {   // (the initial state is streamed without colliding)
+    // (the initial state is streamed without colliding; float64 copies it)
+    if (!have && (!host || host_step > 0 || m->precision == LBFSI_FP64)) {
         e = launch_fields(m, a, 0, 1, host ? (int)host_step : -1, nullptr, s);
         ++*launches;
     }
@@ -337,11 +340,12 @@ int upload_solves(lbfsi_mesh m) {
         s.nbody = m->nbody;
         const size_t bb = (size_t)b * m->nbody;
         for (int p = 0; p < 2; ++p) {
-            s.p[p] = (char*)m->d_p[p] + ((size_t)b * 18 * N + 2 * g0) * es;
+            s.p[p] = (char*)m->d_p[m->precision == LBFSI_FP64 ? 1 : p] + ((size_t)b * 18 * N + 2 * g0) * es;
             s.M[p] = (char*)m->d_M[p] + ((size_t)b * 4 * N + g0) * es;
             s.maps[p] = m->d_maps[p] + bb;
         }
-        s.ppost = m->d_ppost ? (char*)m->d_ppost + ((size_t)b * 18 * N + 2 * g0) * es : nullptr;
+        char* post = (char*)(m->precision == LBFSI_FP64 ? m->d_p[0] : m->d_ppost);
+        s.ppost = post ? post + ((size_t)b * 18 * N + 2 * g0) * es : nullptr;
         s.Y = m->d_Y ? (char*)m->d_Y + ((size_t)b * 2 * N + g0) * es : nullptr;
         s.part = m->d_part + bb * m->host.ntj * 3;
         s.counter = m->d_counter + 4 * b;
@@ -593,9 +597,7 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
         e = cudaMalloc(&m->d_p[k], nb * 18 * N * m->esize);
         if (e == cudaSuccess) e = cudaMalloc(&m->d_M[k], nb * 4 * N * m->esize);
     }
-    if (e == cudaSuccess)
-        e = m->precision == LBFSI_FP64 ? cudaMalloc(&m->d_ppost, nb * 18 * N * m->esize)
-                                       : cudaMalloc(&m->d_Y, nb * 2 * N * m->esize);
+    if (e == cudaSuccess && m->precision == LBFSI_FP32) e = cudaMalloc(&m->d_Y, nb * 2 * N * m->esize);
     // general meshes and float64: departures of the static nodes, solved once
     // per time step size (a float step solves the separable mesh's closed form
     // faster than it reads them; LBFSI_NO_DEPARTURE_CACHE=1 solves them every step instead;
@@ -683,7 +685,7 @@ int lbfsi_init_fields(lbfsi_mesh m, const lbfsi_flow_params* p, const double* rh
     m->changed();
     rc = upload_solves(m);
     if (rc) return rc;
-    e = lbfsi::launch_init(m->precision, m->d_stage, m->d_p[0], m->d_M[0], m->host.Nx, m->nbatch,
+    e = lbfsi::launch_init(m->precision, m->d_stage, m->pops(), m->d_M[0], m->host.Nx, m->nbatch,
                            proto.Cv, m->stream);
     m->launches++;
     if (e != cudaSuccess) return cuda_fail(e, "init kernel");
@@ -762,7 +764,7 @@ int lbfsi_field_ptr(lbfsi_mesh m, int which, void** ptr, int64_t* slots, int64_t
         return fail(LBFSI_EINVAL, "which must be LBFSI_FIELD_MOMENTS or LBFSI_FIELD_POPULATIONS");
     if (!m->initialized) return fail(LBFSI_ESTATE, "init_fields first");
     m->handed_out = true;
-    *ptr = which == LBFSI_FIELD_MOMENTS ? m->d_M[m->cur()] : m->d_p[m->cur()];
+    *ptr = which == LBFSI_FIELD_MOMENTS ? m->d_M[m->cur()] : m->pops();
     if (slots) *slots = (int64_t)m->host.Nx;
     if (row0) *row0 = (int64_t)m->host.G * m->host.nt;
     return LBFSI_OK;
@@ -905,10 +907,10 @@ int lbfsi_get_populations(lbfsi_mesh m, int which, double* f, double* g) {
     if (which != 0 && which != 1) return fail(LBFSI_EINVAL, "which must be 0 or 1");
     if (!m->initialized) return fail(LBFSI_ESTATE, "init_fields first");
     const size_t cnt = (size_t)m->nbatch * 9 * m->host.N, cntx = (size_t)m->nbatch * 9 * m->host.Nx;
-    const void* ps = m->d_p[m->cur()];
+    const void* ps = m->pops();
     if (which == 1 && !m->first()) {
         cudaError_t e = cudaSuccess;
-        if (!m->d_ppost) {
+        if (m->precision == LBFSI_FP32 && !m->d_ppost) {
             e = cudaMalloc(&m->d_ppost, 2 * cntx * m->esize);
             if (e != cudaSuccess) return fail(LBFSI_ENOMEM, "post-collision staging allocation failed");
             const int rc = upload_solves(m);
@@ -922,7 +924,7 @@ int lbfsi_get_populations(lbfsi_mesh m, int which, double* f, double* g) {
             m->launches++;
         }
         if (e != cudaSuccess) return cuda_fail(e, "collide kernel launch");
-        ps = m->d_ppost;
+        ps = m->precision == LBFSI_FP64 ? m->d_p[0] : m->d_ppost;
     }
     std::vector<double> pairs(2 * cnt);
     int rc;
@@ -959,10 +961,10 @@ int lbfsi_set_populations(lbfsi_mesh m, const double* f, const double* g, const 
         unify_cut_copies(m->host, mu.data(), (size_t)m->nbatch * 4, 1);
         const std::vector<double> px = expand_rows(m->host, pairs.data(), (size_t)m->nbatch * 9, 2);
         const std::vector<double> mx = expand_rows(m->host, mu.data(), (size_t)m->nbatch * 4, 1);
-        rc = upload(m, px.data(), m->d_p[c], px.size());
+        rc = upload(m, px.data(), m->pops(), px.size());
         if (!rc) rc = upload(m, mx.data(), m->d_M[c], mx.size());
     } else {
-        rc = upload(m, pairs.data(), m->d_p[c], 2 * cnt);
+        rc = upload(m, pairs.data(), m->pops(), 2 * cnt);
         if (!rc) rc = upload(m, rho_u_T, m->d_M[c], (size_t)m->nbatch * 4 * m->host.N);
     }
     if (rc) return rc;
@@ -1019,7 +1021,7 @@ int lbfsi_checkpoint(lbfsi_mesh m, void* buf, size_t bytes) {
     std::memcpy(p, &h, sizeof(h));
     p += sizeof(h);
     const int c = m->cur();
-    cudaError_t e = cudaMemcpyAsync(p, m->d_p[c], nb * 18 * N * m->esize, cudaMemcpyDeviceToHost, m->stream);
+    cudaError_t e = cudaMemcpyAsync(p, m->pops(), nb * 18 * N * m->esize, cudaMemcpyDeviceToHost, m->stream);
     p += nb * 18 * N * m->esize;
     if (e == cudaSuccess) e = cudaMemcpyAsync(p, m->d_M[c], nb * 4 * N * m->esize, cudaMemcpyDeviceToHost, m->stream);
     p += nb * 4 * N * m->esize;
@@ -1048,7 +1050,7 @@ int lbfsi_restore(lbfsi_mesh m, const void* buf, size_t bytes) {
     const size_t N = (size_t)m->host.Nx, nb = (size_t)m->nbatch;
     const char* p = static_cast<const char*>(buf) + sizeof(h);
     const int c = m->cur();
-    cudaError_t e = cudaMemcpyAsync(m->d_p[c], p, nb * 18 * N * m->esize, cudaMemcpyHostToDevice, m->stream);
+    cudaError_t e = cudaMemcpyAsync(m->pops(), p, nb * 18 * N * m->esize, cudaMemcpyHostToDevice, m->stream);
     p += nb * 18 * N * m->esize;
     if (e == cudaSuccess) e = cudaMemcpyAsync(m->d_M[c], p, nb * 4 * N * m->esize, cudaMemcpyHostToDevice, m->stream);
     p += nb * 4 * N * m->esize;

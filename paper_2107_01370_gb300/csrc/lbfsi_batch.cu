@@ -95,8 +95,8 @@ private:
     std::map<size_t, size_t> free_, used_;
 };
 
-// Step workspaces of the admitted solves (the float path's correction field,
-// the float64 path's post-collision populations), beside the pool so that it
+// Step workspaces of the admitted solves (the bodies' step maps and the float
+// path's correction field), beside the pool so that it
 // admits the solves it always did: blocks of at least CHUNK bytes, kept for
 // the next solves and given back with the batch.  Bounded by the solves the
 // pool can hold at once.
@@ -138,7 +138,7 @@ struct Slot {
     int ntiles = 0;
     SolveDev dev{};
     std::vector<void*> blocks;
-    void* work = nullptr;   // its step workspace (SolveDev::Y or ppost)
+    void* work = nullptr;   // its step workspace (SolveDev::prop, Y)
     // the tile rows its tensor maps were made for (-1: none yet, 0: not used)
     int tma_rows = -1;
 };
@@ -607,16 +607,14 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
         return p;
     };
     bool ok = true;
-    void* p0 = nullptr;   // first population block (the initial state is written there)
+    void* p0 = nullptr;   // population block of the initial state (float64: the state's, the second)
     void* m0 = nullptr;
     for (int p = 0; p < 2 && ok; ++p) {
         void* pb = take(18 * Nx * es);
         void* mb = take(4 * Nx * es);
         ok = ok && pb && mb;
-        if (p == 0) {
-            p0 = pb;
-            m0 = mb;
-        }
+        if (p == (b->precision == LBFSI_FP64 ? 1 : 0)) p0 = pb;
+        if (p == 0) m0 = mb;
         if (ok) {
             sd.p[p] = (char*)pb + 2 * g0 * es;   // row 0
             sd.M[p] = (char*)mb + g0 * es;
@@ -630,14 +628,19 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
     double* stage = nullptr;
     ok = ok && (stage = (double*)take(4 * Nx * sizeof(double))) != nullptr;
     if (ok) {
-        // the body's step map, then the populations' or the field's slots
-        const size_t w = b->precision == LBFSI_FP64 ? 2 : 1, head = 512;
+        // the body's step map, then float the correction field
+        const bool f64 = b->precision == LBFSI_FP64;
+        const size_t head = 512;
         static_assert(sizeof(lbfsi::BodyProp) <= 512, "workspace head");
-        s.work = b->work.alloc(head + w * (w == 2 ? 9 : 2) * Nx * es);
+        s.work = b->work.alloc(head + (f64 ? 0 : 2 * Nx * es));
         ok = s.work != nullptr;
         if (ok) {
             sd.prop = (const lbfsi::BodyProp*)s.work;
-            (w == 2 ? sd.ppost : sd.Y) = (char*)s.work + head + w * g0 * es;
+            if (!f64) sd.Y = (char*)s.work + head + g0 * es;
+        }
+        if (f64) {   // (SolveDev::p, ppost)
+            sd.ppost = sd.p[0];
+            sd.p[0] = sd.p[1];
         }
     }
     if (!ok) {

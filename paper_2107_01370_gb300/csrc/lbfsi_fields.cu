@@ -517,6 +517,19 @@ __device__ __forceinline__ void fields_tile(const FieldArgs& a, const SolveDev& 
     }
 }
 
+// ---- float64, step 0: the initial state, which is streamed as it is, into the
+// post-collision buffer (the same tiles; a thread's five or four directions).
+template <int TI>
+__device__ __forceinline__ void copy_state(const FieldArgs& a, const SolveDev& S, const MeshDev& G, int sb, int blk) {
+    const int half = (int)threadIdx.x / (32 * TI), t = (int)threadIdx.x - half * 32 * TI;
+    const int i = (blk / G.ntj) * TI + t / TILE_J, j = (blk % G.ntj) * TILE_J + t % TILE_J;
+    if (i >= G.nr || j >= G.nt) return;
+    const ptrdiff_t N = G.N, n = (ptrdiff_t)i * G.nt + j;
+    const double2* p = reinterpret_cast<const double2*>(S.p[0]) + (size_t)sb * 9 * N;
+    double2* po = reinterpret_cast<double2*>(S.ppost) + (size_t)sb * 9 * N;
+    for (int q = half ? 5 : 0; q < (half ? 9 : 5); ++q) po[q * N + n] = p[q * N + n];
+}
+
 // Uniform launches (a mesh handle: the records are launch arguments) and table
 // launches (the batch runtime).  R float: TI unused (marching strips).  R double: tiles of TI rows.
 template <typename R, bool GEN, int TI, bool UNIFORM>
@@ -553,7 +566,10 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 32 * MARCH_WARPS : 64 * TI, s
         wall_loads<R, GEN>(a, S, G, sb, blk, kk, ctr);
         return;
     }
-    if (kk == 0u) return;   // the first launch streams the initial state, nothing collides
+    if (kk == 0u) {   // the first launch streams the initial state, nothing collides
+        if constexpr (sizeof(R) == 8) copy_state<TI>(a, S, G, sb, blk);
+        return;
+    }
     const int cur = (int)(kk & 1u);
     stage_maps(a, S, sb, GEN ? S.nbody : 1, cur, smap);
     if constexpr (sizeof(R) == 4) {

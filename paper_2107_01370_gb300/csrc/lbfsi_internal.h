@@ -153,11 +153,12 @@ struct SolveDev {
     // with the population
     float fgref[18];
     float mref[4];   // its moments: rho, rho u_x, rho u_y, 2 rho E
-    void* p[2];                    // populations, (f_q, g_q) pairs [9][N]
+    void* p[2];                    // populations, (f_q, g_q) pairs [9][N] (float64: both the one
+                                   // buffer of the state, ppost the other)
     void* M[2];                    // moments [4][N]
     StepMaps* maps[2];             // [nbody] each
     void* ppost;                   // post-collision pairs [9][N] (float64 path: written by the field
-                                   // launch; float: only for the accessor)
+                                   // launch, read by the stream; float: only for the accessor)
     void* Y;                       // float path: correction field [2][N] of the current state
     double* part;                  // [nbody][ntj][3] load partials of the streamed step
     unsigned* counter;             // [4]: CTA count of the step launch, step number k, loads

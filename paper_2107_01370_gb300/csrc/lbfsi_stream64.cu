@@ -1,6 +1,8 @@
 // Stream launch of the float64 path on structured meshes: streaming of step
 // k+1 from the post-collision populations of step k, which the field launch
-// (lbfsi_fields.cu) has formed.
+// (lbfsi_fields.cu) has formed (k = 0: a copy of the initial state).  The two
+// population buffers are the state's and the post-collision one, not a ping-pong
+// pair: the field launch reads the first and writes the second, this one back.
 //
 // Float64 arithmetic is what bounds it: a warp instruction holds the SM's unit
 // for some 16 cycles, so every operation counts, and so does the chain of one
@@ -74,7 +76,7 @@ __global__ void __launch_bounds__(S64_THREADS, 4) k_stream64(const __grid_consta
         }
     }
     __syncthreads();
-    const double2* __restrict__ pin = reinterpret_cast<const double2*>(kstep ? S.ppost : S.p[cur]) + (size_t)sb * 9 * N;
+    const double2* __restrict__ pin = reinterpret_cast<const double2*>(S.ppost) + (size_t)sb * 9 * N;
     const double* __restrict__ M = reinterpret_cast<const double*>(S.M[cur]) + (size_t)sb * 4 * N;
     double2* __restrict__ pout = reinterpret_cast<double2*>(S.p[cur ^ 1]) + (size_t)sb * 9 * N;
     double* __restrict__ Mout = reinterpret_cast<double*>(S.M[cur ^ 1]) + (size_t)sb * 4 * N;
