@@ -390,7 +390,7 @@ int lbfsi_wall_loads_noalloc(int nr, int ntheta, int nbatch, int precision, cons
 
 /* ---- Batch runtime: many solves on meshes of different sizes, admitted and
  * retired while others run, advanced together (two launches per step for all
- * active solves).  Device memory comes from one pool allocated at creation;
+ * active solves).  Device memory is allocated at creation (one pool);
  * a solve is admitted only if the pool can hold it (continuous batching with
  * memory-based admission).  Solves on identical O-grids share one device copy
  * of the mesh geometry.  The per-step physics is exactly that of lbfsi_step
@@ -414,8 +414,10 @@ typedef struct {
 } lbfsi_solve_desc;
 
 /* Create a batch runtime whose solves live in a device pool of pool_bytes
- * (one cudaMalloc now; none later except when the tile table outgrows its
- * buffer).  precision: LBFSI_FP64 or LBFSI_FP32 for every solve of the batch. */
+ * (allocated now, and beside it the step workspaces of the solves it can hold,
+ * 3 MiB and in float 1/22 of the pool; where these cannot be had, a solve's
+ * workspace comes from the pool too.  No cudaMalloc later except when the tile
+ * tables outgrow their buffers).  precision: LBFSI_FP64 or LBFSI_FP32 for every solve of the batch. */
 int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfsi_batch* out);
 int lbfsi_batch_destroy(lbfsi_batch b);
 

@@ -8,7 +8,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
-#include <memory>
 #include <string>
 #include <vector>
 
@@ -77,7 +76,6 @@ public:
         }
         free_[start] = len;
     }
-    bool owns(const void* p) const { return p && (const char*)p >= base_ && (const char*)p < base_ + size_; }
     size_t free_bytes() const {
         size_t s = 0;
         for (auto& kv : free_) s += kv.second;
@@ -95,33 +93,9 @@ private:
     std::map<size_t, size_t> free_, used_;
 };
 
-// Step workspaces of the admitted solves (the bodies' step maps and the float
-// path's correction field), beside the pool so that it
-// admits the solves it always did: blocks of at least CHUNK bytes, kept for
-// the next solves and given back with the batch.  Bounded by the solves the
-// pool can hold at once.
-class Workspace {
-public:
-    void* alloc(size_t bytes) {
-        for (auto& c : chunks_)
-            if (void* p = c->alloc(bytes)) return p;
-        auto c = std::make_unique<Pool>();
-        if (c->init(std::max(bytes, CHUNK)) != LBFSI_OK) {
-            c = std::make_unique<Pool>();
-            if (c->init(bytes) != LBFSI_OK) return nullptr;
-        }
-        chunks_.push_back(std::move(c));
-        return chunks_.back()->alloc(bytes);
-    }
-    void release(void* p) {
-        for (auto& c : chunks_)
-            if (c->owns(p)) c->release(p);
-    }
-
-private:
-    static constexpr size_t CHUNK = 16u << 20;
-    std::vector<std::unique_ptr<Pool>> chunks_;
-};
+// The body's step map at the head of a solve's workspace.
+constexpr size_t WORK_HEAD = 512;
+static_assert(sizeof(lbfsi::BodyProp) <= WORK_HEAD, "workspace head");
 
 struct MeshEntry {
     lbfsi::HostMesh host;
@@ -138,7 +112,7 @@ struct Slot {
     int ntiles = 0;
     SolveDev dev{};
     std::vector<void*> blocks;
-    void* work = nullptr;   // its step workspace (SolveDev::prop, Y)
+    void* work = nullptr;   // its step workspace (SolveDev::prop, Y), null: among the blocks
     // the tile rows its tensor maps were made for (-1: none yet, 0: not used)
     int tma_rows = -1;
 };
@@ -147,12 +121,14 @@ struct Slot {
 
 struct lbfsi_batch_s {
     Pool pool;
-    Workspace work;
+    // step workspaces of the admitted solves (the bodies' step maps and the float
+    // path's correction field), beside the pool so that it admits the solves it
+    // always did; made with the batch, for as many as the pool can hold (or
+    // empty: the workspaces then come from the pool)
+    Pool work;
     int precision = LBFSI_FP32, variant = 4, order = 0, tile_rows = 16;
-    // reading a solve back: float64 staging of the largest read so far, and
-    // pinned copies of its record and the status word (null: could not be had)
-    double* d_read = nullptr;
-    size_t read_count = 0;
+    // reading a solve back: pinned copies of its record and the status word
+    // (null: could not be had)
     struct Small {
         StepMaps maps;
         unsigned status;
@@ -524,6 +500,8 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
         delete b;
         return rc;
     }
+    // a node takes 176 bytes of the pool and in float 8 of the workspaces
+    b->work.init((size_t)b->max_slots * (WORK_HEAD + 256) + (precision == LBFSI_FP32 ? pool_bytes / 22 : 0));
     cudaError_t e = cudaMalloc(&b->d_meshes, b->max_meshes * sizeof(MeshDev));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_solves, b->max_slots * sizeof(SolveDev));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_status, sizeof(unsigned));
@@ -551,7 +529,7 @@ int lbfsi_batch_destroy(lbfsi_batch b) {
     cudaStreamSynchronize(b->stream);
     if (b->h_get) cudaFreeHost(b->h_get);
     void* ptrs[] = {b->d_meshes, b->d_solves, b->d_tiles, b->d_ftiles, b->d_status, b->d_zero_state,
-                    b->d_zero_loads, b->d_tmaps, b->d_read};
+                    b->d_zero_loads, b->d_tmaps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (b->graph) cudaGraphExecDestroy(b->graph);
@@ -630,13 +608,13 @@ int add_solve(lbfsi_batch b, const lbfsi_body_desc& body_desc, const lbfsi_flow_
     if (ok) {
         // the body's step map, then float the correction field
         const bool f64 = b->precision == LBFSI_FP64;
-        const size_t head = 512;
-        static_assert(sizeof(lbfsi::BodyProp) <= 512, "workspace head");
-        s.work = b->work.alloc(head + (f64 ? 0 : 2 * Nx * es));
-        ok = s.work != nullptr;
+        const size_t bytes = WORK_HEAD + (f64 ? 0 : 2 * Nx * es);
+        void* work = s.work = b->work.alloc(bytes);
+        if (!work) work = take(bytes);
+        ok = work != nullptr;
         if (ok) {
-            sd.prop = (const lbfsi::BodyProp*)s.work;
-            if (!f64) sd.Y = (char*)s.work + head + g0 * es;
+            sd.prop = (const lbfsi::BodyProp*)work;
+            if (!f64) sd.Y = (char*)work + WORK_HEAD + g0 * es;
         }
         if (f64) {   // (SolveDev::p, ppost)
             sd.ppost = sd.p[0];
@@ -901,29 +879,17 @@ int lbfsi_batch_get(lbfsi_batch b, int slot, double* rho_u_T, double* loads, lbf
     const int cur = s.steps_done & 1;
     const size_t N = (size_t)b->meshes[s.mesh].host.N, Nx = (size_t)b->meshes[s.mesh].host.Nx;
     cudaError_t e = cudaSuccess;
-    std::vector<unsigned char> raw;
-    if (rho_u_T && b->precision == LBFSI_FP32 && b->read_count < 4 * N) {
-        // float64 staging of the largest solve read so far
-        if (b->d_read) cudaFree(b->d_read);   // (waits for its last copy)
-        b->read_count = 0;
-        if (cudaMalloc(&b->d_read, 4 * N * sizeof(double)) == cudaSuccess) {
-            b->read_count = 4 * N;
-        } else {
-            b->d_read = nullptr;   // no room: widened on the host
-            cudaGetLastError();
-        }
-    }
     // rows 0 .. nr-1 of the four components (Nx slots apart) straight into the
-    // caller's array, float values widened on the device first
-    const bool direct = rho_u_T && (b->precision == LBFSI_FP64 || b->d_read);
-    if (rho_u_T && b->precision == LBFSI_FP32 && b->d_read) {
-        e = lbfsi::launch_read(b->precision, s.dev.M[cur], Nx, nullptr, b->d_read, (int)N, 4, b->stream);
+    // caller's array, float values widened on the device first: in the population
+    // buffer that the next step writes (72 bytes a node; 32 are needed)
+    if (rho_u_T && b->precision == LBFSI_FP32) {
+        double* wide = (double*)s.dev.p[cur ^ 1];
+        e = lbfsi::launch_read(b->precision, s.dev.M[cur], Nx, nullptr, wide, (int)N, 4, b->stream);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(rho_u_T, b->d_read, 4 * N * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+            e = cudaMemcpyAsync(rho_u_T, wide, 4 * N * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
     } else if (rho_u_T) {
-        if (!direct) raw.resize(4 * N * b->esize);
-        e = cudaMemcpy2DAsync(direct ? (void*)rho_u_T : raw.data(), N * b->esize, s.dev.M[cur], Nx * b->esize,
-                              N * b->esize, 4, cudaMemcpyDeviceToHost, b->stream);
+        e = cudaMemcpy2DAsync(rho_u_T, N * sizeof(double), s.dev.M[cur], Nx * sizeof(double), N * sizeof(double), 4,
+                              cudaMemcpyDeviceToHost, b->stream);
     }
     StepMaps own{}, *rec = b->h_get ? &b->h_get->maps : &own;
     if (e == cudaSuccess && (loads || state))
@@ -931,10 +897,6 @@ int lbfsi_batch_get(lbfsi_batch b, int slot, double* rho_u_T, double* loads, lbf
     if (e != cudaSuccess) return cuda_err(e, "batch results copy");
     const int rc = check_status(b);
     const StepMaps& mp = *rec;
-    if (rho_u_T && !direct) {
-        const float* f = reinterpret_cast<const float*>(raw.data());
-        for (size_t n = 0; n < 4 * N; ++n) rho_u_T[n] = (double)f[n];
-    }
     if (loads)
         for (int c = 0; c < 3; ++c) loads[c] = mp.loads[c];
     if (state) {

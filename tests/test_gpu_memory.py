@@ -64,3 +64,42 @@ def test_fp64_views_follow_the_state_from_the_start(L):
         m.close()
     rho = out[1][0][0][4:-4] / out[0][0][0][4:-4]      # off the wall and far field, whose targets are moments
     assert np.abs(rho - (1.0 + 2.0 ** -8)).max() < 1e-12
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_batch_allocates_nothing_after_its_creation(L, precision):
+    """Solves of growing size admitted, stepped, read and removed one at a time
+    (tile tables and kernels aside)."""
+    prec = L.FP32 if precision == "fp32" else L.FP64
+    cases = [_case(nr, nt) for nr, nt in (((128, 64), (512, 512), (2048, 1100), (2304, 1100)) if precision == "fp32"
+                                          else ((128, 64), (512, 256), (768, 512)))]
+    for k in range(2):                    # (the first batch also loads the kernels)
+        b = L.Batch(640 * MB, precision=prec)
+        before = _free()
+        for case, M0 in cases:
+            s = b.add(case.r, case.e, case.bodies[0], case.flow, 2, M0)
+            b.step(2)
+            assert np.isfinite(b.get(s)[0]).all()
+            b.remove(s)
+        took = before - _free()
+        b.close()
+    assert took <= 8 * MB
+
+
+def test_batch_reads_do_not_disturb_the_run(L):
+    """A float solve read between steps ends where one read at the end does."""
+    case, M0 = _case(48, 64)
+    got = []
+    for reads in (False, True):
+        b = L.Batch(64 * MB, precision=L.FP32)
+        s = b.add(case.r, case.e, case.bodies[0], case.flow, 9, M0)
+        if reads:
+            b.get(s)
+        for _ in range(9):
+            b.step(1)
+            if reads:
+                b.get(s)
+        f, loads, state = b.get(s)
+        got.append((f, loads, state))
+        b.close()
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1]) and got[0][2] == got[1][2]
