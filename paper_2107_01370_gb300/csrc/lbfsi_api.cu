@@ -97,7 +97,8 @@ struct lbfsi_mesh_s {
     void* d_M[2] = {nullptr, nullptr};
     void* d_ppost = nullptr;             // float: post-collision populations, same layout (made when
                                          // the accessor asks)
-    void* d_Y = nullptr;                 // float: correction field [nbatch][2][N]
+    void* d_Y = nullptr;                 // float: correction field [nbatch][2][N] (where the device has
+                                         // no room for it, in d_stage, which is idle but for transfers)
     void* d_dep = nullptr;               // general meshes, float64: cached static departures ((xi, eta)
                                          // [9][Nx], then codes [Nx]; see SolveDev::dep_xe)
     double* d_stage = nullptr;  // [nbatch][4][N] float64 staging
@@ -315,7 +316,7 @@ cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, 
 }
 
 void free_all(lbfsi_mesh m) {
-    void* ptrs[] = {m->d_p[0], m->d_p[1], m->d_M[0], m->d_M[1], m->d_ppost, m->d_Y, m->d_dep, m->d_stage, m->d_maps[0], m->d_maps[1], m->d_state_a, m->d_state_b,
+    void* ptrs[] = {m->d_p[0], m->d_p[1], m->d_M[0], m->d_M[1], m->d_ppost, m->d_Y == m->d_stage ? nullptr : m->d_Y, m->d_dep, m->d_stage, m->d_maps[0], m->d_maps[1], m->d_state_a, m->d_state_b,
                     m->d_loads_tmp, m->d_part, m->d_counter, m->d_bodies, m->d_prop, m->d_meshdev, m->d_solves,
                     m->d_status};
     for (void* p : ptrs)
@@ -597,14 +598,23 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
         e = cudaMalloc(&m->d_p[k], nb * 18 * N * m->esize);
         if (e == cudaSuccess) e = cudaMalloc(&m->d_M[k], nb * 4 * N * m->esize);
     }
-    if (e == cudaSuccess && m->precision == LBFSI_FP32) e = cudaMalloc(&m->d_Y, nb * 2 * N * m->esize);
+    // (what a step can do without is left out where the device has no room)
+    auto spare = [&](void** p, size_t bytes) {
+        if (e != cudaSuccess || cudaMalloc(p, bytes) == cudaSuccess) return;
+        *p = nullptr;
+        cudaGetLastError();
+    };
+    if (m->precision == LBFSI_FP32) {
+        spare(&m->d_Y, nb * 2 * N * m->esize);
+        if (!m->d_Y) m->d_Y = m->d_stage;
+    }
     // general meshes and float64: departures of the static nodes, solved once
     // per time step size (a float step solves the separable mesh's closed form
-    // faster than it reads them; LBFSI_NO_DEPARTURE_CACHE=1 solves them every step instead;
-    // the results are the same)
+    // faster than it reads them; LBFSI_NO_DEPARTURE_CACHE=1, or a device without
+    // room for them, solves them every step instead; the results are the same)
     const char* nc = std::getenv("LBFSI_NO_DEPARTURE_CACHE");
-    if (e == cudaSuccess && (m->host.general || m->precision == LBFSI_FP64) && !(nc && std::atoi(nc) != 0))
-        e = cudaMalloc(&m->d_dep, 9 * N * 2 * m->esize + N * sizeof(unsigned long long));
+    if ((m->host.general || m->precision == LBFSI_FP64) && !(nc && std::atoi(nc) != 0))
+        spare(&m->d_dep, 9 * N * 2 * m->esize + N * sizeof(unsigned long long));
     if (e != cudaSuccess) {
         free_all(m);
         delete m;
@@ -895,6 +905,7 @@ int lbfsi_get_fields(lbfsi_mesh m, double* rho_u_T) {
     } else {
         e = lbfsi::launch_read(m->precision, src, Nx, nullptr, m->d_stage, (int)N, rows, m->stream);
         m->launches++;
+        if (m->d_Y == m->d_stage) m->fields_of = -1;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(rho_u_T, m->d_stage, rows * N * w, cudaMemcpyDeviceToHost, m->stream);
     }

@@ -103,3 +103,36 @@ def test_batch_reads_do_not_disturb_the_run(L):
         got.append((f, loads, state))
         b.close()
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1]) and got[0][2] == got[1][2]
+
+
+@pytest.mark.parametrize("precision,node", [("fp32", 208), ("fp64", 384)])
+def test_handle_runs_where_only_its_state_fits(L, precision, node):
+    """With room for the populations, moments and staging alone (node bytes a
+    node) a handle is made and gives the bits it gives with room to spare: the
+    departure cache and the float correction field's buffer are left out."""
+    import torch
+    prec = L.FP32 if precision == "fp32" else L.FP64
+    case, M0 = _case(4096, 1024)
+    N = 4096 * 1024
+
+    def run():
+        m = L.Mesh(case.r, case.e, case.bodies, precision=prec)
+        m.init_fields(case.flow, M0[None])
+        m.step(1)
+        m.step(1)
+        f = m.get_fields()                # (float: through the staging)
+        m.step(1)
+        m.step(1)
+        f = m.get_fields()
+        m.close()
+        return f
+
+    want = run()
+    torch.cuda.empty_cache()
+    hold = torch.empty(_free() - node * N - 16 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        got = run()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(want, got)
