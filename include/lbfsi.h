@@ -19,6 +19,9 @@
  *    non-physical state) are recorded in a device status word and returned by
  *    the next synchronising call (lbfsi_synchronize, lbfsi_body_forces,
  *    lbfsi_get_*).
+ *  - Several threads may read one handle or batch at once (loads, states,
+ *    fields, status); a call that changes it (steps, states set, solves
+ *    admitted or removed) needs it for itself.
  *
  * Mesh: structured O-grid, node (i, j) at X = (xc, yc) + r[i] e[j], i = 0 on
  * the body wall, i = nr-1 on the far field, j periodic.  Node index

@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -106,6 +107,7 @@ struct lbfsi_mesh_s {
     // between steps (null: could not be had, the reads go to pageable memory)
     StepMaps* h_maps = nullptr;
     unsigned* h_status = nullptr;
+    std::mutex reading;         // held by a read from its first copy until it has taken its values out
     StepMaps* d_maps[2] = {nullptr, nullptr};  // [nbatch][nbody] each
     BodyStateDev* d_state_a = nullptr;          // host-given states staging
     BodyStateDev* d_state_b = nullptr;
@@ -166,13 +168,19 @@ int status_code(unsigned st) {
 }
 
 // The status word behind the stream's work (and the records, whose copy was
-// enqueued before): one copy into pinned memory, one wait.
-int check_status(lbfsi_mesh m) {
+// enqueued before): one copy into pinned memory, one wait.  The caller holds
+// 'reading'.
+int read_status(lbfsi_mesh m) {
     unsigned own = 0, *st = m->h_status ? m->h_status : &own;
     cudaError_t e = cudaMemcpyAsync(st, m->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "status read");
     return status_code(*st);
+}
+
+int check_status(lbfsi_mesh m) {
+    std::lock_guard<std::mutex> hold(m->reading);
+    return read_status(m);
 }
 
 void to_double(const void* src, double* dst, size_t n, int precision) {
@@ -787,11 +795,12 @@ int lbfsi_synchronize(lbfsi_mesh m) {
 
 static int download_maps(lbfsi_mesh m, std::vector<StepMaps>& out) {
     out.resize(m->slots());
+    std::lock_guard<std::mutex> hold(m->reading);
     StepMaps* to = m->h_maps ? m->h_maps : out.data();
     cudaError_t e = cudaMemcpyAsync(to, m->d_maps[m->cur()], out.size() * sizeof(StepMaps),
                                     cudaMemcpyDeviceToHost, m->stream);
     if (e != cudaSuccess) return cuda_fail(e, "maps copy");
-    const int rc = check_status(m);
+    const int rc = read_status(m);
     if (!rc && m->h_maps) std::memcpy(out.data(), m->h_maps, out.size() * sizeof(StepMaps));
     return rc;
 }

@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -133,6 +134,7 @@ struct lbfsi_batch_s {
         StepMaps maps;
         unsigned status;
     }* h_get = nullptr;
+    std::mutex reading;      // held by a read from its first copy until it has taken its values out
     bool own_shape = true;   // no schedule asked for: the shape follows the active solves' sizes
     int shape = 4;           // tile shape launched (rebuild_tiles)
     size_t esize = 4;
@@ -389,8 +391,8 @@ int rebuild_tiles(lbfsi_batch b) {
     return LBFSI_OK;
 }
 
-// (one copy behind the stream's work, one wait)
-int check_status(lbfsi_batch b) {
+// (one copy behind the stream's work, one wait; the caller holds 'reading')
+int read_status(lbfsi_batch b) {
     unsigned own = 0, *hs = b->h_get ? &b->h_get->status : &own;
     cudaError_t e = cudaMemcpyAsync(hs, b->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -404,6 +406,11 @@ int check_status(lbfsi_batch b) {
         return lbfsi::set_error(LBFSI_ECUDA, "a tensor copy of the step did not complete within its wait limit");
     if (st & lbfsi::ST_NONPHYS) return lbfsi::set_error(LBFSI_ENONPHYS, "non-physical state (rho<=0, T<=0 or NaN)");
     return LBFSI_OK;
+}
+
+int check_status(lbfsi_batch b) {
+    std::lock_guard<std::mutex> hold(b->reading);
+    return read_status(b);
 }
 
 // Step launch of one part of the tile table (0 separable, 1 general meshes).
@@ -891,11 +898,12 @@ int lbfsi_batch_get(lbfsi_batch b, int slot, double* rho_u_T, double* loads, lbf
         e = cudaMemcpy2DAsync(rho_u_T, N * sizeof(double), s.dev.M[cur], Nx * sizeof(double), N * sizeof(double), 4,
                               cudaMemcpyDeviceToHost, b->stream);
     }
+    std::lock_guard<std::mutex> hold(b->reading);
     StepMaps own{}, *rec = b->h_get ? &b->h_get->maps : &own;
     if (e == cudaSuccess && (loads || state))
         e = cudaMemcpyAsync(rec, s.dev.maps[cur], sizeof(StepMaps), cudaMemcpyDeviceToHost, b->stream);
     if (e != cudaSuccess) return cuda_err(e, "batch results copy");
-    const int rc = check_status(b);
+    const int rc = read_status(b);
     const StepMaps& mp = *rec;
     if (loads)
         for (int c = 0; c < 3; ++c) loads[c] = mp.loads[c];
