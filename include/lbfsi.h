@@ -490,7 +490,8 @@ int lbfsi_batch_memory(lbfsi_batch b, size_t* free_bytes, size_t* largest_free);
 /* Tile shape and tile-table order of a batch's step launches (the CTA
  * schedule).  order 0: the tiles of each solve together, in slot order;
  * order 1: tile rows outermost across all solves, so the wall and
- * blending-region tiles (the most expensive) start first.  Synchronises. */
+ * blending-region tiles (the most expensive) start first.  Takes effect with
+ * the next step, which synchronises. */
 int lbfsi_batch_set_schedule(lbfsi_batch b, int variant, int order);
 int lbfsi_batch_get_schedule(lbfsi_batch b, int* variant, int* order);
 

@@ -1,9 +1,10 @@
 // Batch runtime (declared in include/lbfsi.h): solves on O-grids of different
 // sizes admitted into a device memory pool and retired while others run, all
-// active solves advanced together by one table launch of the step kernel per
-// step.  Native pieces: a first-fit pool allocator over one cudaMalloc, a
-// cache of device mesh geometry shared by solves on identical O-grids, slot
-// bookkeeping and the tile table (the node-to-CTA schedule) of each launch.
+// active solves advanced together by table launches, per step a step launch and
+// a field launch for each mesh kind that is there (separable, by coordinates).
+// Native pieces: a first-fit pool allocator over one cudaMalloc, a cache of
+// device mesh geometry shared by solves on identical O-grids, slot bookkeeping
+// and the tile tables (the node-to-CTA schedule) of the launches.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -344,7 +345,6 @@ int rebuild_tiles(lbfsi_batch b) {
             t.mesh = s.mesh;
             t.i0 = ti * rows;
             t.j0 = tj * lbfsi::TILE_J;
-            t.tj = tj;
             // a separable tile whose columns do not wrap, of a solve with maps
             const int ntm = b->meshes[s.mesh].host.nt;
             t.tma = part == 0 && tma_on && s.tma_rows == rows && t.j0 >= 4 && t.j0 + lbfsi::TILE_J + 4 <= ntm;

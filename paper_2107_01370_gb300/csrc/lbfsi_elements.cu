@@ -406,7 +406,6 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
     const size_t N = (size_t)a.N;
     const R2* pp = static_cast<const R2*>(a.ppost) + (size_t)b * 9 * N;
     double fcx = 0.0, fcy = 0.0, fcm = 0.0;
-    bool wallnode = false;
     if (n < a.N) {
         const SolveDev& fl = a.flow;
         const R dt = flowv<R>(fl, fl.dt, fl.dt_f), Cv = flowv<R>(fl, fl.Cv, fl.Cv_f);
@@ -416,7 +415,6 @@ __global__ void __launch_bounds__(EM_THREADS, sizeof(R) == 4 ? 5 : 2) k_em_strea
         R2* Qo = static_cast<R2*>(a.dQ) + (size_t)b * N;
         const R2 x = __ldg(static_cast<const R2*>(a.X) + n);
         const int kd = __ldg(a.kind + n);
-        wallnode = kd > 0;
         if (kd < 0) {
             // far field: targets at B = A - dt n_out; the inlet prescribes the
             // free stream's u and T (reading R20)

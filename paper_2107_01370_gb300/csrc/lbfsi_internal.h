@@ -167,7 +167,7 @@ struct SolveDev {
     const BodyProp* prop;          // [nbody]
     double iCv, idt, iPr, muP;     // 1 / Cv, 1 / dt, 1 / Pr, mu / Pr
     float iCv_f, muP_f;
-    // general meshes, uniform launches: departure points of the nodes the
+    // general meshes and float64, uniform launches: departure points of the nodes the
     // blend does not move (g = I, V_G = 0, so the displacement of direction q
     // is -dt c_q for every step): (xi, eta) pairs [9][N] in the element type
     // of the path and per node a code [N] (5 bits per direction: the window
@@ -181,9 +181,9 @@ struct SolveDev {
 // One CTA of a step launch: a tile of one solve.  The entry repeats the
 // solve's counter and maps pointers so that a CTA can read its step number
 // and fetch its maps without first loading the solve record.  tma: stage the
-// tile's M^k and populations by tensor copies (StepArgs::tmaps).
+// tile's populations and Y by tensor copies (StepArgs::tmaps).
 struct TileDev {
-    int solve, mesh, i0, j0, tj, tma;
+    int solve, mesh, i0, j0, tma;
     unsigned* counter;
     StepMaps* maps[2];
 };
@@ -283,8 +283,7 @@ constexpr int GEN_TILE_ROWS_FP32 = 16, GEN_THREADS_FP32 = 256, GEN_MINB_FP32 = 3
 inline int general_tile_rows(int precision, int variant) {
     return precision == 0 ? tile_rows(0, variant) : GEN_TILE_ROWS_FP32;
 }
-// Number of tile shapes of the float step kernel (variants 0 .. n-1); the
-// float64 kernel has one.
+// Number of tile shapes of the step kernel of a precision (variants 0 .. n-1).
 int step_variants(int precision);
 // One-time configuration of a step kernel (shared-memory limit, occupancy);
 // done by the first launch, and by this call before a stream capture.
@@ -293,8 +292,6 @@ constexpr int TILE_J = 32;
 inline int tiles_j(int nt) { return (nt + TILE_J - 1) / TILE_J; }
 cudaError_t launch_init(int precision, const double* M, void* P, void* Mout, int N, int nbatch,
                         double Cv, cudaStream_t s);
-// Build the maps record from explicit states: S_cur (collision), S_next and
-// S_vgprev (stream); loads copied from 'loads' if non-null.
 // The kernels of a step are launched while the one before still runs
 // (programmatic stream serialization) and wait for its end and its writes
 // themselves, first thing (wait_previous): a launch's start -- some 2 to 3 us
@@ -304,7 +301,10 @@ cudaError_t launch_init(int precision, const double* M, void* P, void* Mout, int
 // ellipse 512 x 256 x 8 132 -> 127).  Float64: launches of few blocks only, which
 // find SMs of their own (24 x 32: 91.5 -> 87.9 us); more of them are packed
 // beside the running kernel's on some SMs, whose float64 rate then bounds the
-// step while others idle (128 x 64: 46.5 -> 54.7 us, a 97 x 161 C-grid 106 -> 120).
+// step while others idle (128 x 64: 47.4 -> 59.4 us, a 97 x 161 C-grid 106 -> 120).
+// The line is on the safe side: with the overlap and without, by blocks of the
+// stream launch, 76: 43.0 and 47.2 us; 160: 44.9 and 47.8; 200: 46.3 and 47.2; by
+// coordinates 128: 50.4 and 53.3, 192: 54.4 and 54.6; 256 (128 x 64) the other way.
 constexpr unsigned OVERLAP_BLOCKS_FP64 = 76;   // half the SMs
 template <typename... P, typename... A>
 cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap,
@@ -328,6 +328,8 @@ cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
 // the order given (null: as they lie)
 cudaError_t launch_read(int precision, const void* src, size_t stride, const int* order, double* dst, int N, size_t rows,
                         cudaStream_t s);
+// Build the maps record from explicit states: S_cur (collision), S_next and
+// S_vgprev (stream); loads copied from 'loads' if non-null.
 cudaError_t launch_prepare(const BodyDev* bodies, const BodyStateDev* S_cur,
                            const BodyStateDev* S_next, const BodyStateDev* S_vgprev,
                            const double* loads, double dt, int nbatch, StepMaps* maps,

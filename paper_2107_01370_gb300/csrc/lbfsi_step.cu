@@ -59,21 +59,15 @@ struct Tile {
 constexpr int RS = ROWTAB;
 constexpr int CS = COLTAB + 4;
 
-// Rows of geometry tables a separable tile stages (the tile's nodes).
+// Dynamic shared memory of a block: the staged populations and Y, then the
+// geometry tables of the tile's nodes (separable meshes) or the mirrored row 0
+// of a C-grid.
 template <int TI, int TJ, bool GEN>
 constexpr size_t step_smem_bytes() {
     using T = Tile<TI, TJ>;
     return sizeof(float) * (size_t)(20 * T::PSS + (GEN ? 20 * T::PWS : TI * RS + TJ * CS));
 }
 
-__device__ __forceinline__ void cp_async(float* dst, const float* src) { cp_async4(dst, src); }
-__device__ __forceinline__ void cp_async(double* dst, const double* src) { cp_async8(dst, src); }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// Wait until at most N of this thread's committed groups are still in flight.
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
@@ -342,8 +336,8 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
             }
             if (collide) {
                 R* dy = extra ? sYx + lj + 2 : sY + li * T::PWS + lj + 2;
-                cp_async(dy, Y_in + n);
-                cp_async(dy + ds, Y_in + N + n);
+                cp_async4(dy, Y_in + n);
+                cp_async4(dy + ds, Y_in + N + n);
             }
         }
     } else if (!use_tma && !record) {
@@ -368,8 +362,8 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
                 if (!rowin(i)) continue;
                 const R* src = Y_in + (ptrdiff_t)rw(i) * nt + wrap_nt(j0 - T::HP + lj, nt);
                 R* dst = sY + li * T::PWS + lj + 2;
-                cp_async(dst, src);
-                cp_async(dst + T::PSS, src + N);
+                cp_async4(dst, src);
+                cp_async4(dst + T::PSS, src + N);
             }
         }
     }
