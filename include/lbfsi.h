@@ -233,7 +233,7 @@ typedef struct {
 int lbfsi_create_mesh_cgrid_walls(const lbfsi_mesh_cgrid_walls_desc* d, void* cuda_stream, lbfsi_mesh* out);
 
 /* Create a mesh handle on a C-grid; otherwise as lbfsi_create_mesh_xy (one
- * tile shape): the tiles next to the cut stage the mirrored rows of its other
+ * schedule variant): the tiles next to the cut stage the mirrored rows of its other
  * side.
  * LBFSI_EINVAL for an even ntheta, a bad n_cut, cut nodes that do not
  * coincide, or a mesh that is not subparametric or not positively oriented. */
@@ -444,7 +444,7 @@ typedef struct {
 
 /* Admit a solve on a general O-grid (same contract as lbfsi_batch_add).
  * Identical coordinate sets share one device copy.  These solves run on the
- * general-geometry kernel with its one tile shape, in launches of their own
+ * general-geometry kernel, its tile by their size, in launches of their own
  * in every lbfsi_batch_step; lbfsi_batch_set_schedule and the autotuner change
  * the tiles of the separable-mesh solves only. */
 int lbfsi_batch_add_xy(lbfsi_batch b, const lbfsi_solve_xy_desc* d, int* slot);
@@ -524,9 +524,11 @@ int64_t lbfsi_launch_count(lbfsi_mesh m);
  * 3: 12 x 32, 384 threads; 4: 16 x 32, 512 threads (what lbfsi_get_schedule
  * reports for new mesh handles, with order 1, and new batches, with order 0;
  * until a schedule is set they launch shape 0, 4 or 1 by their number of 16-row
- * tiles: below 152, below 608, above).  Float64 shapes (128 threads per row of 32
+ * tiles: below 152, below 608, above; and handles of more than half the L2's size
+ * launch order 0).  Float64 shapes (128 threads per row of 32
  * nodes): 0: one row per CTA (default), 1: two, 2: four.  Meshes given by node
- * coordinates have one shape (0).
+ * coordinates have one variant (0), whose float tile (8 x 32, or 16 x 32 with 256 or
+ * 512 threads) follows their size.
  * Staging (every float shape): in a float mesh handle whose Ntheta is a
  * multiple of 4, and for the float solves of a batch on separable O-grids
  * whose Ntheta is a multiple of 4, the populations and the correction field of

@@ -81,8 +81,8 @@ struct lbfsi_mesh_s {
     lbfsi::DeviceMesh dmesh;
     lbfsi::CudaMallocMemory mem;
     int nbatch = 0, precision = 0, variant = 4, order = 1, tile_rows = 16, tiles_per_solve = 0;
-    bool own_shape = true;               // no schedule asked for: the shape follows the size
-    int shape = 4;                       // tile shape launched (step_shape)
+    bool own_shape = true, own_order = true;   // no schedule asked for: the shape and the order follow the size
+    int shape = 4, launch_order = 1;     // what is launched (set_shape)
     // the step whose correction field (float64: and post-collision populations)
     // the last call left behind its last step, or -1; and the step at which the
     // last call ended, or -1 once anything changed the state since
@@ -254,16 +254,23 @@ void unify_cut_copies(const lbfsi::HostMesh& h, double* user, size_t blocks, int
 
 lbfsi::StepArgs make_args(lbfsi_mesh m);
 
-// Tile shape of a handle: its schedule's variant or, as long as none was asked
-// for, by its size (default_shape).
-int step_shape(lbfsi_mesh m) {
-    if (!m->own_shape) return m->variant;
-    return lbfsi::default_shape(m->precision, (long long)m->nbatch * m->host.ntj * ((m->host.nr + 15) / 16));
-}
+// Float meshes whose tiles are staged by tensor copies (LBFSI_TMA aside).
+bool tma_mesh(const lbfsi::HostMesh& h) { return !h.box && !h.cgrid && h.nt % 4 == 0; }
 
-// Tile shape, rows and tiles of the handle's schedule.
+// Tile shape, rows and tiles and the CTA order of the handle's schedule or, as
+// long as none was asked for, by its size.
 void set_shape(lbfsi_mesh m) {
-    m->shape = step_shape(m);
+    const lbfsi::HostMesh& h = m->host;
+    const long long tiles16 = (long long)m->nbatch * h.ntj * ((h.nr + 15) / 16);
+    const bool tma = tma_mesh(h);
+    bool moving = false;
+    for (const lbfsi_body_desc& b : m->bodies) moving = moving || b.dof != LBFSI_BODY_FIXED;
+    m->shape = !m->own_shape ? m->variant
+               : m->precision == LBFSI_FP32 && h.general ? lbfsi::default_shape_general(tma, moving, tiles16)
+                                                         : lbfsi::default_shape(m->precision, tiles16);
+    // (the third dimension of a grid, here the solves, has 16 bits)
+    m->launch_order = m->own_order && m->nbatch <= 65535 ? lbfsi::default_order(tma, h.general, (long long)m->nbatch * h.N, tiles16)
+                                                         : m->order;
     m->tile_rows = m->host.general ? lbfsi::general_tile_rows(m->precision, m->shape)
                                    : lbfsi::tile_rows(m->precision, m->shape);
     m->tiles_per_solve = ((m->host.nr + m->tile_rows - 1) / m->tile_rows) * m->host.ntj;
@@ -381,8 +388,7 @@ bool tma_maps(lbfsi_mesh m) {
     if (m->tma_rows == m->tile_rows) return true;
     if (m->tma_rows == 0) return false;
     const char* env = std::getenv("LBFSI_TMA");
-    bool ok = m->precision == LBFSI_FP32 && !m->host.box && !m->host.cgrid && m->host.nt % 4 == 0 &&
-              !(env && std::atoi(env) == 0);
+    bool ok = m->precision == LBFSI_FP32 && tma_mesh(m->host) && !(env && std::atoi(env) == 0);
     const size_t nt = (size_t)m->host.nt, nr = (size_t)m->host.nr, nb = (size_t)m->nbatch;
     const unsigned rows = (unsigned)m->tile_rows, w = (unsigned)(lbfsi::TILE_J + 8);
     for (int c = 0; c < 2 && ok; ++c) ok = lbfsi::encode_box4(&m->tm_p[c], m->d_p[c], 2 * nt, nr, 9, nb, 2 * w, rows + 4, 9);
@@ -405,7 +411,7 @@ lbfsi::StepArgs make_args(lbfsi_mesh m) {
     a.tiles = nullptr;
     a.ntiles = m->nbatch * m->tiles_per_solve;
     a.ustep = (int)m->host_k;
-    a.uorder = m->order;
+    a.uorder = m->launch_order;
     a.status = m->d_status;
     return a;
 }
@@ -566,11 +572,11 @@ int create_common(lbfsi_mesh m, int precision, int nbatch, const lbfsi_body_desc
     if (const char* v = std::getenv("LBFSI_STEP_VARIANT")) {
         const int k = std::atoi(v);
         m->variant = (k >= 0 && k < lbfsi::step_variants(LBFSI_FP32)) ? k : 4;
-        m->own_shape = m->precision == LBFSI_FP64;
+        m->own_shape = m->precision == LBFSI_FP64 || m->host.general;
     }
     if (m->precision == LBFSI_FP64 || m->host.general) m->variant = 0;   // (general: the one shape)
-    set_shape(m);
     m->bodies.assign(bodies, bodies + m->slots());
+    set_shape(m);
     m->solves.assign(m->nbatch, SolveDev{});
     rc = lbfsi::upload_mesh(m->host, m->precision, m->mem, m->stream, m->dmesh);
     if (rc) {
@@ -1096,8 +1102,9 @@ int lbfsi_set_schedule(lbfsi_mesh m, int variant, int order) {
     if (variant < 0 || variant >= (m->host.general ? 1 : lbfsi::step_variants(m->precision)) ||
         (order != 0 && order != 1))
         return fail(LBFSI_EINVAL, "variant or order out of range");
-    if (!m->own_shape && variant == m->variant && order == m->order) return LBFSI_OK;
+    if (!m->own_order && variant == m->variant && order == m->order) return LBFSI_OK;
     drop_graph(m);
+    m->own_order = false;
     m->own_shape = m->host.general;   // (general meshes have the one variant)
     m->variant = variant;
     m->order = order;

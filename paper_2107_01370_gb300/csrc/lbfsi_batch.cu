@@ -137,7 +137,7 @@ struct lbfsi_batch_s {
     }* h_get = nullptr;
     std::mutex reading;      // held by a read from its first copy until it has taken its values out
     bool own_shape = true;   // no schedule asked for: the shape follows the active solves' sizes
-    int shape = 4;           // tile shape launched (rebuild_tiles)
+    int shape = 4, gshape = 1;   // tile shapes launched, separable and general meshes (rebuild_tiles)
     size_t esize = 4;
     cudaStream_t stream = nullptr;
     std::vector<MeshEntry> meshes;
@@ -254,7 +254,7 @@ void drop_graph(lbfsi_batch b) {
 }
 
 int step_rows(lbfsi_batch b, bool general) {
-    return general ? lbfsi::general_tile_rows(b->precision, b->shape) : b->tile_rows;
+    return general ? lbfsi::general_tile_rows(b->precision, b->gshape) : b->tile_rows;
 }
 
 // CTAs of a slot's step launches in the current tile shape (SolveDev::ntiles,
@@ -302,13 +302,15 @@ int rebuild_tiles(lbfsi_batch b) {
     drop_graph(b);
     cudaError_t e = cudaSuccess;
     auto active = [&](const Slot& s, int part) { return s.used && !s.finished && (s.general ? 1 : 0) == part; };
-    b->shape = b->variant;
-    if (b->own_shape && b->precision == LBFSI_FP32) {
+    b->shape = b->gshape = b->variant;
+    if (b->precision == LBFSI_FP32) {
         // as the mesh handle (step_shape)
-        long long n = 0;
-        for (const Slot& s : b->slots)
-            if (active(s, 0)) n += (long long)b->meshes[s.mesh].host.ntj * ((b->meshes[s.mesh].host.nr + 15) / 16);
-        b->shape = lbfsi::default_shape(b->precision, n);
+        long long n[2] = {0, 0};
+        for (int part = 0; part < 2; ++part)
+            for (const Slot& s : b->slots)
+                if (active(s, part)) n[part] += (long long)b->meshes[s.mesh].host.ntj * ((b->meshes[s.mesh].host.nr + 15) / 16);
+        if (b->own_shape) b->shape = lbfsi::default_shape(b->precision, n[0]);
+        b->gshape = lbfsi::default_shape_general(false, true, n[1]);   // (staged by per-thread copies)
     }
     b->tile_rows = lbfsi::tile_rows(b->precision, b->shape);
     e = update_counts(b);
@@ -424,7 +426,7 @@ cudaError_t launch_step_part(lbfsi_batch b, int part, cudaStream_t s) {
     a.ustep = -1;
     a.status = b->d_status;
     a.tmaps = part == 0 && b->precision == LBFSI_FP32 ? b->d_tmaps : nullptr;
-    return lbfsi::launch_step(a, b->precision, part == 1, b->shape, s);
+    return lbfsi::launch_step(a, b->precision, part == 1, part == 1 ? b->gshape : b->shape, s);
 }
 
 // Field launch of one part: the loads of the last step, the fields of the
@@ -464,7 +466,7 @@ cudaError_t launch_run(lbfsi_batch b, int n, cudaStream_t s) {
 int capture_graph(lbfsi_batch b) {
     lbfsi::TraceRange trace_("lbfsi batch graph capture");
     cudaError_t e = lbfsi::prepare_step(b->precision, b->shape, false);
-    if (e == cudaSuccess && b->ntiles[1] > 0) e = lbfsi::prepare_step(b->precision, b->shape, false, true);
+    if (e == cudaSuccess && b->ntiles[1] > 0) e = lbfsi::prepare_step(b->precision, b->gshape, false, true);
     if (e == cudaSuccess && !b->cap_stream) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_err(e, "graph capture setup");
     e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
@@ -500,7 +502,7 @@ int lbfsi_batch_create(size_t pool_bytes, int precision, void* cuda_stream, lbfs
     b->esize = precision == LBFSI_FP64 ? sizeof(double) : sizeof(float);
     b->stream = static_cast<cudaStream_t>(cuda_stream);
     if (precision == LBFSI_FP64) b->variant = 0;
-    b->shape = b->variant;
+    b->shape = b->gshape = b->variant;
     b->tile_rows = lbfsi::tile_rows(precision, b->shape);
     int rc = b->pool.init(pool_bytes);
     if (rc) {

@@ -271,17 +271,15 @@ cudaError_t launch_step(const StepArgs& a, int precision, bool general, int vari
 cudaError_t launch_step_uniform(const StepArgs& a, int precision, int variant, int nbatch,
                                 cudaStream_t s);
 int default_shape(int precision, long long tiles16);
+int default_shape_general(bool tma, bool moving, long long tiles16);
+int default_order(bool tma, bool general, long long nodes, long long tiles16);
 int tile_rows(int precision, int variant);
 // Stream launch of the float64 path (lbfsi_stream64.cu): blocks of 'rows' rows
 // x 32 columns, each row by four warps that share the directions.
 cudaError_t launch_stream64(const StepArgs& a, bool uniform, bool general, int rows, int nbatch, cudaStream_t s);
-// Tile of the float general-geometry kernel, in uniform (mesh handle) and
-// table (batch runtime) launches alike.
-// (16 rows, three blocks per SM: elliptic O-grid 512 x 256 x 8 solves 103 us a
-// launch, 12 rows with four blocks of 192 threads the same, 8 rows 10% slower)
-constexpr int GEN_TILE_ROWS_FP32 = 16, GEN_THREADS_FP32 = 256, GEN_MINB_FP32 = 3;
+// Tile rows of the general-geometry kernel (float: default_shape_general).
 inline int general_tile_rows(int precision, int variant) {
-    return precision == 0 ? tile_rows(0, variant) : GEN_TILE_ROWS_FP32;
+    return precision == 0 ? tile_rows(0, variant) : variant == 0 ? 8 : 16;
 }
 // Number of tile shapes of the step kernel of a precision (variants 0 .. n-1).
 int step_variants(int precision);

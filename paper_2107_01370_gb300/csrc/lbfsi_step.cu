@@ -947,11 +947,15 @@ struct StepKernel {
     }
 };
 
-// The float kernel of a tile shape: separable shapes by variant, one shape on
-// general meshes.
+// The float kernel of a tile shape: separable shapes by variant, on general
+// meshes those of default_shape_general.
 template <bool UNIFORM, typename Fn>
 static cudaError_t with_kernel(bool general, int variant, Fn fn) {
-    if (general) return fn(StepKernel<GEN_TILE_ROWS_FP32, GEN_THREADS_FP32, GEN_MINB_FP32, UNIFORM, true>());
+    if (general) switch (variant) {
+        case 0: return fn(StepKernel<8, 256, 3, UNIFORM, true>());
+        case 1: return fn(StepKernel<16, 256, 3, UNIFORM, true>());
+        default: return fn(StepKernel<16, 512, 2, UNIFORM, true>());
+    }
     switch (variant) {
         case 1: return fn(StepKernel<16, 256, 3, UNIFORM>());
         case 2: return fn(StepKernel<12, 192, 4, UNIFORM>());
@@ -975,6 +979,38 @@ int step_variants(int precision) { return precision == 0 ? 3 : 5; }
 int default_shape(int precision, long long tiles16) {
     if (precision == 0) return 0;
     return tiles16 < 152 ? 0 : tiles16 < 608 ? 4 : 1;
+}
+
+// The same on general meshes (0: 8 x 32 tiles, 1: 16 x 32 / 256 threads, 2: 16 x 32 /
+// 512 threads; 456 blocks of the first two are resident at once, 304 of the
+// third).  8-row tiles as long as they are one wave; then a tile's own time
+// counts, which its nodes that solve their departures and its per-thread copies
+// make long and 512 threads halve; tiles staged by tensor copies keep 256 where no
+// body moves and they are one wave, and from four per SM on.  Measured per step
+// (us) with 0, 1, 2, body at rest and moving.  Ellipse, tensor copies: 40 x 64 (6
+// tiles) 26.4 30.5 28.4, 28.0 38.2 31.7; 200 x 128 x 4 (208) 28.5 28.9 29.1, 31.6
+// 38.5 32.7; 300 x 160 x 4 (380) 34.4 33.1 34.9, 39.7 44.8 38.1; 512 x 256 x 2 (512)
+// 40.6 41.6 38.1, 44.6 44.5 45.0; x 4 (1024, order 0) 61.2 57.9 60.6, 72.3 74.8 69.8;
+// x 15 (3840) - 159.8 170.1, - 202.3 204.5.  C-grid: 60 x 129 x 4 (80) 34.2 38.9 34.9,
+// 34.0 51.5 41.0; 192 x 257 x 4 (432) 40.7 44.0 37.9, 43.9 58.0 44.6; 192 x 385 x 16
+// (2496) 140.0 141.1 131.8, 167.7 173.2 159.8.
+int default_shape_general(bool tma, bool moving, long long tiles16) {
+    if (tiles16 <= 228) return 0;
+    if (!tma) return 2;
+    return tiles16 >= 608 || (!moving && tiles16 <= 456) ? 1 : 2;
+}
+
+// CTA order of a handle where none was asked for (0: solve by solve, 1: the solves
+// of a tile together).  Order 1 shares the mesh's tables between neighbouring
+// blocks; from half the L2's size on (184 bytes of state a node against 129 MB)
+// order 0 finds more of a solve's populations there, as long as a launch is not
+// many waves.  Measured per step (us) with 0 and 1: separable 512 x 256 x 2 32.0
+// 32.2; x 4 43.5 47.5, moving 46.7 50.4; x 8 71.0 75.8, 78.3 79.7; x 16 127.0 128.3,
+// 140.3 139.1; ellipse 256 x 256 x 5 (60 MB) 44.6 43.3, 54.9 52.2; 512 x 256 x 3 (72
+// MB) 52.3 55.1, 57.7 67.1; x 4 57.9 73.8, 74.8 81.2; x 15 159.8 167.5, 202.3 206.5.
+// Without tensor copies (C-grids) the two agree within 2%.
+int default_order(bool tma, bool general, long long nodes, long long tiles16) {
+    return tma && nodes * 184 > 66000000ll && (general || tiles16 < 3040) ? 0 : 1;
 }
 
 int tile_rows(int precision, int variant) {
