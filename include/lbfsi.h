@@ -139,7 +139,7 @@ typedef struct {
 /* Create a mesh handle on an O-grid given by node coordinates; otherwise as
  * lbfsi_create_mesh.  The departure points are found by Newton's method on
  * the bilinear element (Eq. depPnt) instead of the closed form of a
- * separable O-grid; one tile shape (lbfsi_set_schedule accepts variant 0).
+ * separable O-grid; one schedule variant (lbfsi_set_schedule accepts 0).
  * LBFSI_EINVAL for a mesh that is not subparametric or not positively
  * oriented. */
 int lbfsi_create_mesh_xy(const lbfsi_mesh_xy_desc* d, void* cuda_stream, lbfsi_mesh* out);
@@ -185,7 +185,7 @@ typedef struct {
 } lbfsi_mesh_box_desc;
 
 /* Create a mesh handle on a periodic box; otherwise as lbfsi_create_mesh_xy
- * (general-mesh kernel, one tile shape).  LBFSI_EINVAL for odd or too small
+ * (general-mesh kernel, one schedule variant).  LBFSI_EINVAL for odd or too small
  * sizes, a mesh that is not subparametric or not positively oriented, or a
  * moving body. */
 int lbfsi_create_mesh_box(const lbfsi_mesh_box_desc* d, void* cuda_stream, lbfsi_mesh* out);
