@@ -300,7 +300,8 @@ cudaError_t launch_fields(lbfsi_mesh m, const lbfsi::StepArgs& a, int loads, int
 // follows unchanged: a run of one call, and calls with the state or the bodies
 // set in between, form no field that nobody takes (8192 x 512: a fresh run of
 // two steps 502 -> 465 us, blend_mesh and one step 289 -> 252).  With a field's
-// address handed out every call forms them anew.
+// address handed out every call forms them anew; so does one that a caller's
+// stream captures, which may be replayed behind anything.
 // rec: device history of the steps' records, or null.
 // host_step < 0: the step numbers come from the device counters.
 cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, cudaStream_t s, int64_t* launches) {
@@ -308,7 +309,11 @@ cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, 
     lbfsi::StepArgs a = make_args(m);
     const bool host = host_step >= 0;
     cudaError_t e = cudaSuccess;
-    const bool carry = host && !m->handed_out && m->ended_at == host_step, have = carry && m->fields_of == host_step;
+    // (an error, on the legacy stream beside another's capture, comes back from the launches)
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (host && cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    const bool keep = host && st == cudaStreamCaptureStatusNone;
+    const bool carry = keep && !m->handed_out && m->ended_at == host_step, have = carry && m->fields_of == host_step;
     m->changed();
     // (the initial state is streamed without colliding; float64 copies it)
     if (!have && (!host || host_step > 0 || m->precision == LBFSI_FP64)) {
@@ -323,7 +328,7 @@ cudaError_t launch_steps(lbfsi_mesh m, int n, long long host_step, double* rec, 
                               rec ? rec + (size_t)k * m->slots() * 7 : nullptr, s);
         *launches += 2;
     }
-    if (host && e == cudaSuccess) {
+    if (keep && e == cudaSuccess) {
         m->ended_at = host_step + n;
         if (carry) m->fields_of = m->ended_at;
     }
